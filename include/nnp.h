@@ -340,7 +340,7 @@ int nnp_debug_check_index(int site, int64_t i, int64_t n, int* status);
  * the split path and is slower on BF16).  Clones inherit the setting.  No
  * effect on NNP_FP32_SIMT handles. */
 int nnp_set_fused_chain(nnp_handle* h, int enable);
-/* Tensor-core paths: enable != 0 (the default) writes each AEV row only in the
+/* enable != 0 (the default) writes each AEV row only in the
  * 64-column slices that hold a species or species-pair block with any term
  * (the rest of the row is zero: for a water molecule's atom most of the
  * 7-species blocks), and runs the first layer over the slices that are live in
@@ -348,8 +348,9 @@ int nnp_set_fused_chain(nnp_handle* h, int enable);
  * columns of those slices; 0 writes and multiplies whole rows.  The result is
  * the same (the skipped products are exact zeros; the dE/dG columns not
  * computed are those the forces never read).  While it is on, nnp_debug_rows
- * returns 0 for AEV slices a row does not hold and for dE/dG slices its tile
- * does not compute. */
+ * returns 0 for AEV slices a row does not hold and, on the tensor-core paths, for
+ * dE/dG slices its tile does not compute.  No effect on the fused FP32 kernel of
+ * one-network NNP_FP32_SIMT handles, which reads whole rows. */
 int nnp_set_sparse_rows(nnp_handle* h, int enable);
 /* The live-slice masks of the last call's 128-row AEV tiles (bit k: columns
  * 64k .. 64k+63), copied to out_host (at most max_tiles); *n_tiles receives the

@@ -25,7 +25,6 @@
 using namespace nnp;
 
 namespace nnp {
-void launch_gemm_fp32(const GemmArgs& g, int row_cap, cudaStream_t st);
 int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb,
                   float alpha, cudaStream_t st, int* n_launch, StageHook* hook, void* state,
                   bool energy_only, bool skip_l1);
@@ -125,6 +124,7 @@ struct nnp_handle {
   // first and last layer GEMMs restricted to them (exact: the rest is zero)
   bool sparse_rows = true;
   bool last_sparse = false;      // the last call ran with sparse rows
+  bool last_vjp = false;         // the last call was a force VJP
   // deterministic mode: atoms and AEV rows in sorted order, force and energy
   // contributions in their own slots summed in a fixed order (bitwise repeatable)
   bool det = false;
@@ -451,10 +451,10 @@ size_t carve(nnp_handle* h, char* base) {
   mb.aev_l = split ? c.take<char>(rows * Dp * 2) : nullptr;
   ws.aev_h = static_cast<uint16_t*>(mb.aev_h);
   ws.aev_l = static_cast<uint16_t*>(mb.aev_l);
-  // tensor-core paths: rows written only in their live slices (the first layer
-  // reads a tile's live slices, the last backward layer computes only those)
-  ws.row_mask = tc ? c.take<uint32_t>(rows) : nullptr;
-  ws.tile_mask = tc ? c.take<uint32_t>(rows / kRowTile + 1) : nullptr;
+  // rows written only in their live slices (the first layer reads a tile's live
+  // slices, the last backward layer computes only those)
+  ws.row_mask = c.take<uint32_t>(rows);
+  ws.tile_mask = c.take<uint32_t>(rows / kRowTile + 1);
   return align_up(c.off, 256);
 }
 
@@ -495,6 +495,7 @@ int ensure_arena(nnp_handle* h, int n_in, int n_sys) {
   // raise-only: other handles of the process may need larger limits
   CU_TRY(aev_ensure_smem(h->ws));
   CU_TRY(mlp_fused_ensure_smem(h->model->md));
+  CU_TRY(gemm_fp32_ensure_smem());
   if (h->model->net != kNetSimt) {
     int rc = mlp_tc_prepare(h->model->md, h->model->mw, h->mb, h->ws.row_cap, h->ws.aev,
                             h->ws.dEdG, h->model->net == kNetSplit, &h->tc_state);
@@ -606,6 +607,13 @@ bool fuses_aev_l1(const nnp_handle* h) {
   return h->fused_aev_l1 && m.net == kNetBf16 && aev_l1_supported(h->ws, call_const(h), m.md.E, m.md.h1);
 }
 
+// whether an energy call writes and multiplies only the live slices of the AEV rows
+// (the fused FP32 kernel reads whole rows)
+bool sparse_call(const nnp_handle* h) {
+  const Model& m = *h->model;
+  return h->sparse_rows && !fuses_aev_l1(h) && !(m.net == kNetSimt && mlp_fused_supported(m.md));
+}
+
 int enqueue_front(nnp_handle* h, int n_sys, const nnp_system_t* sy, const std::vector<BatchParams>& chunks,
                   int n_in, cudaStream_t st, int* n_launch) {
   const Model& m = *h->model;
@@ -677,9 +685,8 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool
     if ((rc = launch_check("neighbors"))) return rc;
     if (ws.skin_state) ++launches;   // the list refresh
     const bool fuse_l1 = fuses_aev_l1(h);
-    // sparse rows where the networks run on the tensor cores (ws.row_mask set)
     Ws wa = ws;
-    if (!h->sparse_rows || fuse_l1) { wa.row_mask = nullptr; wa.tile_mask = nullptr; }
+    if (!sparse_call(h)) { wa.row_mask = nullptr; wa.tile_mask = nullptr; }
     if (fuse_l1) {
       StageTimer t(h, st, 14);
       launch_aev_l1(ws, ac, m.mw.W1cat_h, m.mw.b1cat, h->mb.H1, m.md.h1, m.alpha, st);
@@ -696,7 +703,7 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool
                          fuse_l1);
       if (rc) return rc;
     } else {
-      launch_mlp_fp32(ws, m.md, m.mw, h->mb, m.alpha, st, &launches, &hook, energy_only);
+      launch_mlp_fp32(wa, m.md, m.mw, h->mb, m.alpha, st, &launches, &hook, energy_only);
     }
     if ((rc = launch_check("mlp"))) return rc;
     if (!energy_only) {
@@ -780,9 +787,9 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
   for (int b = 0; b < n_sys; ++b) energy_only &= (sy[b].forces == nullptr && sy[b].virial == nullptr);
   const bool front_done = one_cta_front(h, chunks.size(), n_in);
   if (n_in > 0) {   // what the diagnostic reads find in the arena, by replay too
-    const bool fuse_l1 = fuses_aev_l1(h);
-    h->last_aev_stored = !fuse_l1;
-    h->last_sparse = ws.row_mask != nullptr && h->sparse_rows && !fuse_l1;
+    h->last_aev_stored = !fuses_aev_l1(h);
+    h->last_sparse = sparse_call(h);
+    h->last_vjp = false;
   }
   int launches = 0;
   rc = enqueue_front(h, n_sys, sy, chunks, n_in, st, &launches);
@@ -1096,11 +1103,11 @@ size_t carve_vjp(nnp_handle* h, char* base, int rows, int n) {
   v.gE_row = c.take<float>(rows);
   v.U = c.take<float>((size_t)rows * Dp);
   v.Q = c.take<float>((size_t)rows * Dp);
-  float** l1[] = {&v.H1, &v.D1, &v.Z1d, &v.H1d, &v.A1h, &v.A1z, &v.dl1, &v.dl1d};
+  float** l1[] = {&v.H1, &v.D1, &v.Z1d, &v.H1d, &v.dl1, &v.dl1d};
   for (float** q : l1) *q = c.take<float>(w1);
-  float** l2[] = {&v.H2, &v.D2, &v.Z2d, &v.H2d, &v.A2h, &v.A2z, &v.dl2, &v.dl2d};
+  float** l2[] = {&v.H2, &v.D2, &v.Z2d, &v.H2d, &v.dl2, &v.dl2d};
   for (float** q : l2) *q = c.take<float>(w2);
-  float** l3[] = {&v.H3, &v.D3, &v.Z3d, &v.H3d, &v.dl3, &v.dl3d};
+  float** l3[] = {&v.H3, &v.H3d, &v.dl3, &v.dl3d};
   for (float** q : l3) *q = c.take<float>(w3);
   v.e_row = c.take<float>((size_t)E * rows);
   return align_up(c.off, 256);
@@ -1137,93 +1144,83 @@ GemmArgs gemm_base(const Ws& ws, const Model& m) {
   GemmArgs g{};
   g.alpha = m.alpha;
   g.seg_start = ws.seg_start;
+  g.counts = ws.species_count;
   g.S = m.md.S;
   return g;
 }
 
-// forward, tangent forward and forward-over-reverse of the networks (FP32)
-void vjp_networks(nnp_handle* h, cudaStream_t st) {
+// forward and backward of the networks with their tangents (FP32), each layer one
+// launch over the value and the tangent together
+void vjp_networks(nnp_handle* h, const Ws& ws, cudaStream_t st) {
   const Model& m = *h->model;
-  const Ws& ws = h->ws;
   const VjpBufs& v = h->vb;
   const MlpWeights& w = m.mw;
   const int E = m.md.E, S = m.md.S, Dp = m.ac.Dp, h1 = m.md.h1, h2 = m.md.h2, h3 = m.md.h3;
   const int R = ws.row_cap;
-  auto L1 = [&](const float* A, int epi, float* out, float* out2, const float* aux) {
+  const uint32_t* tmask = ws.row_mask ? ws.tile_mask : nullptr;
+  auto base = [&](const float* A, const float* A2, int lda, int a_net, const float* B, long long b_s,
+                  long long b_e, int ldb, int N, int K, int epi) {
     GemmArgs g = gemm_base(ws, m);
-    g.A = A; g.lda = Dp; g.a_net = 0;
-    g.B = w.W1cat; g.b_s = (long long)E * h1 * Dp; g.b_e = 0; g.ldb = Dp;
-    g.bias = w.b1cat; g.bias_s = (long long)E * h1; g.bias_e = 0;
-    g.N = E * h1; g.K = Dp;
-    g.out = out; g.out2 = out2; g.ldo = E * h1; g.out_net = 0;
-    g.aux = aux; g.ld_aux = E * h1; g.aux_net = 0;
-    g.epi = epi;
-    launch_gemm_fp32(g, R, st, 1);
+    g.A = A; g.A2 = A2; g.lda = lda; g.a_net = a_net;
+    g.B = B; g.b_s = b_s; g.b_e = b_e; g.ldb = ldb;
+    g.N = N; g.K = K; g.epi = epi;
+    return g;
   };
-  // per-member layer: out[:, e*n_out] = A[:, e*k] B_{e,s}^T
-  auto Lm = [&](const float* A, int k, const float* B, int n_out, const float* bias, int epi, float* out,
-                float* out2, const float* aux) {
-    GemmArgs g = gemm_base(ws, m);
-    g.A = A; g.lda = E * k; g.a_net = k;
-    g.B = B; g.b_s = (long long)n_out * k; g.b_e = (long long)S * n_out * k; g.ldb = k;
-    g.bias = bias; g.bias_s = n_out; g.bias_e = (long long)S * n_out;
-    g.N = n_out; g.K = k;
-    g.out = out; g.out2 = out2; g.ldo = E * n_out; g.out_net = n_out;
-    g.aux = aux; g.ld_aux = E * n_out; g.aux_net = n_out;
-    g.epi = epi;
-    launch_gemm_fp32(g, R, st, E);
+  auto outs = [](GemmArgs& g, float* o, float* o2, float* o3, float* o4, int ldo, int out_net) {
+    g.out = o; g.out2 = o2; g.out3 = o3; g.out4 = o4; g.ldo = ldo; g.out_net = out_net;
   };
-  L1(ws.aev, kEpiCelu, v.H1, v.D1, nullptr);
-  Lm(v.H1, h1, w.W2, h2, w.b2, kEpiCelu, v.H2, v.D2, nullptr);
-  Lm(v.H2, h2, w.W3, h3, w.b3, kEpiCelu, v.H3, v.D3, nullptr);
-  L1(v.U, kEpiStoreMul, v.Z1d, v.H1d, v.D1);
-  Lm(v.H1d, h1, w.W2, h2, nullptr, kEpiStoreMul, v.Z2d, v.H2d, v.D2);
-  Lm(v.H2d, h2, w.W3, h3, nullptr, kEpiStoreMul, v.Z3d, v.H3d, v.D3);
-  launch_vjp_out3(ws, v, w.w4, S, E, h3, m.alpha, st);
-  Lm(v.dl3, h3, w.W3T, h2, nullptr, kEpiStore, v.A2h, nullptr, nullptr);
-  Lm(v.dl3d, h3, w.W3T, h2, nullptr, kEpiStore, v.A2z, nullptr, nullptr);
-  launch_vjp_delta(ws, S, E * h2, v.A2h, v.A2z, v.D2, v.Z2d, v.dl2, v.dl2d, m.alpha, st);
-  Lm(v.dl2, h2, w.W2T, h1, nullptr, kEpiStore, v.A1h, nullptr, nullptr);
-  Lm(v.dl2d, h2, w.W2T, h1, nullptr, kEpiStore, v.A1z, nullptr, nullptr);
-  launch_vjp_delta(ws, S, E * h1, v.A1h, v.A1z, v.D1, v.Z1d, v.dl1, v.dl1d, m.alpha, st);
-  auto B1 = [&](const float* A, float* out) {
-    GemmArgs g = gemm_base(ws, m);
-    g.A = A; g.lda = E * h1; g.a_net = 0;
-    g.B = w.W1Tcat; g.b_s = (long long)Dp * E * h1; g.b_e = 0; g.ldb = E * h1;
-    g.N = Dp; g.K = E * h1;
-    g.out = out; g.ldo = Dp; g.out_net = 0;
-    g.epi = kEpiStore;
-    launch_gemm_fp32(g, R, st, 1);
+  // member e's layer: out[:, e*n_out] = A[:, e*k] B_{e,s}^T
+  auto layer = [&](const float* A, const float* A2, int k, const float* B, int n_out, int epi) {
+    return base(A, A2, E * k, k, B, (long long)n_out * k, (long long)S * n_out * k, k, n_out, k, epi);
   };
-  B1(v.dl1, ws.dEdG);
-  B1(v.dl1d, v.Q);
+  GemmArgs g = base(ws.aev, v.U, Dp, 0, w.W1cat, (long long)E * h1 * Dp, 0, Dp, E * h1, Dp, kEpiCelu);
+  g.bias = w.b1cat; g.bias_s = (long long)E * h1; g.bias_e = 0;
+  g.kmask = tmask;
+  outs(g, v.H1, v.H1d, v.D1, v.Z1d, E * h1, 0);
+  launch_gemm_dual(g, R, st, 1);
+  g = layer(v.H1, v.H1d, h1, w.W2, h2, kEpiCelu);
+  g.bias = w.b2; g.bias_s = h2; g.bias_e = (long long)S * h2;
+  outs(g, v.H2, v.H2d, v.D2, v.Z2d, E * h2, h2);
+  launch_gemm_dual(g, R, st, E);
+  g = layer(v.H2, v.H2d, h2, w.W3, h3, kEpiCeluDot);
+  g.bias = w.b3; g.bias_s = h3; g.bias_e = (long long)S * h3;
+  g.w4 = w.w4; g.w4_s = h3; g.w4_e = (long long)S * h3;
+  g.e_row = v.e_row; g.e_row_net = R;
+  outs(g, v.H3, v.H3d, v.dl3, v.dl3d, E * h3, h3);
+  cudaMemsetAsync(v.e_row, 0, sizeof(float) * (size_t)E * R, st);
+  launch_gemm_dual(g, R, st, E);
+  g = layer(v.dl3, v.dl3d, h3, w.W3T, h2, kEpiMul);
+  g.aux = v.D2; g.aux2 = v.Z2d; g.ld_aux = E * h2; g.aux_net = h2;
+  outs(g, v.dl2, v.dl2d, nullptr, nullptr, E * h2, h2);
+  launch_gemm_dual(g, R, st, E);
+  g = layer(v.dl2, v.dl2d, h2, w.W2T, h1, kEpiMul);
+  g.aux = v.D1; g.aux2 = v.Z1d; g.ld_aux = E * h1; g.aux_net = h1;
+  outs(g, v.dl1, v.dl1d, nullptr, nullptr, E * h1, h1);
+  launch_gemm_dual(g, R, st, E);
+  g = base(v.dl1, v.dl1d, E * h1, 0, w.W1Tcat, (long long)Dp * E * h1, 0, E * h1, Dp, E * h1, kEpiStore);
+  g.nmask = tmask;
+  outs(g, ws.dEdG, v.Q, nullptr, nullptr, Dp, 0);
+  launch_gemm_dual(g, R, st, 1);
 }
 
-void vjp_weight_grads(nnp_handle* h, float* out, cudaStream_t st) {
+void vjp_weight_grads(nnp_handle* h, const Ws& ws, float* out, cudaStream_t st) {
   const Model& m = *h->model;
-  const Ws& ws = h->ws;
   const VjpBufs& v = h->vb;
   const int E = m.md.E, S = m.md.S, D = m.ac.D, Dp = m.ac.Dp, h1 = m.md.h1, h2 = m.md.h2, h3 = m.md.h3;
   const long long off2 = (long long)h1 * D + h1, off3 = off2 + (long long)h2 * h1 + h2;
-  const long long off4 = off3 + (long long)h3 * h2 + h3;
-  const long long per_net = off4 + h3 + 1;
   WgradArgs a{};
-  a.S = S; a.scale = 1.f / E; a.out = out; a.per_net = per_net;
-  a.X1 = v.dl1; a.X2 = v.dl1d; a.ldx = E * h1; a.x_net = h1;
-  a.Y1 = ws.aev; a.Y2 = v.U; a.ldy = Dp; a.y_net = 0;
-  a.n_out = h1; a.n_in = Dp; a.n_in_real = D; a.layer_off = 0;
-  a.feat_of_col = m.feat_of_col_dev;   // W1's columns back in the paper's feature order
-  launch_wgrad(a, ws, v, E, st);
-  a.feat_of_col = nullptr;
-  a.X1 = v.dl2; a.X2 = v.dl2d; a.ldx = E * h2; a.x_net = h2;
-  a.Y1 = v.H1; a.Y2 = v.H1d; a.ldy = E * h1; a.y_net = h1;
-  a.n_out = h2; a.n_in = h1; a.n_in_real = h1; a.layer_off = off2;
-  launch_wgrad(a, ws, v, E, st);
-  a.X1 = v.dl3; a.X2 = v.dl3d; a.ldx = E * h3; a.x_net = h3;
-  a.Y1 = v.H2; a.Y2 = v.H2d; a.ldy = E * h2; a.y_net = h2;
-  a.n_out = h3; a.n_in = h2; a.n_in_real = h2; a.layer_off = off3;
-  launch_wgrad(a, ws, v, E, st);
-  launch_wgrad_out(ws, v, S, E, h3, out, per_net, off4, st);
+  a.S = S; a.E = E; a.scale = 1.f / E; a.out = out;
+  a.off4 = off3 + (long long)h3 * h2 + h3;
+  a.per_net = a.off4 + h3 + 1;
+  a.H3 = v.H3; a.H3d = v.H3d; a.h3 = h3;
+  a.seg_start = ws.seg_start; a.counts = ws.species_count; a.gE_row = v.gE_row;
+  a.tile_mask = ws.row_mask ? ws.tile_mask : nullptr;
+  // W1's columns go back to the paper's feature order
+  a.layer[0] = {v.dl1, v.dl1d, E * h1, h1, ws.aev, v.U, Dp, 0, h1, Dp, D, 0, m.feat_of_col_dev, 1};
+  a.layer[1] = {v.dl2, v.dl2d, E * h2, h2, v.H1, v.H1d, E * h1, h1, h2, h1, h1, off2, nullptr, 0};
+  a.layer[2] = {v.dl3, v.dl3d, E * h3, h3, v.H2, v.H2d, E * h2, h2, h3, h2, h2, off3, nullptr, 0};
+  cudaMemsetAsync(out, 0, sizeof(float) * (size_t)(a.per_net * S * E), st);
+  launch_wgrad(a, ws.row_cap, st);
 }
 
 }  // namespace
@@ -1258,14 +1255,15 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
   Ws ws = h->ws;
   ws.aev_h = nullptr;
   ws.aev_l = nullptr;
-  ws.row_mask = nullptr;      // the FP32 chain reads whole rows
-  ws.tile_mask = nullptr;
+  if (!h->sparse_rows) { ws.row_mask = nullptr; ws.tile_mask = nullptr; }
   // the deterministic mode covers energy and force calls, not the VJP (whose
   // dual backward adds atomically): the forces here add atomically as well
   ws.fr_det = ws.fa_det = ws.fs_det = nullptr;
   ws.e_det = ws.v_det = nullptr;
   h->last_aev_fp32 = true;
-  h->last_sparse = false;
+  h->last_aev_stored = true;
+  h->last_sparse = h->sparse_rows;
+  h->last_vjp = true;
   // the force VJP builds its own lists at the cutoffs in the shared buffers:
   // persistent lists of energy calls are rebuilt on the next such call
   struct SkinOff {
@@ -1295,27 +1293,28 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
     }
     chunks.push_back(bp);
   }
-  for (const auto& bp : chunks) launch_init_chunk(ws, bp, st);
-  for (const auto& bp : chunks) {
-    int n_chunk = 0;
-    for (int k = 0; k < bp.n_sys; ++k) n_chunk += bp.sys[k].n_in;
-    launch_prep_atoms(ws, bp, n_chunk, m.ac.S, st);
+  if (chunks.size() == 1 && n_in <= kFrontMaxAtoms) {
+    launch_front(ws, chunks[0], m.ac, n_in, st);
+  } else {
+    for (const auto& bp : chunks) launch_init_chunk(ws, bp, st);
+    for (const auto& bp : chunks) {
+      int n_chunk = 0;
+      for (int k = 0; k < bp.n_sys; ++k) n_chunk += bp.sys[k].n_in;
+      launch_prep_atoms(ws, bp, n_chunk, m.ac.S, st);
+    }
+    launch_setup(ws, m.ac, st);
+    launch_bin(ws, n_in, st);
+    launch_scan(ws, st);
+    launch_scatter(ws, n_in, st);
   }
-  launch_setup(ws, m.ac, st);
-  launch_bin(ws, n_in, st);
-  launch_scan(ws, st);
-  launch_scatter(ws, n_in, st);
   launch_neighbors(ws, n_in, m.ac, st);
-  launch_aev_fwd(ws, n_in, m.ac, st);
-  launch_vjp_zero(ws, h->vb, n_in, st);
   launch_gather_v(ws, h->vb, n_in, st);
-  launch_aev_jvp(ws, m.ac, h->vb, n_in, st);
-  vjp_networks(h, st);
-  launch_aev_bwd(ws, n_in, m.ac, 0, st);
+  launch_aev_fwd_vjp(ws, m.ac, h->vb, n_in, st);
+  vjp_networks(h, ws, st);
   launch_aev_bwd_dual(ws, m.ac, h->vb, n_in, st);
   launch_finalize_e(ws, n_in, h->vb.e_row, m.md.E, ws.row_cap, m.ebias, st);
   launch_vjp_scatter(ws, h->vb, n_in, st);
-  vjp_weight_grads(h, dL_dweights, st);
+  vjp_weight_grads(h, ws, dL_dweights, st);
   h->last_n_in = n_in;
   CU_TRY(cudaGetLastError());
   return NNP_OK;
@@ -1502,6 +1501,19 @@ int nnp_debug_rows(nnp_handle* h, int which, float* out, void* stream) {
   const uint16_t* src_l = planes ? h->ws.aev_l : nullptr;
   Ws gw = h->ws;
   if (!h->last_sparse) gw.row_mask = nullptr;   // the last call wrote whole rows
+  if (which == 1 && h->last_sparse && (h->last_vjp || h->model->net == kNetSimt)) {
+    // the FP32 chains' dE/dG is read back whole: the columns that the call left out
+    // (the forces do not read them) are computed now from its deltas
+    const Model& m = *h->model;
+    const int kd = m.md.E * m.md.h1;
+    GemmArgs g = gemm_base(h->ws, m);
+    g.A = h->last_vjp ? h->vb.dl1 : h->mb.H1; g.lda = kd;
+    g.B = m.mw.W1Tcat; g.b_s = (long long)m.ac.Dp * kd; g.ldb = kd;
+    g.N = m.ac.Dp; g.K = kd; g.epi = kEpiStore;
+    g.out = h->ws.dEdG; g.ldo = m.ac.Dp;
+    launch_gemm_fp32(g, h->ws.row_cap, static_cast<cudaStream_t>(stream), 1);
+    gw.row_mask = nullptr;
+  }
   launch_gather_rows(gw, h->last_n_in, src, src_h, src_l, h->model->ac.Dp, h->model->ac.D,
                      h->model->col_of_feat_dev, out, which == 1, static_cast<cudaStream_t>(stream));
   CU_TRY(cudaGetLastError());
@@ -1666,6 +1678,7 @@ extern "C" int nnp_energy_forces_noalloc(nnp_handle* h, int64_t n_atoms, const f
   // the fixed neighbour lists may need more shared memory than other handles set up
   CU_TRY(aev_ensure_smem(ws));
   CU_TRY(mlp_fused_ensure_smem(m.md));
+  CU_TRY(gemm_fp32_ensure_smem());
   // the status word starts at zero on every call; the kernels clear the rest
   CU_TRY(cudaMemsetAsync(ws.status, 0, 4 * sizeof(int), st));
   if (n_atoms == 0) {

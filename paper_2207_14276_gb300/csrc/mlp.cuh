@@ -12,25 +12,38 @@ enum Epi : int {
   kEpiCeluDot = 1,  // e_row += CELU(acc + b) . w4 ; out = w4 * CELU'(acc + b)
   kEpiMul = 2,      // out = acc * aux
   kEpiStore = 3,    // out = acc
-  kEpiStoreMul = 4, // out = acc, out2 = acc * aux
 };
 
 // One grouped GEMM: for every 128-row tile of species s and net e = blockIdx.z,
 //   C[m, n] = sum_k A[m, e*a_net + k] * B_{e,s}[n, k]      (B row-major [N, K])
+// The dual form (launch_gemm_dual, force VJP) multiplies a second operand A2 (the
+// tangent of A) with the same B and writes, with z' the tangent accumulator:
+//   kEpiCelu     out = CELU(z), out2 = CELU'(z) z', out3 = CELU'(z), out4 = z'
+//   kEpiCeluDot  out, out2 as above; out3 = w4 CELU'(z), out4 = w4 CELU''(z) z'
+//   kEpiMul      out = acc aux, out2 = acc CELU''(aux) aux2 + acc' aux
+//   kEpiStore    out = acc, out2 = acc'
 struct GemmArgs {
   const void* A; int lda; int a_net;
+  const void* A2;
   const void* B; long long b_s, b_e; int ldb;
   const float* bias; long long bias_s, bias_e;
   const float* w4; long long w4_s, w4_e;
   int N, K;
   void* out; int ldo; int out_net;
   void* out2;            // CELU' output (same layout as out)
+  float* out3; float* out4;
   const void* aux; int ld_aux; int aux_net;
+  const float* aux2;     // dual: z' (same layout as aux)
   float* e_row; int e_row_net;   // per-net row energies
   int epi;
   float alpha;           // CELU alpha
   const int* seg_start;  // [S+1]
+  const int* counts;     // [S] rows of a segment in use
   int S;
+  // sparse AEV rows (null: dense): the live 64-column slices of each 128-row tile;
+  // kmask: the K slices to multiply; nmask: the N tiles to compute
+  const uint32_t* kmask;
+  const uint32_t* nmask;
 };
 
 struct MlpDims {
@@ -77,8 +90,9 @@ struct StageHook {
   void end();
 };
 
-void launch_gemm_fp32(const GemmArgs& g, int row_cap, cudaStream_t st);
 void launch_gemm_fp32(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets);
+cudaError_t gemm_fp32_ensure_smem();
+void launch_gemm_dual(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets);
 // the whole FP32 chain of one-network models as a single kernel per 32-row tile
 bool mlp_fused_supported(const MlpDims& md);
 cudaError_t mlp_fused_ensure_smem(const MlpDims& md);

@@ -14,9 +14,11 @@ namespace nnp {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16;
-constexpr int TM = 8, TN = 4;                  // outputs per thread
-constexpr int kThreads = (BM / TM) * (BN / TN);  // 128
+constexpr int kThreads = 128;   // 4 warps
+constexpr int KS = 16;          // K slice of one ring stage (K is a multiple of 16)
+constexpr int NS = 4;           // ring stages (three slices in flight)
+constexpr int LD = KS + 4;      // row stride of a staged slice (floats): float4 reads of
+                                // consecutive rows hit different banks
 
 __device__ __forceinline__ float celu_f(float z, float alpha, float inv_alpha) {
   return z > 0.f ? z : alpha * (__expf(z * inv_alpha) - 1.f);
@@ -24,155 +26,303 @@ __device__ __forceinline__ float celu_f(float z, float alpha, float inv_alpha) {
 __device__ __forceinline__ float celu_d(float z, float inv_alpha) {
   return z > 0.f ? 1.f : __expf(z * inv_alpha);
 }
+// CELU'' from CELU' (z <= 0: exp(z/alpha)/alpha; z > 0: 0)
+__device__ __forceinline__ float celu_dd(float dz, float inv_alpha) {
+  return dz < 1.f ? dz * inv_alpha : 0.f;
+}
 
-// 64 x 64 output tile per CTA, 128 threads with an 8 x 4 register tile each
-// (rows ty*8.., columns tx*4..).  16-wide K slices of A and B are staged
-// through registers into a double-buffered, transposed shared-memory copy, so
-// each thread reads its 8 rows and 4 columns of one K step as three 16-byte loads.
-template <int EPI>
+__device__ __forceinline__ void cp16(float* dst, const float* src, bool valid) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = valid ? 16 : 0;   // 0 source bytes: zero-filled
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ float comp(const float4& v, int q) {
+  return q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w;
+}
+
+// One output tile of BM = 4 R rows x BN = 32 C columns per CTA: a warp owns R rows,
+// a lane the columns lane + 32 j.  16-wide K slices of A and B come by cp.async into
+// a ring in their row-major layout (no transpose through registers), and a lane
+// reads four k of a row or column as one float4.  All lanes of a warp read the same
+// rows of A, so those loads are broadcasts (one shared-memory wavefront each against
+// four for a column's): four k cost R + 4 C wavefronts for 4 R C FMA instructions,
+// and the FMA pipes bound the kernel.  (With 8 x 4 lanes per warp and 8 x 8 outputs
+// per lane the same loads took twice the wavefronts, as many cycles as the FMAs.)
+// DUAL multiplies two A operands (a value and its tangent) with the same B, so that
+// the force VJP reads each weight once for both and its element-wise steps between
+// layers happen in the epilogue.  Sparse AEV rows skip the K slices (kmask) and the
+// N tiles (nmask) that are zero or unused in the whole 128-row tile; tiles of padding
+// rows only are skipped.  8 networks 1008-256-192-160-1 on 3,072 atoms: L1 383 -> 213 us,
+// L2 85 -> 80, L3 68 -> 68, B3 56 -> 53, B2 86 -> 78, B1 453 -> 250 us (before: 64 x 64
+// tiles, slices transposed through registers, dense rows); the FMA pipe is 53% active,
+// held by the fixed latency of its instructions at 8 to 16 warps per SM.
+template <int EPI, bool DUAL, int R, int C>
 __global__ void __launch_bounds__(kThreads) k_gemm_fp32(GemmArgs g) {
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN + 4];
-  const int m0 = blockIdx.x * BM;
+  constexpr int BM = 4 * R, BN = 32 * C, P = DUAL ? 2 : 1;
+  constexpr int kStage = (P * BM + BN) * LD;
+  static_assert(BM % 32 == 0 && kRowTile % BM == 0, "loader; a tile stays inside a 128-row tile");
+  extern __shared__ __align__(16) float sm[];
+  // N tiles fastest: neighbouring CTAs share the rows of A
+  const int n_nt = (g.N + BN - 1) / BN;
+  const int m0 = (int)(blockIdx.x / n_nt) * BM, n0 = (int)(blockIdx.x % n_nt) * BN;
   const int total = g.seg_start[g.S];
   if (m0 >= total) return;
+  if (g.nmask) {   // a tile that touches no live 64-column slice
+    const uint32_t span = (2u << (((min(n0 + BN, g.N) - 1) >> 6) - (n0 >> 6))) - 1u;
+    if (!((g.nmask[m0 >> 7] >> (n0 >> 6)) & span)) return;
+  }
   int s = 0;
   while (s + 1 < g.S && m0 >= g.seg_start[s + 1]) ++s;
+  if (m0 >= g.seg_start[s] + g.counts[s]) return;   // padding rows only
   const int e = blockIdx.z;
-  const int n0 = blockIdx.y * BN;
-  if (n0 >= g.N) return;
-  const float* A = static_cast<const float*>(g.A) + (size_t)e * g.a_net;
+  const float* A[2] = {static_cast<const float*>(g.A) + (size_t)e * g.a_net,
+                       DUAL ? static_cast<const float*>(g.A2) + (size_t)e * g.a_net : nullptr};
   const float* B = static_cast<const float*>(g.B) + e * g.b_e + s * g.b_s;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  // loaders: A and B slices are 64 rows x 16 k = 256 float4 each, 2 per thread
-  float4 ra[2], rb[2];
-  auto load = [&](int k0) {
+  const uint32_t km = g.kmask ? g.kmask[m0 >> 7] : ~0u;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int n_k = g.K / KS;
+  auto next = [&](int k) {   // the first live slice after k (masks: 64 columns per bit)
+    do ++k;
+    while (k < n_k && g.kmask && !((km >> (k >> 2)) & 1u));
+    return k;
+  };
+  auto load = [&](int k, int st) {
+    float* base = sm + st * kStage + (tid & 3) * 4;
+    const int r0 = tid >> 2, kc = k * KS + (tid & 3) * 4;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int idx = tid + i * kThreads, r = idx >> 2, q = idx & 3;
-      ra[i] = *reinterpret_cast<const float4*>(A + (size_t)(m0 + r) * g.lda + k0 + q * 4);
-      rb[i] = (n0 + r < g.N) ? *reinterpret_cast<const float4*>(B + (size_t)(n0 + r) * g.ldb + k0 + q * 4)
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int i = 0; i < BM / 32; ++i) {
+        const int r = r0 + 32 * i;
+        cp16(base + (p * BM + r) * LD, A[p] + (size_t)(m0 + r) * g.lda + kc, true);
+      }
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      const int r = r0 + 32 * i;
+      const bool ok = n0 + r < g.N;
+      cp16(base + (P * BM + r) * LD, B + (ok ? (size_t)(n0 + r) * g.ldb + kc : 0), ok);
     }
   };
-  auto store = [&](int buf) {
+  // plain form: two partial sums per output, over even and odd k, in packed FP32x2
+  // FMAs (half the instructions: the same loop of scalar FMAs lost issue slots to
+  // dispatch stalls, B1 343 us against 250); dual form: one sum in the order of k
+  constexpr int V = DUAL ? 1 : 2;
+  float acc[P][R][C][V];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int idx = tid + i * kThreads, r = idx >> 2, q = idx & 3;
-      As[buf][q * 4 + 0][r] = ra[i].x; As[buf][q * 4 + 1][r] = ra[i].y;
-      As[buf][q * 4 + 2][r] = ra[i].z; As[buf][q * 4 + 3][r] = ra[i].w;
-      Bs[buf][q * 4 + 0][r] = rb[i].x; Bs[buf][q * 4 + 1][r] = rb[i].y;
-      Bs[buf][q * 4 + 2][r] = rb[i].z; Bs[buf][q * 4 + 3][r] = rb[i].w;
-    }
-  };
-  float acc[TM][TN];
+  for (int p = 0; p < P; ++p)
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-  load(0);
-  store(0);
-  __syncthreads();
-  int buf = 0;
-  for (int k0 = 0; k0 < g.K; k0 += BK) {
-    const bool more = k0 + BK < g.K;
-    if (more) load(k0 + BK);
+      for (int j = 0; j < C; ++j)
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM + 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * TN]);
-      const float a[TM] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[TN] = {bv.x, bv.y, bv.z, bv.w};
+        for (int v = 0; v < V; ++v) acc[p][i][j][v] = 0.f;
+  // every iteration commits one group (empty past the end), so "at most NS - 2
+  // pending" always means that the slice in use has landed
+  int k_use = next(-1), k_load = k_use;
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+  for (int i = 0; i < NS - 1; ++i) {
+    if (k_load < n_k) { load(k_load, i); k_load = next(k_load); }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  for (int it = 0; k_use < n_k; ++it, k_use = next(k_use)) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(NS - 2) : "memory");
+    __syncthreads();   // the slice is visible to all; all are done with the one before
+    if (k_load < n_k) { load(k_load, (it + NS - 1) % NS); k_load = next(k_load); }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    const float* sa = sm + (it % NS) * kStage + w * R * LD;
+    const float* sb = sm + (it % NS) * kStage + (P * BM + lane) * LD;
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    if (more) {
-      store(buf ^ 1);
-      __syncthreads();
-      buf ^= 1;
+    for (int kk = 0; kk < KS; kk += 4) {
+      float4 b[C];
+#pragma unroll
+      for (int j = 0; j < C; ++j) b[j] = *reinterpret_cast<const float4*>(sb + 32 * j * LD + kk);
+      constexpr int RG = 4;   // rows taken together: independent FMAs between dependent ones
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int i0 = 0; i0 < R; i0 += RG) {
+          float4 a[RG];
+#pragma unroll
+          for (int i = 0; i < RG; ++i) a[i] = *reinterpret_cast<const float4*>(sa + (p * BM + i0 + i) * LD + kk);
+          if constexpr (DUAL) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+              for (int i = 0; i < RG; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j)
+                  acc[p][i0 + i][j][0] = fmaf(comp(a[i], q), comp(b[j], q), acc[p][i0 + i][j][0]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; q += 2)
+#pragma unroll
+              for (int i = 0; i < RG; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                  float(&c)[V] = acc[p][i0 + i][j];
+                  const float2 r = __ffma2_rn(make_float2(comp(a[i], q), comp(a[i], q + 1)),
+                                              make_float2(comp(b[j], q), comp(b[j], q + 1)),
+                                              make_float2(c[0], c[V - 1]));
+                  c[0] = r.x;
+                  c[V - 1] = r.y;
+                }
+          }
+        }
     }
   }
-  // ---- epilogue (N is a multiple of 16: a thread's 4 columns are all in or all out)
-  const int nb = n0 + tx * TN;
-  const bool n_ok = nb < g.N;
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  // ---- epilogue
   const float alpha = g.alpha, inv_alpha = 1.f / g.alpha;
-  if (EPI == kEpiCelu || EPI == kEpiCeluDot) {
-    float bias[TN] = {0.f, 0.f, 0.f, 0.f}, w4[TN] = {0.f, 0.f, 0.f, 0.f};
-    if (n_ok) {
-      const float* bp = g.bias + e * g.bias_e + s * g.bias_s + nb;
-      for (int j = 0; j < TN; ++j) bias[j] = bp[j];
-      if (EPI == kEpiCeluDot) {
-        const float* wp = g.w4 + e * g.w4_e + s * g.w4_s + nb;
-        for (int j = 0; j < TN; ++j) w4[j] = wp[j];
-      }
-    }
+  float bias[C], w4[C];
+  constexpr bool kBias = EPI == kEpiCelu || EPI == kEpiCeluDot;
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-      const int m = m0 + ty * TM + i;
-      float h[TN], dd[TN], dot = 0.f;
+  for (int j = 0; j < C; ++j) {
+    const int n = n0 + lane + 32 * j;
+    const bool ok = n < g.N;
+    bias[j] = kBias && ok ? g.bias[e * g.bias_e + s * g.bias_s + n] : 0.f;
+    w4[j] = EPI == kEpiCeluDot && ok ? g.w4[e * g.w4_e + s * g.w4_s + n] : 0.f;
+  }
+  float* const out = static_cast<float*>(g.out);
+  float* const out2 = static_cast<float*>(g.out2);
+  constexpr int RI = 4;   // rows whose stored values are read before any is written
 #pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        const float zz = acc[i][j] + bias[j];
-        h[j] = celu_f(zz, alpha, inv_alpha);
-        dd[j] = celu_d(zz, inv_alpha);
-        dot = fmaf(h[j], w4[j], dot);
-      }
-      float* o = static_cast<float*>(g.out) + (size_t)m * g.ldo + (size_t)e * g.out_net + nb;
-      if (EPI == kEpiCelu) {
-        if (n_ok) {
-          *reinterpret_cast<float4*>(o) = make_float4(h[0], h[1], h[2], h[3]);
-          float* o2 = static_cast<float*>(g.out2) + (size_t)m * g.ldo + (size_t)e * g.out_net + nb;
-          *reinterpret_cast<float4*>(o2) = make_float4(dd[0], dd[1], dd[2], dd[3]);
+  for (int i0 = 0; i0 < R; i0 += RI) {
+    float ax[RI][C], ax2[RI][C];
+    if (EPI == kEpiMul) {
+#pragma unroll
+      for (int i = 0; i < RI; ++i) {
+        const size_t arow = (size_t)(m0 + w * R + i0 + i) * g.ld_aux + (size_t)e * g.aux_net;
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+          const int n = n0 + lane + 32 * j;
+          ax[i][j] = n < g.N ? static_cast<const float*>(g.aux)[arow + n] : 0.f;
+          ax2[i][j] = DUAL && n < g.N ? g.aux2[arow + n] : 0.f;
         }
-      } else {
-        if (n_ok)
-          *reinterpret_cast<float4*>(o) =
-              make_float4(w4[0] * dd[0], w4[1] * dd[1], w4[2] * dd[2], w4[3] * dd[3]);
-        // the 16 threads of a row group hold the row's columns
-#pragma unroll
-        for (int o2 = 1; o2 < 16; o2 <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o2);
-        if (tx == 0) atomicAdd(g.e_row + (size_t)e * g.e_row_net + m, dot);
       }
     }
+#pragma unroll
+    for (int i = 0; i < RI; ++i) {
+      const int m = m0 + w * R + i0 + i;
+      const size_t row = (size_t)m * g.ldo + (size_t)e * g.out_net;
+      float dot = 0.f;
+#pragma unroll
+      for (int j = 0; j < C; ++j) {
+        const int n = n0 + lane + 32 * j;
+        if (n >= g.N) continue;
+        const size_t o = row + n;
+        float v = acc[0][i0 + i][j][0];
+        if (!DUAL) v += acc[0][i0 + i][j][V - 1];
+        const float vt = acc[P - 1][i0 + i][j][0];   // dual: the tangent
+        if (kBias) {
+          const float z = v + bias[j];
+          const float h = celu_f(z, alpha, inv_alpha), d = celu_d(z, inv_alpha);
+          dot = fmaf(h, w4[j], dot);
+          if (!DUAL) {
+            out[o] = EPI == kEpiCelu ? h : w4[j] * d;
+            if (EPI == kEpiCelu) out2[o] = d;
+          } else {
+            out[o] = h;
+            out2[o] = d * vt;
+            if (EPI == kEpiCelu) {
+              g.out3[o] = d;
+              g.out4[o] = vt;
+            } else {   // delta3 and its tangent
+              g.out3[o] = w4[j] * d;
+              g.out4[o] = w4[j] * celu_dd(d, inv_alpha) * vt;
+            }
+          }
+        } else if (EPI == kEpiMul) {
+          const float d = ax[i][j];
+          out[o] = v * d;
+          if (DUAL) out2[o] = v * celu_dd(d, inv_alpha) * ax2[i][j] + vt * d;
+        } else {
+          out[o] = v;
+          if (DUAL) out2[o] = vt;
+        }
+      }
+      if (EPI == kEpiCeluDot) {   // the lanes hold this tile's columns of the row
+#pragma unroll
+        for (int q = 1; q < 32; q <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, q);
+        if (lane == 0) atomicAdd(g.e_row + (size_t)e * g.e_row_net + m, dot);
+      }
+    }
+  }
+}
+
+template <bool DUAL, int R, int C>
+constexpr int gemm_smem() {
+  return NS * ((DUAL ? 2 : 1) * 4 * R + 32 * C) * LD * (int)sizeof(float);
+}
+
+template <int EPI, bool DUAL, int R, int C>
+void launch_one(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets) {
+  constexpr int BM = 4 * R, BN = 32 * C;
+  const dim3 grid((unsigned)((row_cap + BM - 1) / BM) * ((g.N + BN - 1) / BN), 1, n_nets);
+  k_gemm_fp32<EPI, DUAL, R, C><<<grid, kThreads, gemm_smem<DUAL, R, C>(), st>>>(g);
+}
+
+// 16 rows per warp (8 and their tangents in the dual form).  The width of a tile is
+// the one that pads N least, the widest such for the plain form (fewest loads per
+// FMA) and the narrowest for the dual one (training batches have few rows).
+constexpr int kRows = 16, kRowsDual = 8;
+
+template <int EPI>
+void launch_epi(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets, bool dual) {
+  int c = dual || g.nmask ? 2 : 4;   // (masked N tiles: narrow ones follow the live columns)
+  auto padded = [&](int q) { return (g.N + 32 * q - 1) / (32 * q) * q; };
+  for (int q = 2; q <= 4; ++q)
+    if (padded(q) < padded(c)) c = q;
+  if (dual) {
+    if (c == 2) launch_one<EPI, true, kRowsDual, 2>(g, row_cap, st, n_nets);
+    else if (c == 3) launch_one<EPI, true, kRowsDual, 3>(g, row_cap, st, n_nets);
+    else launch_one<EPI, true, kRowsDual, 4>(g, row_cap, st, n_nets);
   } else {
-    if (!n_ok) return;
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-      const int m = m0 + ty * TM + i;
-      float v[TN] = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]};
-      float* o = static_cast<float*>(g.out) + (size_t)m * g.ldo + (size_t)e * g.out_net + nb;
-      if (EPI == kEpiMul || EPI == kEpiStoreMul) {
-        const float4 a = *reinterpret_cast<const float4*>(
-            static_cast<const float*>(g.aux) + (size_t)m * g.ld_aux + (size_t)e * g.aux_net + nb);
-        if (EPI == kEpiStoreMul) {
-          *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
-          o = static_cast<float*>(g.out2) + (size_t)m * g.ldo + (size_t)e * g.out_net + nb;
-        }
-        v[0] *= a.x; v[1] *= a.y; v[2] *= a.z; v[3] *= a.w;
-      }
-      *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
-    }
+    if (c == 2) launch_one<EPI, false, kRows, 2>(g, row_cap, st, n_nets);
+    else if (c == 3) launch_one<EPI, false, kRows, 3>(g, row_cap, st, n_nets);
+    else launch_one<EPI, false, kRows, 4>(g, row_cap, st, n_nets);
+  }
+}
+
+template <int EPI, int C>
+cudaError_t allow_smem() {
+  cudaError_t e = cudaFuncSetAttribute((const void*)k_gemm_fp32<EPI, false, kRows, C>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       gemm_smem<false, kRows, C>());
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute((const void*)k_gemm_fp32<EPI, true, kRowsDual, C>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem<true, kRowsDual, C>());
+}
+template <int EPI>
+cudaError_t allow_epi() {
+  cudaError_t e = allow_smem<EPI, 2>();
+  if (e == cudaSuccess) e = allow_smem<EPI, 3>();
+  return e == cudaSuccess ? allow_smem<EPI, 4>() : e;
+}
+
+void launch_any(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets, bool dual) {
+  switch (g.epi) {
+    case kEpiCelu: launch_epi<kEpiCelu>(g, row_cap, st, n_nets, dual); break;
+    case kEpiCeluDot: launch_epi<kEpiCeluDot>(g, row_cap, st, n_nets, dual); break;
+    case kEpiMul: launch_epi<kEpiMul>(g, row_cap, st, n_nets, dual); break;
+    default: launch_epi<kEpiStore>(g, row_cap, st, n_nets, dual); break;
   }
 }
 
 }  // namespace
 
-void launch_gemm_fp32(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets) {
-  dim3 grid((row_cap + BM - 1) / BM, (g.N + BN - 1) / BN, n_nets);
-  switch (g.epi) {
-    case kEpiCelu: k_gemm_fp32<kEpiCelu><<<grid, kThreads, 0, st>>>(g); break;
-    case kEpiCeluDot: k_gemm_fp32<kEpiCeluDot><<<grid, kThreads, 0, st>>>(g); break;
-    case kEpiMul: k_gemm_fp32<kEpiMul><<<grid, kThreads, 0, st>>>(g); break;
-    case kEpiStoreMul: k_gemm_fp32<kEpiStoreMul><<<grid, kThreads, 0, st>>>(g); break;
-    default: k_gemm_fp32<kEpiStore><<<grid, kThreads, 0, st>>>(g); break;
-  }
+cudaError_t gemm_fp32_ensure_smem() {
+  cudaError_t e = allow_epi<kEpiCelu>();
+  if (e == cudaSuccess) e = allow_epi<kEpiCeluDot>();
+  if (e == cudaSuccess) e = allow_epi<kEpiMul>();
+  return e == cudaSuccess ? allow_epi<kEpiStore>() : e;
 }
 
-void launch_gemm_fp32(const GemmArgs& g, int row_cap, cudaStream_t st) {
-  launch_gemm_fp32(g, row_cap, st, 1);
+void launch_gemm_fp32(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets) {
+  launch_any(g, row_cap, st, n_nets, false);
+}
+void launch_gemm_dual(const GemmArgs& g, int row_cap, cudaStream_t st, int n_nets) {
+  launch_any(g, row_cap, st, n_nets, true);
 }
 
 // the six GEMMs of one forward + backward-to-input pass over every species
@@ -192,6 +342,7 @@ void launch_mlp_fp32(const Ws& ws, const MlpDims& md, const MlpWeights& mw, cons
   GemmArgs g{};
   g.alpha = alpha;
   g.seg_start = ws.seg_start;
+  g.counts = ws.species_count;
   g.S = S;
   g.e_row = mb.e_row;
   g.e_row_net = R;
@@ -203,9 +354,11 @@ void launch_mlp_fp32(const Ws& ws, const MlpDims& md, const MlpWeights& mw, cons
   g.N = E * h1; g.K = Dp;
   g.out = mb.H1; g.out2 = mb.D1; g.ldo = E * h1; g.out_net = 0;
   g.epi = kEpiCelu;
+  g.kmask = ws.row_mask ? ws.tile_mask : nullptr;
   if (hook) hook->begin(3);
   launch_gemm_fp32(g, R, st, 1);
   if (hook) hook->end();
+  g.kmask = nullptr;
   // L2: per member
   g.A = mb.H1; g.lda = E * h1; g.a_net = h1;
   g.B = mw.W2; g.b_s = (long long)h2 * h1; g.b_e = (long long)S * h2 * h1; g.ldb = h1;
@@ -257,6 +410,7 @@ void launch_mlp_fp32(const Ws& ws, const MlpDims& md, const MlpWeights& mw, cons
   g.N = Dp; g.K = E * h1;
   g.out = ws.dEdG; g.ldo = Dp; g.out_net = 0;
   g.epi = kEpiStore;
+  g.nmask = ws.row_mask ? ws.tile_mask : nullptr;
   if (hook) hook->begin(8);
   launch_gemm_fp32(g, R, st, 1);
   if (hook) hook->end();

@@ -13,37 +13,50 @@ struct VjpBufs {
   float* Q;         // [rows][Dp] q = H_e u
   float *H1, *D1, *Z1d, *H1d;   // [rows][E*h1]
   float *H2, *D2, *Z2d, *H2d;   // [rows][E*h2]
-  float *H3, *D3, *Z3d, *H3d;   // [rows][E*h3]
-  float *A1h, *A1z, *dl1, *dl1d;
-  float *A2h, *A2z, *dl2, *dl2d;
+  float *H3, *H3d;              // [rows][E*h3]
+  float *dl1, *dl1d;
+  float *dl2, *dl2d;
   float *dl3, *dl3d;
   float* e_row;     // [E][rows]
 };
 
-struct WgradArgs {
+// One layer of the weight-gradient launch: X (deltas and their tangents) against
+// Y (the layer's inputs and their tangents)
+struct WgradLayer {
   const float *X1, *X2;
   int ldx, x_net;
   const float *Y1, *Y2;
   int ldy, y_net;
-  int n_out, n_in, n_in_real, S;
+  int n_out, n_in, n_in_real;   // n_in_real: columns of W (the rest is padding)
+  long long off;                // of W within a network's flat parameters
+  const int16_t* feat_of_col;   // first layer: paper index of the feature of AEV column k
+  int masked;                   // Y holds sparse AEV rows: skip a tile's dead slices
+};
+
+struct WgradArgs {
+  WgradLayer layer[3];
+  int tile0[4];                 // first tile of each layer; [3]: the output layer's
+  const float *H3, *H3d;        // output layer: [rows][E*h3]
+  int h3;
+  long long off4;
+  int S, E;
   float scale;
   float* out;
-  long long per_net, layer_off;
-  const int16_t* feat_of_col;   // first layer: paper index of the feature of AEV column k
+  long long per_net;
+  const int* seg_start;
+  const int* counts;
+  const float* gE_row;
+  const uint32_t* tile_mask;    // null: dense rows
+  int group;                    // 128-row tiles per CTA
 };
 
 cudaError_t vjp_set_smem(const Ws& ws);
-void launch_vjp_zero(const Ws& ws, const VjpBufs& vb, int n_in, cudaStream_t st);
 void launch_gather_v(const Ws& ws, const VjpBufs& vb, int n_in, cudaStream_t st);
-void launch_aev_jvp(const Ws& ws, const AevConst& ac, const VjpBufs& vb, int n_in, cudaStream_t st);
+// the AEV rows (FP32) and their tangents along v
+void launch_aev_fwd_vjp(const Ws& ws, const AevConst& ac, const VjpBufs& vb, int n_in, cudaStream_t st);
+// forces and their tangents
 void launch_aev_bwd_dual(const Ws& ws, const AevConst& ac, const VjpBufs& vb, int n_in, cudaStream_t st);
-void launch_vjp_out3(const Ws& ws, const VjpBufs& vb, const float* w4, int S, int E, int h3, float alpha,
-                     cudaStream_t st);
-void launch_vjp_delta(const Ws& ws, int S, int width, const float* Ah, const float* Az, const float* D,
-                      const float* Zd, float* dl, float* dld, float alpha, cudaStream_t st);
-void launch_wgrad(const WgradArgs& a, const Ws& ws, const VjpBufs& vb, int E, cudaStream_t st);
-void launch_wgrad_out(const Ws& ws, const VjpBufs& vb, int S, int E, int h3, float* out, long long per_net,
-                      long long off4, cudaStream_t st);
+void launch_wgrad(WgradArgs a, int row_cap, cudaStream_t st);
 void launch_vjp_scatter(const Ws& ws, const VjpBufs& vb, int n_in, cudaStream_t st);
 
 }  // namespace nnp
