@@ -9,6 +9,8 @@ from __future__ import annotations
 import ctypes
 import os
 
+import numpy as np
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 # NNP_DEBUG_BOUNDS=1 in the environment selects the bounds-checked build
 DEBUG_BOUNDS = os.environ.get("NNP_DEBUG_BOUNDS", "0") not in ("", "0")
@@ -100,6 +102,10 @@ class RequestT(ctypes.Structure):
                 ("forces", ctypes.c_void_p)]
 
 
+# the same layouts for filling a whole batch's descriptors column by column
+SYSTEM_DTYPE = np.dtype(SystemT)
+VJP_SYSTEM_DTYPE = np.dtype(VjpSystemT)
+
 _lib = None
 
 
@@ -119,7 +125,7 @@ def lib():
     L.nnp_destroy.restype = None
     L.nnp_reserve.argtypes = [P, i64, i, i, i]
     L.nnp_energy_forces.argtypes = [P, i64, P, P, P, P, P, P, P, P]
-    L.nnp_energy_forces_batch.argtypes = [P, i, ctypes.POINTER(SystemT), P]
+    L.nnp_energy_forces_batch.argtypes = [P, i, P, P]   # SystemT array
     L.nnp_energy_forces_host.argtypes = [P, i64, P, P, P, P, P, P, P]
     L.nnp_sync_status.argtypes = [P, P]
     L.nnp_aev_dim.argtypes = [P]
@@ -146,7 +152,7 @@ def lib():
     L.nnp_server_submit.argtypes = [P, ctypes.POINTER(RequestT), ctypes.POINTER(ctypes.c_uint64)]
     L.nnp_server_poll.argtypes = [P, ctypes.c_uint64, i, ctypes.POINTER(ctypes.c_double)]
     L.nnp_server_stats.argtypes = [P, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong)]
-    L.nnp_force_vjp_batch.argtypes = [P, i, ctypes.POINTER(VjpSystemT), P, P]
+    L.nnp_force_vjp_batch.argtypes = [P, i, P, P, P]    # VjpSystemT array
     L.nnp_force_vjp.argtypes = [P, i64, P, P, P, P, ctypes.c_double, P, P, P, P, P, P]
     L.nnp_n_weights.argtypes = [P]
     L.nnp_n_weights.restype = i64

@@ -17,6 +17,7 @@ class NNPFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, coords, weights, potential, species, box=None, mask=None):
         E, F = potential.energy_forces(coords.detach().contiguous(), species, box, mask)
+        ctx.set_materialize_grads(False)   # an unused output's gradient stays None
         ctx.potential, ctx.species, ctx.box, ctx.mask = potential, species, box, mask
         ctx.save_for_backward(coords)
         return E, F
@@ -25,11 +26,11 @@ class NNPFunction(torch.autograd.Function):
     def backward(ctx, gE, gF):
         (coords,) = ctx.saved_tensors
         pot = ctx.potential
-        gE = torch.zeros(1, dtype=torch.float64, device=coords.device) if gE is None else gE
+        gE = 0.0 if gE is None else float(gE.reshape(-1)[0])
         gF = torch.zeros_like(coords) if gF is None else gF
         sys = {"coords": coords.detach().contiguous(), "species": ctx.species, "box": ctx.box,
                "mask": ctx.mask}
-        _, _, G, W = pot.force_vjp_batch([sys], [float(gE.reshape(-1)[0])], [gF])
+        _, _, G, W = pot.force_vjp_batch([sys], [gE], [gF])
         return G[0], W, None, None, None, None
 
 
@@ -39,24 +40,16 @@ class NNPBatchFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, coords, weights, potential, species, sizes, boxes=None):
-        xs = torch.split(coords.detach().contiguous(), sizes)
-        ss = torch.split(species, sizes)
-        systems = [{"coords": x.contiguous(), "species": s.contiguous(),
-                    "box": None if boxes is None else boxes[k]}
-                   for k, (x, s) in enumerate(zip(xs, ss))]
-        outs = potential.energy_forces_batch(systems)
-        E = torch.cat([o["energy"] for o in outs])
-        F = torch.cat([o["forces"] for o in outs])
-        ctx.potential, ctx.systems, ctx.sizes = potential, systems, sizes
+        x, sp = coords.detach().contiguous(), species.contiguous()
+        E, F = potential.energy_forces_flat(x, sp, sizes, boxes)
+        ctx.set_materialize_grads(False)   # an unused output's gradient stays None
+        ctx.potential, ctx.x, ctx.sp, ctx.sizes, ctx.boxes = potential, x, sp, sizes, boxes
         return E, F
 
     @staticmethod
     def backward(ctx, gE, gF):
-        n = len(ctx.systems)
-        dev = ctx.systems[0]["coords"].device
-        gE = torch.zeros(n, dtype=torch.float64, device=dev) if gE is None else gE
-        gF = torch.zeros((sum(ctx.sizes), 3), device=dev) if gF is None else gF
-        gEs = gE.detach().double().cpu().tolist()
-        gFs = [g.contiguous() for g in torch.split(gF.detach().float(), ctx.sizes)]
-        _, _, G, W = ctx.potential.force_vjp_batch(ctx.systems, gEs, gFs)
-        return torch.cat(G), W, None, None, None, None
+        n = len(ctx.sizes)
+        gEs = [0.0] * n if gE is None else gE.detach().double().cpu().tolist()
+        gFs = torch.zeros_like(ctx.x) if gF is None else gF.detach().float().contiguous()
+        G, W = ctx.potential.force_vjp_flat(ctx.x, ctx.sp, ctx.sizes, ctx.boxes, gEs, gFs)
+        return G, W, None, None, None, None

@@ -87,25 +87,26 @@ __global__ void __launch_bounds__(kWarps * 32) k_aev_fwd_vjp(Ws ws, AevConst ac,
   float* U = vb.U + (size_t)slot * ac.Dp;
   load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
   const uint32_t msk = ws.row_mask ? row_slices(H, ac, lane, pair_su) : ~0u;
+  // (the values are formed exactly as in k_aev_fwd: CELU'' jumps at z = 0, so a
+  // gradient depends on the last bits of G where a pre-activation is next to zero)
+  const float inv_rc_r = 1.f / ac.rc_r, inv_rc_a = 1.f / ac.rc_a;
   stage_list(H.off_r[ac.S], ws.nb_r + (size_t)p * ws.cap_r, xi, d, ws, lane,
              [&](int t, int j, const Geo& g) {
                const float4 vj = vb.v_pos[j];
-               const float r = sqrtf(g.dx * g.dx + g.dy * g.dy + g.dz * g.dz);
-               const float rdot = (g.dx * (vj.x - vi.x) + g.dy * (vj.y - vi.y) + g.dz * (vj.z - vi.z)) / r;
+               const float rdot = (g.dx * (vj.x - vi.x) + g.dy * (vj.y - vi.y) + g.dz * (vj.z - vi.z)) / g.r;
                float f, df, ddf;
-               fcut3(r, ac.rc_r, &f, &df, &ddf);
-               rad[t] = make_float4(r, f, df, rdot);
+               fcut3(g.r, ac.rc_r, &f, &df, &ddf);
+               rad[t] = make_float4(g.r, fcut(g.r, ac.rc_r, inv_rc_r), df, rdot);
              });
   stage_list(H.off_a[ac.S], ws.nb_a + (size_t)p * ws.cap_a, xi, d, ws, lane,
              [&](int t, int j, const Geo& g) {
                const float4 vj = vb.v_pos[j];
-               const float r = sqrtf(g.dx * g.dx + g.dy * g.dy + g.dz * g.dz);
-               const float inv = 1.f / r;
+               const float inv = rcp_approx(g.r);
                const float dvx = vj.x - vi.x, dvy = vj.y - vi.y, dvz = vj.z - vi.z;
                float f, df, ddf;
-               fcut3(r, ac.rc_a, &f, &df, &ddf);
-               angv[t] = make_float4(g.dx * inv, g.dy * inv, g.dz * inv, r);
-               angf[t] = make_float4(f, df, (g.dx * dvx + g.dy * dvy + g.dz * dvz) * inv, inv);
+               fcut3(g.r, ac.rc_a, &f, &df, &ddf);
+               angv[t] = make_float4(g.dx * inv, g.dy * inv, g.dz * inv, g.r);
+               angf[t] = make_float4(fcut(g.r, ac.rc_a, inv_rc_a), df, (g.dx * dvx + g.dy * dvy + g.dz * dvz) * inv, inv);
                angd[t] = make_float4(dvx, dvy, dvz, 0.f);
              });
   __syncwarp();
@@ -159,8 +160,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_aev_fwd_vjp(Ws ws, AevConst ac,
                          ((uj.x - chat * uk.x) * dk.x + (uj.y - chat * uk.y) * dk.y +
                           (uj.z - chat * uk.z) * dk.z) * fk.w;
       const float c = ac.cos_scale * chat;
-      const float sn = fmaxf(sin_theta(uj, uk, chat, ac.cos_scale), 1e-6f);
-      const float m_cs = -c * rcp_approx(sn);
+      const float sn = sin_theta(uj, uk, chat, ac.cos_scale);
+      const float m_cs = -c * rcp_approx(fmaxf(sn, 1e-6f));
       const float rb = 0.5f * (uj.w + uk.w), rbdot = 0.5f * (fj.z + fk.z);
       const float fjk = ac.ang_pre * fj.x * fk.x;
       const float fjkdot = ac.ang_pre * (fj.y * fj.z * fk.x + fj.x * fk.y * fk.z);

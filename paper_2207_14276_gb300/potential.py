@@ -6,6 +6,7 @@ only allocates device memory and supplies the CUDA stream.
 from __future__ import annotations
 
 import ctypes
+import struct
 
 import numpy as np
 import torch
@@ -21,6 +22,40 @@ def _ptr(t):
 def _stream_ptr(stream):
     s = stream if stream is not None else torch.cuda.current_stream()
     return ctypes.c_void_p(s.cuda_stream)
+
+
+# one nnp_system_t: a pack per system costs less than a dozen ctypes field stores
+_pack_system = struct.Struct("=qQQQdddiiQQQQ").pack
+
+
+def _packed(s, o):
+    """The nnp_system_t of one system dict and its output tensors."""
+    x, m, box = s["coords"], s.get("mask"), s.get("box")
+    f, v, a = o.get("forces"), o.get("virial"), o.get("atom_energies")
+    edges = (0.0, 0.0, 0.0, 0) if box is None else (float(box[0]), float(box[1]), float(box[2]), 1)
+    return _pack_system(x.shape[0], x.data_ptr(), s["species"].data_ptr(),
+                        0 if m is None else m.data_ptr(), *edges, 0, o["energy"].data_ptr(),
+                        0 if f is None else f.data_ptr(), 0 if v is None else v.data_ptr(),
+                        0 if a is None else a.data_ptr())
+
+
+def _flat_systems(dtype, coords, species, sizes, boxes):
+    """(descriptors, first atom of each system) of a concatenated batch."""
+    n = np.asarray(sizes, dtype=np.int64).reshape(-1)
+    if len(n) == 0 or coords.shape[0] != n.sum() or species.shape[0] != n.sum() or (n < 0).any():
+        raise RuntimeError(f"sizes add up to {int(n.sum())} atoms, coords and species hold "
+                           f"{coords.shape[0]} and {species.shape[0]}")
+    off = (np.cumsum(n) - n).astype(np.uint64)
+    arr = np.zeros(len(n), dtype=dtype)
+    arr["n_atoms"] = n
+    arr["coords"] = coords.data_ptr() + 12 * off
+    arr["species"] = species.data_ptr() + off
+    if boxes is not None:
+        for k in range(len(n)):
+            if boxes[k] is not None:
+                arr["periodic"][k] = 1
+                arr["box"][k] = [float(boxes[k][c]) for c in range(3)]
+    return arr, off
 
 
 class Potential:
@@ -184,9 +219,7 @@ class Potential:
                             virial=False, outputs=None, forces=True):
         """systems: list of dicts with coords, species, optional box and mask (cuda tensors).
         Returns a list of dicts with energy [1], forces [n,3] (and virial / atom energies)."""
-        L = lib()
         n_sys = len(systems)
-        arr = (_lib.SystemT * max(n_sys, 1))()
         outs = outputs
         if outs is None:
             outs = []
@@ -201,23 +234,16 @@ class Potential:
                 if atom_energies:
                     o["atom_energies"] = torch.empty(n, dtype=torch.float32, device=dev)
                 outs.append(o)
-        for k, (s, o) in enumerate(zip(systems, outs)):
-            d = arr[k]
-            d.n_atoms = s["coords"].shape[0]
-            d.coords = s["coords"].data_ptr()
-            d.species = s["species"].data_ptr()
-            d.mask = s["mask"].data_ptr() if s.get("mask") is not None else None
-            box = s.get("box")
-            d.periodic = 1 if box is not None else 0
-            if box is not None:
-                for c in range(3):
-                    d.box[c] = float(box[c])
-            d.energy = o["energy"].data_ptr()
-            d.forces = o["forces"].data_ptr() if "forces" in o else None
-            d.virial = o["virial"].data_ptr() if "virial" in o else None
-            d.atom_energies = o["atom_energies"].data_ptr() if "atom_energies" in o else None
+        buf = b"".join([_packed(s, o) for s, o in zip(systems, outs)])
+        buf += bytes(_lib.SYSTEM_DTYPE.itemsize * n_sys - len(buf))   # fewer outputs: refused below
+        self._run_batch(buf, n_sys, stream, check_status)
+        return outs
+
+    def _run_batch(self, descriptors, n_sys, stream, check_status=True):
+        # descriptors: bytes or an array of nnp_system_t
+        d = descriptors if isinstance(descriptors, bytes) else descriptors.ctypes.data
         for attempt in range(2):
-            check(L.nnp_energy_forces_batch(self._h, n_sys, arr, _stream_ptr(stream)))
+            check(lib().nnp_energy_forces_batch(self._h, n_sys, d, _stream_ptr(stream)))
             if not check_status:
                 break
             rc = self.sync_status(stream)
@@ -225,7 +251,20 @@ class Potential:
                 continue
             check(rc)
             break
-        return outs
+
+    def energy_forces_flat(self, coords, species, sizes, boxes=None):
+        """Energies [n_sys] and forces [sum(sizes), 3] of systems concatenated along the
+        atom axis (coords and species contiguous cuda tensors; boxes: per-system boxes
+        or None).  The descriptors are offsets into the flat tensors, filled for the
+        whole batch at once: one Python pass per system, two allocations and two
+        concatenations cost a training step on 64 molecules 1.1 ms of 2.1 ms."""
+        arr, off = _flat_systems(_lib.SYSTEM_DTYPE, coords, species, sizes, boxes)
+        E = torch.empty(len(sizes), dtype=torch.float64, device=coords.device)
+        F = torch.empty((coords.shape[0], 3), dtype=torch.float32, device=coords.device)
+        arr["energy"] = E.data_ptr() + 8 * np.arange(len(sizes), dtype=np.uint64)
+        arr["forces"] = F.data_ptr() + 12 * off
+        self._run_batch(arr, len(sizes), None)
+        return E, F
 
     def energy_forces_host(self, coords, species, box=None, mask=None, virial=False):
         """Host numpy arrays in and out; copies and synchronisation inside the library."""
@@ -255,42 +294,47 @@ class Potential:
         floats; dL_dF: list of cuda float32 [n,3].  Returns (energies [n_sys] float64,
         forces list, dL/dcoords list, dL/dweights flat float32)."""
         n_sys = len(systems)
-        arr = (_lib.VjpSystemT * n_sys)()
         dev = systems[0]["coords"].device
         E = torch.empty(n_sys, dtype=torch.float64, device=dev)
-        Fs, Gs, keep = [], [], []
-        for k, s in enumerate(systems):
-            n = s["coords"].shape[0]
-            F = torch.empty((n, 3), dtype=torch.float32, device=dev)
-            G = torch.empty((n, 3), dtype=torch.float32, device=dev)
-            v = dL_dF[k].contiguous().float()
-            keep.append(v)
-            d = arr[k]
-            d.sys.n_atoms = n
-            d.sys.coords = s["coords"].data_ptr()
-            d.sys.species = s["species"].data_ptr()
-            d.sys.mask = s["mask"].data_ptr() if s.get("mask") is not None else None
-            box = s.get("box")
-            d.sys.periodic = 1 if box is not None else 0
-            if box is not None:
-                for c in range(3):
-                    d.sys.box[c] = float(box[c])
-            d.sys.energy = E.data_ptr() + 8 * k
-            d.sys.forces = F.data_ptr()
-            d.dL_dE = float(dL_dE[k])
-            d.dL_dF = v.data_ptr()
-            d.dL_dcoords = G.data_ptr()
-            Fs.append(F)
-            Gs.append(G)
+        Fs = [torch.empty((s["coords"].shape[0], 3), dtype=torch.float32, device=dev) for s in systems]
+        Gs = [torch.empty_like(f) for f in Fs]
+        keep = [dL_dF[k].contiguous().float() for k in range(n_sys)]
+        arr = np.zeros(n_sys, dtype=_lib.VJP_SYSTEM_DTYPE)
+        arr["sys"] = np.frombuffer(b"".join([_packed(s, {"energy": E[k:k + 1], "forces": Fs[k]})
+                                             for k, s in enumerate(systems)]), dtype=_lib.SYSTEM_DTYPE)
+        arr["dL_dE"] = [float(dL_dE[k]) for k in range(n_sys)]
+        arr["dL_dF"] = np.array([v.data_ptr() for v in keep], dtype=np.uint64)
+        arr["dL_dcoords"] = np.array([g.data_ptr() for g in Gs], dtype=np.uint64)
+        return E, Fs, Gs, self._run_vjp(arr, n_sys, dev, stream)
+
+    def force_vjp_flat(self, coords, species, sizes, boxes, dL_dE, dL_dF):
+        """force_vjp_batch of systems concatenated along the atom axis (as in
+        energy_forces_flat): (dL/dcoords [sum(sizes), 3], dL/dweights).  dL_dE: per-system
+        floats; dL_dF: contiguous cuda float32 [sum(sizes), 3]."""
+        n_sys, dev = len(sizes), coords.device
+        arr = np.zeros(n_sys, dtype=_lib.VJP_SYSTEM_DTYPE)
+        sys, off = _flat_systems(_lib.SYSTEM_DTYPE, coords, species, sizes, boxes)
+        E = torch.empty(n_sys, dtype=torch.float64, device=dev)
+        F = torch.empty((coords.shape[0], 3), dtype=torch.float32, device=dev)
+        G = torch.empty_like(F)
+        sys["energy"] = E.data_ptr() + 8 * np.arange(n_sys, dtype=np.uint64)
+        sys["forces"] = F.data_ptr() + 12 * off
+        arr["sys"] = sys
+        arr["dL_dE"] = dL_dE
+        arr["dL_dF"] = dL_dF.data_ptr() + 12 * off
+        arr["dL_dcoords"] = G.data_ptr() + 12 * off
+        return G, self._run_vjp(arr, n_sys, dev, None)
+
+    def _run_vjp(self, arr, n_sys, dev, stream):
         W = torch.empty(self.n_weights, dtype=torch.float32, device=dev)
         for attempt in range(2):
-            check(lib().nnp_force_vjp_batch(self._h, n_sys, arr, _ptr(W), _stream_ptr(stream)))
+            check(lib().nnp_force_vjp_batch(self._h, n_sys, arr.ctypes.data, _ptr(W), _stream_ptr(stream)))
             rc = self.sync_status(stream)
             if rc == _lib.NNP_ERR_CAPACITY and attempt == 0:
                 continue
             check(rc)
             break
-        return E, Fs, Gs, W
+        return W
 
     def profile(self, enable=True):
         check(lib().nnp_profile(self._h, 1 if enable else 0))
