@@ -82,6 +82,13 @@ struct Model {
 
 }  // namespace
 
+// descriptors and arguments of a graph's kernel node
+struct FrontSent {
+  nnp::BatchParams bp;
+  int a, b;
+  unsigned grid;
+};
+
 struct nnp_handle {
   Model* model = nullptr;
   size_t budget = 0;
@@ -92,7 +99,9 @@ struct nnp_handle {
   bool dirty = true;  // capacities changed: re-carve before the next call
   Ws ws{};
   MlpBufs mb{};
-  int* status_host = nullptr;  // pinned: [4] status words, then out_host
+  int* status_host = nullptr;  // pinned: [4] status words, [4] published ones, then out_host
+  bool pub_valid = false;      // the last call's end copies the status word to the published one
+  cudaStream_t pub_stream = nullptr;   // and ran on this stream
   double* out_host = nullptr;  // pinned [10]: energy and virial of a host-buffer call
   int last_launches = 0;
   int last_n_in = 0;
@@ -106,9 +115,12 @@ struct nnp_handle {
   size_t vjp_bytes = 0;
   int vjp_rows = 0;
   VjpBufs vb{};
-  // the part of a call after its descriptors are on the device, as a CUDA graph
+  // the calls of one shape as a CUDA graph
   cudaStream_t cap_stream = nullptr;
+  cudaGraph_t graph = nullptr;      // kept: the nodes below belong to it
   cudaGraphExec_t gexec = nullptr;
+  std::vector<cudaGraphNode_t> front_nodes;   // the kernels that take the descriptors
+  std::vector<FrontSent> front_sent;          // what those nodes hold now
   std::string gsig;       // shape signature of the captured call
   std::string last_sig;   // shape signature of the previous eager call
   int last_launches_graph = 0;
@@ -370,6 +382,8 @@ size_t carve(nnp_handle* h, char* base) {
   Carve c{base};
   Ws& ws = h->ws;
   ws.status = c.take<int>(4);
+  // (the bounds-checked build's last kernel may still set a flag)
+  ws.status_pub = kBoundsChecked ? nullptr : h->status_host + 4;
   ws.sys = c.take<SysDev>(nsys);
   ws.cell_cap = (int)cells;
   ws.row_cap = (int)rows;
@@ -575,16 +589,15 @@ void split_box(double L, float* hi, float* lo, float* inv) {
 // the chain in one CTA
 constexpr int kFrontMaxAtoms = 2048;
 
-// A batch's work is enqueued in two parts.  enqueue_front launches the kernels
-// that take the per-call descriptors (pointers, sizes, boxes) as parameters and
-// leave them in ws.sys; enqueue_rest launches the others, which read them from
-// there.  The second part depends only on the batch's shape and the handle's
-// settings, so its CUDA graph serves every call of that shape, whatever buffers
-// the call brings.
-// (A graph over both parts replayed only when every pointer repeated: a caller
-// that allocates its outputs got eager launches or a new capture instead.
-// water9000 with BF16 networks and outputs allocated on each call 268 -> 212 us, two
-// hybrid MD steps on 20k atoms 426 -> 354 us.)
+// A call's kernels are, first, those that take the per-call descriptors (pointers,
+// sizes, boxes) as parameters and leave them in ws.sys (front_launches), then the
+// others, which read them from there (enqueue_rest) and depend only on the batch's
+// shape and the handle's settings.  A shape's CUDA graph holds both; the nodes of the
+// first part get the call's descriptors before each launch, so that the graph serves
+// every call of its shape, whatever buffers the call brings, in one launch.
+// (Keyed by the pointers, a caller that allocates its outputs got eager launches or a
+// new capture instead: water9000 with BF16 networks and outputs allocated on each call
+// 268 us, with the first part launched eagerly 212 us, with its nodes updated 203 us.)
 bool one_cta_front(const nnp_handle* h, size_t n_chunks, int n_in) {
   return n_chunks == 1 && n_in > 0 && n_in <= kFrontMaxAtoms && !h->ws.skin_state;
 }
@@ -614,51 +627,7 @@ bool sparse_call(const nnp_handle* h) {
   return h->sparse_rows && !fuses_aev_l1(h) && !(m.net == kNetSimt && mlp_fused_supported(m.md));
 }
 
-int enqueue_front(nnp_handle* h, int n_sys, const nnp_system_t* sy, const std::vector<BatchParams>& chunks,
-                  int n_in, cudaStream_t st, int* n_launch) {
-  const Model& m = *h->model;
-  Ws& ws = h->ws;
-  int launches = 0, rc = NNP_OK;
-  // systems without atoms: the outputs are the empty sums
-  for (int b = 0; b < n_sys; ++b)
-    if (sy[b].n_atoms == 0) {
-      CU_TRY(cudaMemsetAsync(sy[b].energy, 0, sizeof(double), st));
-      if (sy[b].virial) CU_TRY(cudaMemsetAsync(sy[b].virial, 0, 9 * sizeof(double), st));
-      launches += 1 + (sy[b].virial ? 1 : 0);
-    }
-  // persistent lists: the displacement check decides on the device whether this
-  // call rebuilds them (a new batch layout or a capacity change always does)
-  if (ws.skin_state) {
-    const bool forced = !h->lists_valid;
-    CU_TRY(cudaMemsetAsync(ws.skin_state, 0, sizeof(int), st));
-    CU_TRY(cudaMemsetAsync(ws.skin_state + 1, forced ? 1 : 0, sizeof(int), st));
-    launches += 2;
-    if (!forced)
-      for (const auto& bp : chunks) {
-        int n_chunk = 0;
-        for (int k = 0; k < bp.n_sys; ++k) n_chunk += bp.sys[k].n_in;
-        if (n_chunk > 0) { launch_skin_check(ws, bp, n_chunk, st); ++launches; }
-      }
-    if ((rc = launch_check("displacement check"))) return rc;
-  }
-  // small one-chunk batches: the whole front end in one single-CTA launch
-  if (one_cta_front(h, chunks.size(), n_in)) {
-    StageTimer t(h, st, 0);
-    launch_front(ws, chunks[0], call_const(h), n_in, st);
-    ++launches;
-  } else {
-    for (const auto& bp : chunks) { launch_init_chunk(ws, bp, st); ++launches; }
-    for (const auto& bp : chunks) {
-      int n_chunk = 0;
-      for (int k = 0; k < bp.n_sys; ++k) n_chunk += bp.sys[k].n_in;
-      if (n_chunk > 0) { launch_prep_atoms(ws, bp, n_chunk, m.ac.S, st); ++launches; }
-    }
-  }
-  *n_launch += launches;
-  return launch_check("init/prep");
-}
-
-// front_done: enqueue_front ran the whole front end; energy_only: no system asks
+// front_done: the whole front end ran in the first part's one CTA; energy_only: no system asks
 // for forces or a virial
 int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool energy_only,
                  cudaStream_t st, int* n_launch) {
@@ -722,6 +691,79 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool
   CU_TRY(cudaGetLastError());
   *n_launch += launches;
   return rc;
+}
+
+void drop_graph(nnp_handle* h) {
+  if (h->gexec) cudaGraphExecDestroy(h->gexec);
+  if (h->graph) cudaGraphDestroy(h->graph);
+  h->gexec = nullptr;
+  h->graph = nullptr;
+  h->front_nodes.clear();
+  h->front_sent.clear();
+}
+
+// a call's graph: its first part as kernel nodes, the rest captured behind them
+int capture_call(nnp_handle* h, const std::vector<FrontLaunch>& front, int n_in, bool front_done,
+                 bool any_virial, bool energy_only) {
+  if (!h->cap_stream) CU_TRY(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+  drop_graph(h);
+  CU_TRY(cudaGraphCreate(&h->graph, 0));
+  for (const FrontLaunch& f : front) {
+    void* args[4];
+    f.args(args);
+    cudaKernelNodeParams p{};
+    p.func = const_cast<void*>(f.fn);
+    p.gridDim = dim3(f.grid);
+    p.blockDim = dim3(f.block);
+    p.kernelParams = args;
+    cudaGraphNode_t node, *prev = h->front_nodes.empty() ? nullptr : &h->front_nodes.back();
+    CU_TRY(cudaGraphAddKernelNode(&node, h->graph, prev, prev ? 1 : 0, &p));
+    h->front_nodes.push_back(node);
+  }
+  CU_TRY(cudaStreamBeginCaptureToGraph(h->cap_stream, h->graph, &h->front_nodes.back(), nullptr, 1,
+                                       cudaStreamCaptureModeThreadLocal));
+  int rest = 0;
+  const int rc = enqueue_rest(h, n_in, front_done, any_virial, energy_only, h->cap_stream, &rest);
+  cudaGraph_t same = nullptr;
+  const cudaError_t ec = cudaStreamEndCapture(h->cap_stream, &same);
+  cudaError_t ei = cudaSuccess;
+  if (rc == NNP_OK && ec == cudaSuccess) ei = cudaGraphInstantiate(&h->gexec, h->graph, 0);
+  if (rc != NNP_OK || ec != cudaSuccess || ei != cudaSuccess) {
+    if (ei != cudaSuccess) h->gexec = nullptr;
+    drop_graph(h);
+    if (rc) return rc;
+    return fail(NNP_ERR_CUDA, std::string(ec != cudaSuccess ? "graph capture: " : "graph instantiation: ") +
+                                  cudaGetErrorString(ec != cudaSuccess ? ec : ei));
+  }
+  h->last_launches_graph = rest + (int)front.size();
+  return NNP_OK;
+}
+
+// this call's descriptors into the graph's first nodes, where they differ from the
+// ones sent last
+int update_front(nnp_handle* h, const std::vector<FrontLaunch>& front) {
+  const bool first = h->front_sent.size() != front.size();
+  if (first) h->front_sent.resize(front.size());
+  for (size_t i = 0; i < front.size(); ++i) {
+    const FrontLaunch& f = front[i];
+    FrontSent& sent = h->front_sent[i];
+    const size_t nb = offsetof(BatchParams, sys) + (size_t)f.bp->n_sys * sizeof(SysIn);
+    if (!first && sent.a == f.a && sent.b == f.b && sent.grid == f.grid && !std::memcmp(&sent.bp, f.bp, nb))
+      continue;
+    void* args[4];
+    f.args(args);
+    cudaKernelNodeParams p{};
+    p.func = const_cast<void*>(f.fn);
+    p.gridDim = dim3(f.grid);
+    p.blockDim = dim3(f.block);
+    p.kernelParams = args;
+    CU_TRY(cudaGraphExecKernelNodeSetParams(h->gexec, h->front_nodes[i], &p));
+    std::memcpy(&sent.bp, f.bp, nb);
+    sent.a = f.a;
+    sent.b = f.b;
+    sent.grid = f.grid;
+  }
+  return NNP_OK;
 }
 
 // enqueue the whole chain for a batch whose descriptors are already validated
@@ -791,13 +833,25 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     h->last_sparse = sparse_call(h);
     h->last_vjp = false;
   }
+  const bool forced = ws.skin_state && !h->lists_valid;
+  const std::vector<FrontLaunch> front = front_launches(ws, chunks, call_const(h), n_in, front_done, forced);
+  h->pub_valid = ws.status_pub != nullptr && n_in > 0;
+  h->pub_stream = st;
+  // systems without atoms: the outputs are the empty sums
   int launches = 0;
-  rc = enqueue_front(h, n_sys, sy, chunks, n_in, st, &launches);
-  if (rc) return rc;
-  // the rest of a call of the previous call's shape (sizes, outputs wanted,
-  // settings, arena) is replayed from a CUDA graph: captured on the shape's second
-  // occurrence, replayed afterwards
-  if (!h->profile && n_in > 0) {
+  for (int b = 0; b < n_sys; ++b)
+    if (sy[b].n_atoms == 0) {
+      CU_TRY(cudaMemsetAsync(sy[b].energy, 0, sizeof(double), st));
+      if (sy[b].virial) CU_TRY(cudaMemsetAsync(sy[b].virial, 0, 9 * sizeof(double), st));
+      launches += 1 + (sy[b].virial ? 1 : 0);
+    }
+  // a stream under capture (the caller's own graph) gets the kernels themselves
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess) {
+    cudaGetLastError();
+    capturing = cudaStreamCaptureStatusActive;
+  }
+  if (!h->profile && n_in > 0 && capturing == cudaStreamCaptureStatusNone) {
     std::string sig;
     sig.reserve(128);
     auto put = [&](const void* p, size_t nb) { sig.append(static_cast<const char*>(p), nb); };
@@ -809,35 +863,17 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     put(&ws.row_cap, sizeof(int));
     put(&ws.cell_cap, sizeof(int));
     put(&h->skin, sizeof(h->skin));
-    const bool flags[] = {ws.skin_state != nullptr, front_done,    any_virial,     energy_only,
+    const bool flags[] = {ws.skin_state != nullptr, front_done,      any_virial,     energy_only,
                           h->fused_chain,           h->fused_aev_l1, h->sparse_rows, h->det};
     put(flags, sizeof(flags));
+    for (const FrontLaunch& f : front) put(&f.fn, sizeof(f.fn));   // the nodes, whose grids may change
+    // captured on the shape's second occurrence in a row, replayed afterwards
     if (!(h->gexec && sig == h->gsig) && sig == h->last_sig) {
-      if (!h->cap_stream) CU_TRY(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
-      CU_TRY(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-      int rest = 0;
-      rc = enqueue_rest(h, n_in, front_done, any_virial, energy_only, h->cap_stream, &rest);
-      cudaGraph_t graph = nullptr;
-      const cudaError_t ec = cudaStreamEndCapture(h->cap_stream, &graph);
-      if (rc) {
-        if (graph) cudaGraphDestroy(graph);
-        return rc;
-      }
-      if (ec != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
-        return fail(NNP_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ec));
-      }
-      if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
-      const cudaError_t ei = cudaGraphInstantiate(&h->gexec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (ei != cudaSuccess) {
-        h->gexec = nullptr;
-        return fail(NNP_ERR_CUDA, std::string("graph instantiation: ") + cudaGetErrorString(ei));
-      }
+      if ((rc = capture_call(h, front, n_in, front_done, any_virial, energy_only))) return rc;
       h->gsig = sig;
-      h->last_launches_graph = rest;
     }
     if (h->gexec && sig == h->gsig) {
+      if ((rc = update_front(h, front))) return rc;
       CU_TRY(cudaGraphLaunch(h->gexec, st));
       h->last_launches = launches + h->last_launches_graph;
       h->last_n_in = n_in;
@@ -846,6 +882,12 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     }
     h->last_sig = sig;
   }
+  for (const FrontLaunch& f : front) {
+    StageTimer t(h, st, 0);
+    f.launch(st);
+    ++launches;
+  }
+  if ((rc = launch_check("init/prep"))) return rc;
   rc = enqueue_rest(h, n_in, front_done, any_virial, energy_only, st, &launches);
   if (rc) return rc;
   h->last_launches = launches;
@@ -881,9 +923,10 @@ const char* nnp_last_error(void) { return g_err.c_str(); }
 namespace {
 bool alloc_host_words(nnp_handle* h) {
   void* p = nullptr;
-  if (cudaMallocHost(&p, 16 + 10 * sizeof(double)) != cudaSuccess) return false;
+  if (cudaMallocHost(&p, 32 + 10 * sizeof(double)) != cudaSuccess) return false;
+  std::memset(p, 0, 32);
   h->status_host = static_cast<int*>(p);
-  h->out_host = reinterpret_cast<double*>(static_cast<char*>(p) + 16);
+  h->out_host = reinterpret_cast<double*>(static_cast<char*>(p) + 32);
   return true;
 }
 }  // namespace
@@ -931,7 +974,7 @@ void nnp_destroy(nnp_handle* h) {
   if (!h) return;
   if (h->arena || h->stage || h->vjp_arena) cudaDeviceSynchronize();
   if (h->tc_state) mlp_tc_release(h->tc_state);
-  if (h->gexec) cudaGraphExecDestroy(h->gexec);
+  drop_graph(h);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->arena) cudaFree(h->arena);
   if (h->stage) cudaFree(h->stage);
@@ -1037,6 +1080,14 @@ int nnp_sync_status(nnp_handle* h, void* stream) {
   g_err.clear();
   if (!h) return fail(NNP_ERR_ARG, "null handle");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (h->arena && h->pub_valid && st == h->pub_stream) {
+    // the call's last kernel left the status word in host memory: only a raised flag
+    // is read back and cleared
+    CU_TRY(cudaStreamSynchronize(st));
+    volatile int* pub = h->status_host + 4;
+    if (pub[0] == 0) return NNP_OK;
+    pub[0] = 0;
+  }
   if (h->arena) CU_TRY(enqueue_status_read(h, st));
   CU_TRY(cudaStreamSynchronize(st));
   return h->arena ? status_result(h) : NNP_OK;
@@ -1293,15 +1344,11 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
     }
     chunks.push_back(bp);
   }
-  if (chunks.size() == 1 && n_in <= kFrontMaxAtoms) {
-    launch_front(ws, chunks[0], m.ac, n_in, st);
-  } else {
-    for (const auto& bp : chunks) launch_init_chunk(ws, bp, st);
-    for (const auto& bp : chunks) {
-      int n_chunk = 0;
-      for (int k = 0; k < bp.n_sys; ++k) n_chunk += bp.sys[k].n_in;
-      launch_prep_atoms(ws, bp, n_chunk, m.ac.S, st);
-    }
+  const bool front_done = chunks.size() == 1 && n_in <= kFrontMaxAtoms;
+  h->pub_valid = ws.status_pub != nullptr;
+  h->pub_stream = st;
+  for (const FrontLaunch& f : front_launches(ws, chunks, m.ac, n_in, front_done, false)) f.launch(st);
+  if (!front_done) {
     launch_setup(ws, m.ac, st);
     launch_bin(ws, n_in, st);
     launch_scan(ws, st);
@@ -1448,6 +1495,7 @@ int nnp_debug_wait_probe(nnp_handle* h, unsigned limit, void* stream) {
     int rc = ensure_arena(h, 1, 1);
     if (rc) return rc;
   }
+  h->pub_valid = false;
   launch_wait_probe(h->ws.status, limit, static_cast<cudaStream_t>(stream));
   CU_TRY(cudaGetLastError());
   return NNP_OK;
@@ -1708,10 +1756,9 @@ extern "C" int nnp_energy_forces_noalloc(nnp_handle* h, int64_t n_atoms, const f
       if (e != cudaSuccess) return fail(NNP_ERR_CUDA, std::string(name) + ": " + cudaGetErrorString(e));
       return NNP_OK;
     };
-    launch_init_chunk(ws, bp, st);
-    if ((rc = stage_ok("init"))) return rc;
-    launch_prep_atoms(ws, bp, n, m.ac.S, st);
-    if ((rc = stage_ok("prep"))) return rc;
+    const std::vector<BatchParams> chunks(1, bp);
+    for (const FrontLaunch& f : front_launches(ws, chunks, m.ac, n, false, false)) f.launch(st);
+    if ((rc = stage_ok("init/prep"))) return rc;
     launch_setup(ws, m.ac, st);
     launch_bin(ws, n, st);
     launch_scan(ws, st);

@@ -10,11 +10,16 @@ namespace {
 __global__ void k_finalize(Ws ws, const float* e_row, int E, int e_row_net,
                            const double* ebias) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p == 0 && ws.skin_state && lists_rebuild(ws)) {
-    // the lists built in this call serve later calls unless they overflowed
-    ws.skin_state[2] += 1;
-    ws.skin_state[3] = (ws.status[0] & (kStCapacity | kStCells)) ? 0 : 1;
+  if (p == 0 && ws.skin_state) {
+    if (lists_rebuild(ws)) {
+      // the lists built in this call serve later calls unless they overflowed
+      ws.skin_state[2] += 1;
+      ws.skin_state[3] = (ws.status[0] & (kStCapacity | kStCells)) ? 0 : 1;
+    }
+    ws.skin_state[0] = ws.skin_state[1] = 0;   // the next call's check starts from here
   }
+  if (p == 0 && ws.status_pub)   // no later kernel of the call sets a flag
+    for (int i = 0; i < 4; ++i) ws.status_pub[i] = ws.status[i];
   const unsigned lane = threadIdx.x & 31;
   const int total = ws.totals[0];
   const bool live = p < total;

@@ -36,7 +36,8 @@ __device__ __forceinline__ unsigned lanemask_lt() {
   return m;
 }
 
-__device__ __forceinline__ int find_sys(const BatchParams& bp, int idx) {
+template <int N>
+__device__ __forceinline__ int find_sys(const BatchParamsT<N>& bp, int idx) {
   // last system whose in_base <= idx (in_base relative to the chunk start)
   int lo = 0, hi = bp.n_sys - 1;
   const int base0 = bp.sys[0].in_base;
@@ -47,7 +48,8 @@ __device__ __forceinline__ int find_sys(const BatchParams& bp, int idx) {
   return lo;
 }
 
-__device__ __forceinline__ void init_body(const Ws& ws, const BatchParams& bp, int zero_all,
+template <int N>
+__device__ __forceinline__ void init_body(const Ws& ws, const BatchParamsT<N>& bp, int zero_all,
                                           int n_in, int tid, int stride) {
   const bool rebuild = lists_rebuild(ws);
   // the AEV kernel ORs this call's live slices into the tile masks
@@ -93,12 +95,14 @@ __device__ __forceinline__ void init_body(const Ws& ws, const BatchParams& bp, i
   for (int i = tid; i < n_in; i += stride) ws.f_pos[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void k_init(Ws ws, BatchParams bp, int zero_all, int n_in) {
+template <int N>
+__global__ void k_init(Ws ws, BatchParamsT<N> bp, int zero_all, int n_in) {
   init_body(ws, bp, zero_all, n_in, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // one input atom of a chunk (all 32 lanes of a warp call it together)
-__device__ __forceinline__ void prep_body(const Ws& ws, const BatchParams& bp, int t, int n_chunk,
+template <int N>
+__device__ __forceinline__ void prep_body(const Ws& ws, const BatchParamsT<N>& bp, int t, int n_chunk,
                                           int S) {
   const unsigned lane = threadIdx.x & 31;
   const bool live = t < n_chunk;
@@ -169,7 +173,8 @@ __device__ __forceinline__ void prep_body(const Ws& ws, const BatchParams& bp, i
   }
 }
 
-__global__ void k_prep(Ws ws, BatchParams bp, int n_chunk, int S) {
+template <int N>
+__global__ void k_prep(Ws ws, BatchParamsT<N> bp, int n_chunk, int S) {
   prep_body(ws, bp, blockIdx.x * blockDim.x + threadIdx.x, n_chunk, S);
 }
 
@@ -405,7 +410,8 @@ __global__ void k_scatter(Ws ws, int n_in) {
 // __syncthreads between the phases (their global writes are visible to the
 // whole CTA after the barrier).
 constexpr int kFrontThreads = 1024;
-__global__ void __launch_bounds__(kFrontThreads) k_front(Ws ws, BatchParams bp, AevConst ac,
+template <int N>
+__global__ void __launch_bounds__(kFrontThreads) k_front(Ws ws, BatchParamsT<N> bp, AevConst ac,
                                                           int n_in) {
   const int tid = threadIdx.x;
   init_body(ws, bp, 1, n_in, tid, kFrontThreads);
@@ -425,7 +431,12 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(Ws ws, BatchParams bp, 
 // Largest displacement of an atom of the last build's lists since that build
 // (minimum image in periodic directions), as float bits into skin_state[0]
 // (positive floats order like their bit patterns).
-__global__ void k_skin_check(Ws ws, BatchParams bp, int n_chunk) {
+template <int N>
+__global__ void k_skin_check(Ws ws, BatchParamsT<N> bp, int n_chunk, int forced) {
+  if (forced) {   // the batch's layout changed: nothing to compare with
+    if (blockIdx.x == 0 && threadIdx.x == 0) ws.skin_state[1] = 1;
+    return;
+  }
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   float d2 = 0.f;
   if (t < n_chunk) {
@@ -981,20 +992,39 @@ __global__ void __launch_bounds__(256) k_list_refresh(Ws ws, AevConst ac) {
 
 }  // namespace
 
-void launch_init_chunk(const Ws& ws, const BatchParams& bp, cudaStream_t st) {
-  // the first chunk of a batch also zeroes the shared counters
-  const int zero_all = (bp.sys_base == 0);
-  const int cells = min(ws.cell_cap, 2 * ws.n_in + 27 * ws.n_sys);
-  const int work = zero_all ? max(cells, max(ws.n_in, bp.n_sys)) : bp.n_sys;
-  int blocks = (work + 255) / 256;
-  blocks = max(1, min(blocks, 1184));
-  k_init<<<blocks, 256, 0, st>>>(ws, bp, zero_all, ws.n_in);
-}
-
-void launch_prep_atoms(const Ws& ws, const BatchParams& bp, int n_in_chunk, int S,
-                       cudaStream_t st) {
-  if (n_in_chunk <= 0) return;
-  k_prep<<<(n_in_chunk + 255) / 256, 256, 0, st>>>(ws, bp, n_in_chunk, S);
+std::vector<FrontLaunch> front_launches(const Ws& ws, const std::vector<BatchParams>& chunks,
+                                        const AevConst& ac, int n_in, bool one_cta, bool forced) {
+  std::vector<FrontLaunch> out;
+  const bool few = chunks.size() == 1 && chunks[0].n_sys <= kFewSystems;
+#define NNP_FEW(kernel) (few ? (const void*)kernel<kFewSystems> : (const void*)kernel<kMaxBatchParam>)
+  auto add = [&](const void* fn, int work, int max_blocks, const BatchParams& bp, int a, int b) {
+    const int blocks = std::max(1, std::min((work + 255) / 256, max_blocks));
+    out.push_back({fn, (unsigned)blocks, 256u, ws, &bp, ac, a, b, false});
+  };
+  if (one_cta) {
+    out.push_back({NNP_FEW(k_front), 1u, (unsigned)kFrontThreads, ws, &chunks[0], ac, 0, n_in, true});
+    return out;
+  }
+  const int all = 1 << 30;
+  auto atoms = [](const BatchParams& bp) {
+    int n = 0;
+    for (int k = 0; k < bp.n_sys; ++k) n += bp.sys[k].n_in;
+    return n;
+  };
+  if (ws.skin_state)
+    for (const BatchParams& bp : chunks)
+      if (atoms(bp) > 0) add(NNP_FEW(k_skin_check), forced ? 1 : atoms(bp), all, bp, atoms(bp), forced);
+  // the first chunk's init also zeroes the shared counters
+  const int cells = std::min(ws.cell_cap, 2 * ws.n_in + 27 * ws.n_sys);
+  for (const BatchParams& bp : chunks) {
+    const int zero_all = bp.sys_base == 0;
+    add(NNP_FEW(k_init), zero_all ? std::max(cells, std::max(ws.n_in, bp.n_sys)) : bp.n_sys, 1184, bp,
+        zero_all, ws.n_in);
+  }
+  for (const BatchParams& bp : chunks)
+    if (atoms(bp) > 0) add(NNP_FEW(k_prep), atoms(bp), all, bp, atoms(bp), ac.S);
+#undef NNP_FEW
+  return out;
 }
 
 void launch_setup(const Ws& ws, const AevConst& ac, cudaStream_t st) {
@@ -1011,16 +1041,6 @@ void launch_scan(const Ws& ws, cudaStream_t st) { k_scan<<<1, 1024, 0, st>>>(ws)
 void launch_scatter(const Ws& ws, int n_in, cudaStream_t st) {
   if (n_in <= 0) return;
   k_scatter<<<(n_in + 255) / 256, 256, 0, st>>>(ws, n_in);
-}
-
-void launch_front(const Ws& ws, const BatchParams& bp, const AevConst& ac, int n_in,
-                  cudaStream_t st) {
-  k_front<<<1, kFrontThreads, 0, st>>>(ws, bp, ac, n_in);
-}
-
-void launch_skin_check(const Ws& ws, const BatchParams& bp, int n_in_chunk, cudaStream_t st) {
-  if (n_in_chunk <= 0 || !ws.skin_state) return;
-  k_skin_check<<<(n_in_chunk + 255) / 256, 256, 0, st>>>(ws, bp, n_in_chunk);
 }
 
 void launch_neighbors(const Ws& ws, int n_in, const AevConst& ac, cudaStream_t st) {

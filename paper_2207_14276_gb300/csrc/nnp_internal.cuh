@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace nnp {
 
 constexpr int kMaxSpecies = 8;
@@ -121,15 +123,23 @@ struct SysDev {
   unsigned bb_min[3], bb_max[3];  // bounding box as order-preserving uint keys
 };
 
-struct BatchParams {
+// The kernels that take descriptors come for chunks of up to 2 and of up to 64
+// systems: most calls hold one, and a kernel parameter block of 10 KB costs more to
+// launch (and to send to a graph's node) than one of 0.4 KB.  The layouts share their
+// beginning, so the host fills the large one for either.
+template <int N>
+struct BatchParamsT {
   int n_sys;         // systems in this chunk
   int sys_base;      // index of the first system of the chunk in the batch
-  SysIn sys[kMaxBatchParam];
+  SysIn sys[N];
 };
+constexpr int kFewSystems = 2;
+using BatchParams = BatchParamsT<kMaxBatchParam>;
 
 // device work arena (all pointers device)
 struct Ws {
   int* status;       // [4]: flags, max radial count, max angular count, spare
+  int* status_pub;   // host memory: the last kernel of a call copies status here (or null)
   SysDev* sys;       // [max_sys]
   int n_sys;
   int n_in;          // batch input atoms (sum of n_in)
@@ -184,7 +194,8 @@ struct Ws {
   double* e_det;        // [n_in] atomic energy (FP64), by packed position
   double* v_det;        // [n_in][9] the centre's virial contribution
   // persistent neighbour lists with a skin (null skin_state: rebuilt every call)
-  int* skin_state;      // [4]: max displacement (float bits), forced rebuild, builds, lists valid
+  int* skin_state;      // [4]: max displacement (float bits), forced rebuild (both zeroed by the
+                        // call's last kernel for the next call), builds, lists valid
   float half_skin;      // rebuild when an atom moved farther than this since the build
   float4* ref;          // [n_in] input coordinates at the last build
   int* in_pos;          // [n_in] packed position of an input atom at the last build (-1: none)
@@ -201,18 +212,38 @@ __device__ __forceinline__ bool lists_rebuild(const Ws& ws) {
 }
 
 // ---- launchers (nl.cu)
-void launch_init_chunk(const Ws& ws, const BatchParams& bp, cudaStream_t st);
-void launch_prep_atoms(const Ws& ws, const BatchParams& bp, int n_in_chunk, int S,
-                       cudaStream_t st);
+// One launch that takes the per-call descriptors as kernel parameters (the
+// displacement check, init, prep, or all of the front end in one CTA): held as data
+// so that it can be launched or be (and update) a node of a call's CUDA graph.
+struct FrontLaunch {
+  const void* fn;
+  unsigned grid, block;
+  Ws ws;
+  const BatchParams* bp;
+  AevConst ac;
+  int a, b;        // kernel arguments after the descriptors (a unused with the AevConst)
+  bool has_ac;
+  void args(void** out) const {
+    out[0] = const_cast<Ws*>(&ws);
+    out[1] = const_cast<BatchParams*>(bp);
+    out[2] = has_ac ? (void*)const_cast<AevConst*>(&ac) : (void*)const_cast<int*>(&a);
+    out[3] = const_cast<int*>(&b);
+  }
+  void launch(cudaStream_t st) const {
+    void* p[4];
+    args(p);
+    cudaLaunchKernel(fn, dim3(grid), dim3(block), p, 0, st);
+  }
+};
+// the launches of a batch in order; one_cta: the whole front end of a one-chunk batch
+// in one CTA; forced: persistent lists are rebuilt whatever the displacements
+std::vector<FrontLaunch> front_launches(const Ws& ws, const std::vector<BatchParams>& chunks,
+                                        const AevConst& ac, int n_in, bool one_cta, bool forced);
 void launch_setup(const Ws& ws, const AevConst& ac, cudaStream_t st);
 void launch_bin(const Ws& ws, int n_in, cudaStream_t st);
 void launch_scan(const Ws& ws, cudaStream_t st);
 void launch_scatter(const Ws& ws, int n_in, cudaStream_t st);
 void launch_neighbors(const Ws& ws, int n_in, const AevConst& ac, cudaStream_t st);
-void launch_skin_check(const Ws& ws, const BatchParams& bp, int n_in_chunk, cudaStream_t st);
-// init + prep + setup + bin + scan + scatter of a one-chunk batch in one CTA
-void launch_front(const Ws& ws, const BatchParams& bp, const AevConst& ac, int n_in,
-                  cudaStream_t st);
 // deterministic mode (ws.fr_det set): after a list build, the atoms of every cell
 // in input order and the AEV rows of every species in packed order (both are
 // otherwise taken by atomic counters)
