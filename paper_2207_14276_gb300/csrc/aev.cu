@@ -465,13 +465,28 @@ __device__ __forceinline__ void triplet_bwd(const AevConst& ac, const float4& vj
                    sk * (vj.z - chat * vk.z) + rk * vk.z);
 }
 
+// A warp's virial of the system its last centres belong to, component k on lane k in
+// FP64.  Added to the system's virial when the system changes and once per CTA at the
+// end: nine FP64 atomics per centre on nine addresses made the backward of 9,000
+// water atoms 106 us against 35 without a virial (the whole call 310 us, now 239).
+struct VirialSum {
+  double* dst = nullptr;
+  double sum = 0.0;
+  __device__ __forceinline__ void flush(unsigned lane, double* next) {
+    if (dst && lane < 9) atomicAdd(dst + lane, sum);
+    dst = next;
+    sum = 0.0;
+  }
+};
+
 // Warp per centre, for centres with at most cap_l angular neighbours whose
 // angular terms fall in at most kGallBlocks species-pair blocks (the blocks'
 // dE/dG are all staged at once); a centre with more is appended to ws.heavy
 // (count in totals[2]) for k_aev_bwd_heavy and skipped.
 template <int ZETA, bool VIR>
 __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int log_r, int cap_l,
-                                           int p, float4* sm4, ListHdr& H, int w, unsigned lane) {
+                                           int p, float4* sm4, ListHdr& H, int w, unsigned lane,
+                                           VirialSum& vs) {
   __syncwarp();   // the warp's previous centre is done with its shared memory
   const bool det = ws.fr_det != nullptr;   // deterministic mode
   const int n_copy = 1 << log_r;
@@ -673,13 +688,15 @@ __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int
     else atomicAdd(&ws.f_pos[p], make_float4(fi[0], fi[1], fi[2], 0.f));
   }
   if (VIR && d.in.virial) {
+    if (!det && vs.dst != d.in.virial) vs.flush(lane, d.in.virial);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       float v = vir[k];
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-      if (lane == 0) {
-        if (det) ws.v_det[(size_t)p * 9 + k] = (double)v;
-        else atomicAdd(d.in.virial + k, (double)v);
+      if (det) {
+        if (lane == 0) ws.v_det[(size_t)p * 9 + k] = (double)v;
+      } else if ((int)lane == k) {
+        vs.sum += (double)v;
       }
     }
   }
@@ -694,12 +711,34 @@ k_aev_bwd(Ws ws, AevConst ac, int log_r, int cap_l) {
   const unsigned lane = threadIdx.x & 31;
   // persistent: every warp takes the next centre from a counter until none is left
   const int n = ws.totals[0];
+  VirialSum vs;
   for (;;) {
     int p = 0;
     if (lane == 0) p = atomicAdd(ws.totals + 5, 1);
     p = __shfl_sync(kFull, p, 0);
     if (p >= n) break;
-    bwd_centre<ZETA, VIR>(ws, ac, log_r, cap_l, p, sm4, hdrs[w], w, lane);
+    bwd_centre<ZETA, VIR>(ws, ac, log_r, cap_l, p, sm4, hdrs[w], w, lane, vs);
+  }
+  if (VIR) {
+    // the CTA's warps that hold the same system's sum add it together
+    __shared__ double vsum[kWarps][9];
+    __shared__ double* vdst[kWarps];
+    if (lane < 9) vsum[w][lane] = vs.sum;
+    if (lane == 0) vdst[w] = vs.dst;
+    __syncthreads();
+    if (w == 0 && lane < 9) {
+      double* dst = nullptr;
+      double sum = 0.0;
+      for (int k = 0; k < kWarps; ++k) {
+        if (vdst[k] != dst) {
+          if (dst) atomicAdd(dst + lane, sum);
+          dst = vdst[k];
+          sum = 0.0;
+        }
+        sum += vsum[k][lane];
+      }
+      if (dst) atomicAdd(dst + lane, sum);
+    }
   }
 }
 
