@@ -11,9 +11,7 @@
 //   k_scan     exclusive scan of the cell counts
 //   k_scatter  packed (cell-ordered) float4 coordinates and index maps
 //   k_neighbors one CTA per home cell: the atoms of the 27 neighbour cells are
-//              staged in shared memory, sorted by species, and listed per
-//              octant of the home cell (the candidates near that octant's
-//              atoms); one warp per centre scans its octant's list, keeps pairs
+//              staged in shared memory; one warp per centre scans them, keeps pairs
 //              with R <= rc_r, marks R <= rc_a and writes species-sorted lists
 //              (per-centre search from global memory when a neighbourhood does
 //              not fit the stage)
@@ -608,316 +606,250 @@ __device__ void centre_lists_global(const Ws& ws, const AevConst& ac, int p, int
 }
 
 
-// Species-sorted radial (R <= rc_r) and angular (R <= rc_a) lists of centre p
-// from the candidates cand[t] / cand_j[t], t in [sp_start[s], sp_start[s+1])
-// for species s (coordinates already shifted to the centre's periodic image;
-// dimensions flagged in min_img take the minimum image per pair instead).  With
-// idx, position t of the scan is candidate idx[t] (a subset of the candidates in
-// their order, sp_start counting positions of idx).
+constexpr int kNbThreads = 256;   // 8 warps
+constexpr int kNbWarps = kNbThreads / 32;
+constexpr int kCandCap = 1536;    // staged candidates of one home cell (15 bits of a kept entry)
+
+// per warp: counts, then list positions, of each species (radial, angular)
+struct NbCount {
+  int r[kMaxSpecies], a[kMaxSpecies];
+};
+
+// Lists of centre p from the staged candidates (coordinates already shifted to the
+// centre's periodic image, padded to a multiple of 64 with points out of reach; MI:
+// the dimensions flagged in min_img take the minimum image per pair instead; w:
+// species | range << 8, candidate q of range r being packed atom r_beg[r] + q - r_off[r]).
+// One warp: a scan keeps the candidates within the list cutoff (two chunks of 32 per
+// pass, appended in candidate order: candidate number, bit 15 for the angular cutoff),
+// then the kept ones are counted and placed by species, so that a list is
+// species-sorted and inside a species in candidate order.
+template <bool MI>
 __device__ __forceinline__ void centre_lists_staged(const Ws& ws, const AevConst& ac, int p,
-                                                    const float4* cand, const int* cand_j,
-                                                    const int* sp_start, const int* min_img,
-                                                    const SysDev& d,
-                                                    const uint16_t* idx = nullptr) {
-  const unsigned lane = threadIdx.x & 31;
+                                                    const float4* cand, int total, const int* r_beg,
+                                                    const int* r_off, uint16_t* kept, NbCount& nc,
+                                                    const int* min_img, const SysDev& d) {
+  const unsigned lane = threadIdx.x & 31, lt = lanemask_lt();
   const float4 xi = ws.xyzq[p];
   const float rl = ac.rc_r + ac.skin, al = ac.rc_a + ac.skin;   // list cutoffs
   const float rr2 = rl * rl, ra2 = al * al;
-  const bool any_mi = min_img[0] | min_img[1] | min_img[2];
-  uint16_t* hdr = ws.nb_cnt + (size_t)p * 16;
+  int cnt = 0;
+  auto dist2 = [&](int t) {
+    const float4 xj = cand[t];
+    float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+    if (MI) {
+      float n;
+      if (min_img[0]) { n = rintf(dx / d.in.box_hi[0]); dx = fmaf(-n, d.in.box_hi[0], dx); dx = fmaf(-n, d.in.box_lo[0], dx); }
+      if (min_img[1]) { n = rintf(dy / d.in.box_hi[1]); dy = fmaf(-n, d.in.box_hi[1], dy); dy = fmaf(-n, d.in.box_lo[1], dy); }
+      if (min_img[2]) { n = rintf(dz / d.in.box_hi[2]); dz = fmaf(-n, d.in.box_hi[2], dz); dz = fmaf(-n, d.in.box_lo[2], dz); }
+    }
+    return dx * dx + dy * dy + dz * dz;
+  };
+  auto keep = [&](int t, float r2) {
+    const bool k = r2 <= rr2 && r2 > 1e-12f && (!MI || t < total);   // (the centre itself: r2 = 0)
+    const unsigned bal = __ballot_sync(0xffffffffu, k);
+    const int at = cnt + __popc(bal & lt);
+    if (k && at < kStageCap) kept[at] = (uint16_t)(t | (r2 <= ra2 ? 0x8000 : 0));
+    cnt += __popc(bal);
+  };
+  __syncwarp();   // the previous centre's entries are no longer read
+  if (lane < kMaxSpecies) nc.r[lane] = nc.a[lane] = 0;
+  for (int t0 = 0; t0 < total; t0 += 64) {
+    const int ta = t0 + (int)lane, tb = ta + 32;
+    const float a = dist2(ta), b = dist2(tb);
+    keep(ta, a);
+    keep(tb, b);
+  }
+  __syncwarp();
+  const int nst = min(cnt, kStageCap);
+  // a chunk's kept entries: candidate, species | range << 8, the lanes of the same
+  // species and those of them inside the angular cutoff
+  struct Entry {
+    int q, wv;
+    unsigned same, ang;
+    bool valid;
+  };
+  auto entry = [&](int t) {
+    Entry e;
+    e.valid = t < nst;
+    const unsigned k = e.valid ? kept[t] : 0u;
+    e.q = (int)(k & 0x7fffu);
+    e.wv = e.valid ? __float_as_int(cand[e.q].w) : 0xff;
+    e.same = __match_any_sync(0xffffffffu, e.wv & 0xff);
+    e.ang = __ballot_sync(0xffffffffu, (k & 0x8000u) != 0u) & e.same;
+    return e;
+  };
+  for (int t0 = 0; t0 < nst; t0 += 32) {
+    const Entry e = entry(t0 + (int)lane);
+    if (e.valid && !(e.same & lt)) {   // the species' first lane
+      nc.r[e.wv & 0xff] += __popc(e.same);
+      nc.a[e.wv & 0xff] += __popc(e.ang);
+    }
+    __syncwarp();
+  }
+  const int cr = lane < kMaxSpecies ? nc.r[lane] : 0, ca = lane < kMaxSpecies ? nc.a[lane] : 0;
+  int off_r = cr, off_a = ca;   // inclusive sums over the species, then exclusive
+#pragma unroll
+  for (int o = 1; o < kMaxSpecies; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, off_r, o), v = __shfl_up_sync(0xffffffffu, off_a, o);
+    if ((int)lane >= o) { off_r += u; off_a += v; }
+  }
+  const int all_a = __shfl_sync(0xffffffffu, off_a, kMaxSpecies - 1);
+  off_r -= cr;
+  off_a -= ca;
+  if (lane < kMaxSpecies) {
+    // the header: counts clamped so that the lists stay inside their capacity
+    uint16_t* hdr = ws.nb_cnt + (size_t)p * 16;
+    hdr[lane] = (uint16_t)max(0, min(cr, ws.cap_r - off_r));
+    hdr[8 + lane] = (uint16_t)max(0, min(ca, ws.cap_a - off_a));
+    nc.r[lane] = off_r;
+    nc.a[lane] = off_a;
+  }
+  __syncwarp();
   int* out_r = ws.nb_r + (size_t)p * ws.cap_r;
   int* out_a = ws.nb_a + (size_t)p * ws.cap_a;
-  int wr_r = 0, wr_a = 0;
-  // candidate t of the staged list: within the radial / angular list cutoff?
-  auto test = [&](int t, int end, int& j, bool& keep, bool& ang) {
-    keep = ang = false;
-    j = 0;
-    if (t < end) {
-      const int c = idx ? (int)idx[t] : t;
-      const float4 xj = cand[c];
-      j = cand_j[c];
-      float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-      if (any_mi) {
-        float n;
-        if (min_img[0]) { n = rintf(dx / d.in.box_hi[0]); dx = fmaf(-n, d.in.box_hi[0], dx); dx = fmaf(-n, d.in.box_lo[0], dx); }
-        if (min_img[1]) { n = rintf(dy / d.in.box_hi[1]); dy = fmaf(-n, d.in.box_hi[1], dy); dy = fmaf(-n, d.in.box_lo[1], dy); }
-        if (min_img[2]) { n = rintf(dz / d.in.box_hi[2]); dz = fmaf(-n, d.in.box_hi[2], dz); dz = fmaf(-n, d.in.box_lo[2], dz); }
-      }
-      const float r2 = dx * dx + dy * dy + dz * dz;
-      keep = (r2 <= rr2) && (r2 > 1e-12f) && (j != p);
-      ang = keep && (r2 <= ra2);
+  for (int t0 = 0; t0 < nst; t0 += 32) {
+    const Entry e = entry(t0 + (int)lane);
+    const int sp = e.wv & 0xff, r = e.wv >> 8;
+    int base_r = 0, base_a = 0;
+    if (e.valid) {
+      base_r = nc.r[sp];
+      base_a = nc.a[sp];
+      const int j = r_beg[r] + e.q - r_off[r];
+      const int at = base_r + __popc(e.same & lt), aa = base_a + __popc(e.ang & lt);
+      const bool in = NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j, ws.totals[0]);
+      if (at < ws.cap_r && in) out_r[at] = j;
+      if (((e.ang >> lane) & 1u) && aa < ws.cap_a && in) out_a[aa] = j;
     }
-  };
-  for (int s = 0; s < ac.S; ++s) {
-    int cr = 0, ca = 0;
-    const int end = sp_start[s + 1];
-    // two 32-candidate chunks per pass (independent loads and tests), appended
-    // in candidate order
-    for (int t0 = sp_start[s]; t0 < end; t0 += 64) {
-      int j0, j1;
-      bool k0, a0, k1, a1;
-      test(t0 + (int)lane, end, j0, k0, a0);
-      test(t0 + 32 + (int)lane, end, j1, k1, a1);
-      const unsigned br0 = __ballot_sync(0xffffffffu, k0), ba0 = __ballot_sync(0xffffffffu, a0);
-      const unsigned br1 = __ballot_sync(0xffffffffu, k1), ba1 = __ballot_sync(0xffffffffu, a1);
-      const unsigned lt = lanemask_lt();
-      if (k0) {
-        const int at = wr_r + cr + __popc(br0 & lt);
-        if (at < ws.cap_r && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j0, ws.totals[0])) out_r[at] = j0;
-      }
-      if (a0) {
-        const int at = wr_a + ca + __popc(ba0 & lt);
-        if (at < ws.cap_a && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j0, ws.totals[0])) out_a[at] = j0;
-      }
-      cr += __popc(br0);
-      ca += __popc(ba0);
-      if (k1) {
-        const int at = wr_r + cr + __popc(br1 & lt);
-        if (at < ws.cap_r && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j1, ws.totals[0])) out_r[at] = j1;
-      }
-      if (a1) {
-        const int at = wr_a + ca + __popc(ba1 & lt);
-        if (at < ws.cap_a && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j1, ws.totals[0])) out_a[at] = j1;
-      }
-      cr += __popc(br1);
-      ca += __popc(ba1);
+    __syncwarp();   // every lane has read its species' positions
+    if (e.valid && !(e.same & lt)) {
+      nc.r[sp] = base_r + __popc(e.same);
+      nc.a[sp] = base_a + __popc(e.ang);
     }
-    const int keep_r = max(0, min(cr, ws.cap_r - wr_r));
-    const int keep_a = max(0, min(ca, ws.cap_a - wr_a));
-    if (lane == 0) {
-      hdr[s] = (uint16_t)keep_r;
-      hdr[8 + s] = (uint16_t)keep_a;
-    }
-    wr_r += cr;
-    wr_a += ca;
+    __syncwarp();
   }
-  if (lane == 0) {
-    for (int s = ac.S; s < 8; ++s) { hdr[s] = 0; hdr[8 + s] = 0; }
-    if (wr_r > ws.cap_r || wr_a > ws.cap_a || wr_r > kStageCap) {
-      atomicOr(ws.status, kStCapacity);
-      atomicMax(ws.status + 1, wr_r);
-      atomicMax(ws.status + 2, wr_a);
-    }
+  if (lane == 0 && (cnt > ws.cap_r || all_a > ws.cap_a || cnt > kStageCap)) {
+    atomicOr(ws.status, kStCapacity);
+    atomicMax(ws.status + 1, cnt);
+    atomicMax(ws.status + 2, all_a);
   }
 }
 
-constexpr int kNbThreads = 256;   // 8 warps
-constexpr int kCandCap = 2048;    // staged candidates of one home cell
-constexpr int kOctCap = 512;      // candidates of one octant list
-constexpr int kOctMin = 256;      // octant lists only for more candidates than this
-
-// octant of a point of the home cell about the cell's centre mid
-__device__ __forceinline__ int octant_of(const float4& x, const float* mid) {
-  return (x.x >= mid[0] ? 1 : 0) | (x.y >= mid[1] ? 2 : 0) | (x.z >= mid[2] ? 4 : 0);
-}
-
-// One CTA per home cell (grid-stride over the cells of the batch).  The atoms of
-// the 27 neighbour cells are staged once in shared memory, shifted to the home
-// cell's periodic image and stably sorted by species; then one warp per centre
-// of the home cell scans them species by species and appends the accepted
-// neighbours to its lists, which come out species-sorted without a sort pass.
-__global__ void __launch_bounds__(kNbThreads) k_neighbors(Ws ws, AevConst ac) {
+// One CTA per home cell, the next cell from a device counter.  The atoms of the 27
+// neighbour cells are staged once in shared memory in cell order (one warp per
+// neighbour cell), shifted to the home cell's periodic image; then one warp per centre
+// of the home cell scans them.  Few cells (small systems): several CTAs share a cell's
+// centres.  Bound by instruction issue (about 1,170 warp instructions per centre with
+// 405 candidates, 70% issue active on 20k atoms) and, below one wave of cells, by the
+// chain of loads and barriers of a cell.  Sorting every cell's candidates by species
+// before the scan and listing them per octant of the home cell (what this replaced)
+// shortened the scan but cost 1,450 instructions and four more barriers per cell:
+// solvated100k 219 -> 164 us, 20k atoms 52 -> 34, 72k atoms of water 116 -> 94, 6k
+// solvated atoms 36 -> 17, a 24-atom molecule 9.1 -> 4.8; a 9,000-atom water box, whose
+// 512 cells do not fill the grid, 20 -> 24 us.
+__global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac) {
   __shared__ float4 cand[kCandCap];
-  __shared__ int cand_j[kCandCap];
-  __shared__ uint16_t chunk_cnt[kCandCap / 32][kMaxSpecies];
+  __shared__ uint16_t kept[kNbWarps][kStageCap];
+  __shared__ NbCount counts[kNbWarps];
   __shared__ int r_beg[27], r_off[28];
   __shared__ float r_shift[27][3];
-  __shared__ int sp_start[kMaxSpecies + 1];
   __shared__ int min_img[3];
-  // octant lists: the candidates (positions in cand, in order) within the list
-  // cutoff of the bounding box of the home cell's atoms in each octant
-  __shared__ uint16_t oct_idx[8][kOctCap];
-  __shared__ int oct_sp[8][kMaxSpecies + 1];
-  __shared__ int oct_n[8];
-  __shared__ unsigned oct_key[8][6];   // box as order-preserving keys: min x y z, max x y z
-  __shared__ float oct_mid[3];
+  __shared__ int item_sh;
   const int tid = threadIdx.x, w = tid >> 5;
   const unsigned lane = tid & 31;
   if (!lists_rebuild(ws)) return;
   const int n_cells = ws.totals[1];
-  for (int gc = blockIdx.x; gc < n_cells; gc += gridDim.x) {
+  // work items: (cell, part) with `parts` CTAs per cell where the cells would not
+  // fill the grid
+  const int parts = n_cells > 0 ? max(1, min((int)gridDim.x / n_cells, 8)) : 1;
+  const int n_items = n_cells * parts;
+  int item = blockIdx.x;
+  while (item < n_items) {
+    // the next item is fetched while this one is worked on
+    int next = 0;
+    if (tid == 0) next = (int)gridDim.x + atomicAdd(ws.totals + 3, 1);
+    const int gc = item / parts, part = item % parts;
     const int cbeg = ws.cell_start[gc], cend = ws.cell_start[gc + 1];
-    if (cbeg == cend) continue;   // uniform across the CTA
-    const int b = ws.pos_sys[cbeg];
-    const SysDev& d = ws.sys[b];
-    const int per = d.in.periodic;
-    const int nc[3] = {d.nc[0], d.nc[1], d.nc[2]};
-    const int lc = gc - d.cell_base;
-    const int cc[3] = {lc / (nc[1] * nc[2]), (lc / nc[2]) % nc[1], lc % nc[2]};
-    // ---- the 27 (or fewer) neighbour cells: thread t < 27 takes offset (t/9, t/3%3, t%3)
-    if (w == 0) {
-      int cnt = 0, beg = 0;
-      float sh[3] = {0.f, 0.f, 0.f};
-      if (lane < 27) {
-        const int o[3] = {(int)lane / 9, ((int)lane / 3) % 3, (int)lane % 3};
-        bool ok = true;
-        int k[3];
-        for (int c = 0; c < 3; ++c) {
-          if (per && nc[c] < 3) {
-            // every cell of this dimension once, minimum image per pair
-            k[c] = o[c];
-            ok &= o[c] < nc[c];
-          } else {
-            k[c] = cc[c] + o[c] - 1;
-            if (per) {
-              if (k[c] < 0) { k[c] += nc[c]; sh[c] = -d.in.box_hi[c]; }
-              else if (k[c] >= nc[c]) { k[c] -= nc[c]; sh[c] = d.in.box_hi[c]; }
+    const int first = cbeg + part * kNbWarps;   // this CTA's first centre
+    if (first < cend) {   // uniform across the CTA
+      const SysDev& d = ws.sys[ws.pos_sys[cbeg]];
+      const int per = d.in.periodic;
+      if (w == 0) {
+        const int nc[3] = {d.nc[0], d.nc[1], d.nc[2]};
+        const int lc = gc - d.cell_base;
+        const int cc[3] = {lc / (nc[1] * nc[2]), (lc / nc[2]) % nc[1], lc % nc[2]};
+        // the 27 (or fewer) neighbour cells: lane < 27 takes offset (l/9, l/3%3, l%3)
+        int cnt = 0, beg = 0;
+        float sh[3] = {0.f, 0.f, 0.f};
+        if (lane < 27) {
+          const int o[3] = {(int)lane / 9, ((int)lane / 3) % 3, (int)lane % 3};
+          bool ok = true;
+          int k[3];
+          for (int c = 0; c < 3; ++c) {
+            if (per && nc[c] < 3) {
+              // every cell of this dimension once, minimum image per pair
+              k[c] = o[c];
+              ok &= o[c] < nc[c];
             } else {
-              ok &= (k[c] >= 0 && k[c] < nc[c]);
+              k[c] = cc[c] + o[c] - 1;
+              if (per) {
+                if (k[c] < 0) { k[c] += nc[c]; sh[c] = -d.in.box_hi[c]; }
+                else if (k[c] >= nc[c]) { k[c] -= nc[c]; sh[c] = d.in.box_hi[c]; }
+              } else {
+                ok &= (k[c] >= 0 && k[c] < nc[c]);
+              }
             }
           }
-        }
-        if (ok) {
-          const int g = d.cell_base + (k[0] * nc[1] + k[1]) * nc[2] + k[2];
-          beg = ws.cell_start[g];
-          cnt = ws.cell_start[g + 1] - beg;
-        }
-        r_beg[lane] = beg;
-        r_shift[lane][0] = sh[0]; r_shift[lane][1] = sh[1]; r_shift[lane][2] = sh[2];
-      }
-      int incl = cnt;
-      for (int o2 = 1; o2 < 32; o2 <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o2);
-        if ((int)lane >= o2) incl += u;
-      }
-      if (lane < 27) r_off[lane] = incl - cnt;
-      if (lane == 26) r_off[27] = incl;
-      if (lane < 3) min_img[lane] = (per && nc[lane] < 3) ? 1 : 0;
-    }
-    __syncthreads();
-    const int total = r_off[27];
-    if (total > kCandCap) {
-      // too many candidates to stage: per-centre search from global memory,
-      // with the candidate arrays as the warps' staging space
-      int* stj = reinterpret_cast<int*>(cand) + w * kStageCap;
-      uint8_t* stt = reinterpret_cast<uint8_t*>(reinterpret_cast<int*>(cand) + 8 * kStageCap) + w * kStageCap;
-      for (int p = cbeg + w; p < cend; p += kNbThreads / 32) centre_lists_global(ws, ac, p, stj, stt);
-      __syncthreads();
-      continue;
-    }
-    const int n_chunks = (total + 31) >> 5;
-    // ---- stable species sort of the candidates: counts per 32-chunk, offsets, placement
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int ch = w; ch < n_chunks; ch += kNbThreads / 32) {
-        const int q = ch * 32 + (int)lane;
-        const bool valid = q < total;
-        int r = 0;
-        if (valid) {
-          int lo = 0, hi = 26;   // last range with r_off <= q
-          while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (r_off[mid] <= q) lo = mid; else hi = mid - 1;
+          if (ok) {
+            const int g = d.cell_base + (k[0] * nc[1] + k[1]) * nc[2] + k[2];
+            beg = ws.cell_start[g];
+            cnt = ws.cell_start[g + 1] - beg;
           }
-          r = lo;
+          r_beg[lane] = beg;
+          r_shift[lane][0] = sh[0]; r_shift[lane][1] = sh[1]; r_shift[lane][2] = sh[2];
         }
-        const int j = valid ? r_beg[r] + q - r_off[r] : 0;
-        const float4 xj = valid ? ws.xyzq[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const int sp = valid ? __float_as_int(xj.w) : -1;
-        if (pass == 0) {
-          for (int s = 0; s < ac.S; ++s) {
-            const unsigned bal = __ballot_sync(0xffffffffu, sp == s);
-            if (lane == 0) chunk_cnt[ch][s] = (uint16_t)__popc(bal);
-          }
-        } else {
-          const unsigned same = __match_any_sync(0xffffffffu, sp);
-          if (valid) {
-            const int pos = sp_start[sp] + chunk_cnt[ch][sp] + __popc(same & lanemask_lt());
-            cand[pos] = make_float4(xj.x + r_shift[r][0], xj.y + r_shift[r][1], xj.z + r_shift[r][2], xj.w);
-            cand_j[pos] = j;
-          }
+        int incl = cnt;
+        for (int o2 = 1; o2 < 32; o2 <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, incl, o2);
+          if ((int)lane >= o2) incl += u;
         }
+        if (lane < 27) r_off[lane] = incl - cnt;
+        if (lane == 26) r_off[27] = incl;
+        if (lane < 3) min_img[lane] = (per && nc[lane] < 3) ? 1 : 0;
       }
       __syncthreads();
-      if (pass == 0) {
-        if (tid < ac.S) {   // thread s: exclusive offsets of species s over the chunks
-          int run = 0;
-          for (int ch = 0; ch < n_chunks; ++ch) {
-            const int v = chunk_cnt[ch][tid];
-            chunk_cnt[ch][tid] = (uint16_t)run;
-            run += v;
+      const int total = r_off[27];
+      if (total > kCandCap) {
+        // too many candidates to stage: per-centre search from global memory, with
+        // the candidate array as the warps' staging space
+        static_assert(sizeof(cand) >= kNbWarps * kStageCap * 5, "staging space of the global search");
+        int* stj = reinterpret_cast<int*>(cand) + w * kStageCap;
+        uint8_t* stt = reinterpret_cast<uint8_t*>(reinterpret_cast<int*>(cand) + kNbWarps * kStageCap) + w * kStageCap;
+        for (int p = first + w; p < cend; p += kNbWarps * parts) centre_lists_global(ws, ac, p, stj, stt);
+      } else {
+        for (int r = w; r < 27; r += kNbWarps) {
+          const int beg = r_beg[r], off = r_off[r], n = r_off[r + 1] - off;
+          const float sx = r_shift[r][0], sy = r_shift[r][1], sz = r_shift[r][2];
+          for (int t = (int)lane; t < n; t += 32) {
+            const float4 x = ws.xyzq[beg + t];
+            cand[off + t] = make_float4(x.x + sx, x.y + sy, x.z + sz,
+                                        __int_as_float(__float_as_int(x.w) | (r << 8)));
           }
-          sp_start[tid + 1] = run;   // count for now
         }
+        // the last pass's padding: out of every centre's reach
+        for (int q = total + tid; q < ((total + 63) & ~63); q += kNbThreads)
+          cand[q] = make_float4(1e18f, 1e18f, 1e18f, 0.f);
         __syncthreads();
-        if (tid == 0) {
-          sp_start[0] = 0;
-          for (int s = 0; s < ac.S; ++s) sp_start[s + 1] += sp_start[s];
-        }
-        __syncthreads();
-      }
-    }
-    // ---- octant lists (when no dimension takes the minimum image per pair):
-    // warp o keeps, species by species and in candidate order, the candidates
-    // within the list cutoff of the bounding box of the home cell's atoms in
-    // octant o; a centre then scans only its octant's list (the same neighbours
-    // in the same order, a superset of them being tested).  A list longer than
-    // kOctCap is not used; neighbourhoods of at most kOctMin candidates (small
-    // molecules) are scanned whole, which costs less than building the lists.
-    const bool use_oct = !(min_img[0] | min_img[1] | min_img[2]) && total > kOctMin;
-    if (use_oct) {
-      if (tid < 48) oct_key[tid / 6][tid % 6] = (tid % 6) < 3 ? 0xffffffffu : 0u;
-      if (tid < 3) oct_mid[tid] = d.origin[tid] + ((float)cc[tid] + 0.5f) / d.inv_cell[tid];
-      __syncthreads();
-      for (int p = cbeg + tid; p < cend; p += kNbThreads) {
-        const float4 x = ws.xyzq[p];
-        const int o = octant_of(x, oct_mid);
-        atomicMin(&oct_key[o][0], float_key(x.x));
-        atomicMin(&oct_key[o][1], float_key(x.y));
-        atomicMin(&oct_key[o][2], float_key(x.z));
-        atomicMax(&oct_key[o][3], float_key(x.x));
-        atomicMax(&oct_key[o][4], float_key(x.y));
-        atomicMax(&oct_key[o][5], float_key(x.z));
-      }
-      __syncthreads();
-      {
-        const int o = w;
-        int cnt = 0;
-        if (oct_key[o][0] <= oct_key[o][3]) {   // the octant holds atoms
-          const float lo[3] = {key_float(oct_key[o][0]), key_float(oct_key[o][1]), key_float(oct_key[o][2])};
-          const float hi[3] = {key_float(oct_key[o][3]), key_float(oct_key[o][4]), key_float(oct_key[o][5])};
-          // the centres' own test decides; this one only has to keep every
-          // candidate it could accept, so its cutoff has a margin for rounding
-          const float rl = ac.rc_r + ac.skin;
-          const float rl2 = rl * rl * (1.f + 1e-5f) + 1e-6f;
-          for (int s = 0; s < ac.S; ++s) {
-            if (lane == 0) oct_sp[o][s] = cnt;
-            const int end = sp_start[s + 1];
-            for (int t0 = sp_start[s]; t0 < end; t0 += 32) {
-              const int t = t0 + (int)lane;
-              bool in = false;
-              if (t < end) {
-                const float4 c = cand[t];
-                const float ex = fmaxf(fmaxf(lo[0] - c.x, c.x - hi[0]), 0.f);
-                const float ey = fmaxf(fmaxf(lo[1] - c.y, c.y - hi[1]), 0.f);
-                const float ez = fmaxf(fmaxf(lo[2] - c.z, c.z - hi[2]), 0.f);
-                in = ex * ex + ey * ey + ez * ez <= rl2;
-              }
-              const unsigned bal = __ballot_sync(0xffffffffu, in);
-              if (in) {
-                const int at = cnt + __popc(bal & lanemask_lt());
-                if (at < kOctCap) oct_idx[o][at] = (uint16_t)t;
-              }
-              cnt += __popc(bal);
-            }
-          }
-          if (lane == 0) oct_sp[o][ac.S] = cnt;
-        }
-        if (lane == 0) oct_n[o] = cnt;
-      }
-      __syncthreads();
-    }
-    // ---- one warp per centre of the home cell
-    for (int p = cbeg + w; p < cend; p += kNbThreads / 32) {
-      if (use_oct) {
-        const int o = octant_of(ws.xyzq[p], oct_mid);
-        if (oct_n[o] <= kOctCap) {
-          centre_lists_staged(ws, ac, p, cand, cand_j, oct_sp[o], min_img, d, oct_idx[o]);
-          continue;
+        const bool mi = min_img[0] | min_img[1] | min_img[2];
+        for (int p = first + w; p < cend; p += kNbWarps * parts) {
+          if (mi) centre_lists_staged<true>(ws, ac, p, cand, total, r_beg, r_off, kept[w], counts[w], min_img, d);
+          else centre_lists_staged<false>(ws, ac, p, cand, total, r_beg, r_off, kept[w], counts[w], min_img, d);
         }
       }
-      centre_lists_staged(ws, ac, p, cand, cand_j, sp_start, min_img, d);
     }
-    __syncthreads();   // the stage is rebuilt for the next home cell
+    if (tid == 0) item_sh = next;
+    __syncthreads();   // the stage is rebuilt for the next item
+    item = item_sh;
+    __syncthreads();   // ... and item_sh may be overwritten
   }
 }
 
@@ -1048,7 +980,8 @@ void launch_neighbors(const Ws& ws, int n_in, const AevConst& ac, cudaStream_t s
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = std::max(1, std::min(ws.cell_cap, 4 * std::max(sms, 1)));
+  // one wave of CTAs (six per SM by shared memory), each taking cells until none is left
+  const int grid = std::max(1, std::min(ws.cell_cap, 6 * std::max(sms, 1)));
   if (ws.skin_state && ac.skin > 0.f) {
     // persistent lists: the search (when it runs) fills the lists at the cutoffs
     // + skin; every call then derives the lists at the cutoffs from them
