@@ -270,6 +270,17 @@ k_aev_fwd(Ws ws, AevConst ac) {
   const int w = threadIdx.x >> 5;
   const unsigned lane = threadIdx.x & 31;
   const bool sparse = ws.row_mask != nullptr;
+  // grouped rows: the first row of each (species, slice) group
+  __shared__ int group_row0[kMaxSpecies][32];
+  if (ws.row_key && w < ac.S) {
+    const int c = ws.row_hist[w * 32 + lane];
+    int incl = c;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(kFull, incl, o);
+      if ((int)lane >= o) incl += u;
+    }
+    group_row0[w][lane] = ws.seg_start[w] + incl - c;
+  }
   fill_pair_table(pair_su, ac);
   __syncthreads();
   // persistent: every warp takes the next centre from a counter until none is left
@@ -280,8 +291,19 @@ k_aev_fwd(Ws ws, AevConst ac) {
     if (lane == 0) p = atomicAdd(ws.totals + 4, 1);
     p = __shfl_sync(kFull, p, 0);
     if (p >= n) break;
-    if (!NNP_IN_BOUNDS(ws.status, kSiteAevRow, ws.pos_slot[p], ws.row_cap)) continue;
-    const size_t row = (size_t)ws.pos_slot[p] * ac.Dp;
+    int slot;
+    if (ws.row_key) {
+      const uint32_t k = ws.row_key[p];
+      slot = group_row0[__float_as_int(ws.xyzq[p].w)][k & 31] + (int)(k >> 5);
+      if (lane == 0 && NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) {
+        ws.pos_slot[p] = slot;
+        ws.slot_pos[slot] = p;
+      }
+    } else {
+      slot = ws.pos_slot[p];
+    }
+    if (!NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) continue;
+    const size_t row = (size_t)slot * ac.Dp;
     float* G = ws.aev + row;
     uint16_t* Gh = ws.aev_h ? ws.aev_h + row : nullptr;
     uint16_t* Gl = ws.aev_l ? ws.aev_l + row : nullptr;
@@ -289,7 +311,6 @@ k_aev_fwd(Ws ws, AevConst ac) {
     aev_centre<ZETA>(ws, ac, p, sm4 + (size_t)w * aev_fwd_warp_f4(ws.cap_a, ws.cap_r), hdrs[w], lane,
                      pair_su, [&](int f, float v) { put_g(G, Gh, Gl, f, v); }, sparse, &m);
     if (sparse && lane == 0) {
-      const int slot = ws.pos_slot[p];
       ws.row_mask[slot] = m;
       atomicOr(ws.tile_mask + (slot >> 7), m);
     }

@@ -469,6 +469,8 @@ size_t carve(nnp_handle* h, char* base) {
   // slices, the last backward layer computes only those)
   ws.row_mask = c.take<uint32_t>(rows);
   ws.tile_mask = c.take<uint32_t>(rows / kRowTile + 1);
+  ws.row_key = c.take<uint32_t>(n);
+  ws.row_hist = c.take<int>(kMaxSpecies * 32);
   return align_up(c.off, 256);
 }
 
@@ -627,12 +629,23 @@ bool sparse_call(const nnp_handle* h) {
   return h->sparse_rows && !fuses_aev_l1(h) && !(m.net == kNetSimt && mlp_fused_supported(m.md));
 }
 
+// the work space as this call's kernels see it: rows are grouped by their live slices
+// where they are sparse (not in the deterministic mode, whose rows are in packed order)
+Ws call_ws(const nnp_handle* h) {
+  Ws ws = h->ws;
+  if (!sparse_call(h) || h->det) {
+    ws.row_key = nullptr;
+    ws.row_hist = nullptr;
+  }
+  return ws;
+}
+
 // front_done: the whole front end ran in the first part's one CTA; energy_only: no system asks
 // for forces or a virial
 int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool energy_only,
                  cudaStream_t st, int* n_launch) {
   const Model& m = *h->model;
-  Ws& ws = h->ws;
+  const Ws ws = call_ws(h);
   int launches = 0, rc = NNP_OK;
   const AevConst ac = call_const(h);
   if (n_in > 0) {
@@ -834,7 +847,7 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     h->last_vjp = false;
   }
   const bool forced = ws.skin_state && !h->lists_valid;
-  const std::vector<FrontLaunch> front = front_launches(ws, chunks, call_const(h), n_in, front_done, forced);
+  const std::vector<FrontLaunch> front = front_launches(call_ws(h), chunks, call_const(h), n_in, front_done, forced);
   h->pub_valid = ws.status_pub != nullptr && n_in > 0;
   h->pub_stream = st;
   // systems without atoms: the outputs are the empty sums
@@ -1307,6 +1320,8 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
   ws.aev_h = nullptr;
   ws.aev_l = nullptr;
   if (!h->sparse_rows) { ws.row_mask = nullptr; ws.tile_mask = nullptr; }
+  ws.row_key = nullptr;       // rows as the binning assigned them
+  ws.row_hist = nullptr;
   // the deterministic mode covers energy and force calls, not the VJP (whose
   // dual backward adds atomically): the forces here add atomically as well
   ws.fr_det = ws.fa_det = ws.fs_det = nullptr;
@@ -1437,6 +1452,7 @@ int nnp_set_deterministic(nnp_handle* h, int enable) {
 int nnp_set_sparse_rows(nnp_handle* h, int enable) {
   g_err.clear();
   if (!h) return fail(NNP_ERR_ARG, "null handle");
+  if (h->sparse_rows != (enable != 0)) h->lists_valid = false;   // the rows' order belongs to the lists
   h->sparse_rows = enable != 0;
   return NNP_OK;
 }
@@ -1444,6 +1460,7 @@ int nnp_set_sparse_rows(nnp_handle* h, int enable) {
 int nnp_set_fused_aev_l1(nnp_handle* h, int enable) {
   g_err.clear();
   if (!h) return fail(NNP_ERR_ARG, "null handle");
+  if (h->fused_aev_l1 != (enable != 0)) h->lists_valid = false;   // the rows' order belongs to the lists
   h->fused_aev_l1 = enable != 0;
   return NNP_OK;
 }

@@ -87,6 +87,8 @@ __device__ __forceinline__ void init_body(const Ws& ws, const BatchParamsT<N>& b
     ws.species_fill[tid] = 0;
   }
   if (tid < 4) ws.totals[tid] = 0;
+  if (ws.row_hist)
+    for (int i = tid; i < kMaxSpecies * 32; i += stride) ws.row_hist[i] = 0;
   // the batch's cell grids hold at most 2 n + 27 cells per system (k_setup)
   const int cells = min(ws.cell_cap, 2 * n_in + 27 * ws.n_sys);
   for (int i = tid; i < cells; i += stride) ws.cell_count[i] = 0;
@@ -459,12 +461,35 @@ __global__ void k_skin_check(Ws ws, BatchParamsT<N> bp, int n_chunk, int forced)
   if ((threadIdx.x & 31) == 0 && key > 0) atomicMax(ws.skin_state, key);
 }
 
+// The AEV row of packed atom p (species sp) joins the group of its highest live
+// 64-column slice (one warp; cr, ca: lane s's radial and angular neighbours of species
+// s).  The library stores the blocks of common species first, so the highest live slice
+// tells how far a row's nonzero values reach; with the rows of a species in that order
+// a 128-row tile holds rows of like reach, and the layers that work on the union of a
+// tile's slices skip more.  1000 solute atoms in 33,000 waters: 2.25 live slices per
+// tile against 3.92 with the rows in input order, L1 333 -> 270 us and B1 372 -> 205 us;
+// the counter costs the search 6 us.
+__device__ __forceinline__ void group_row(const Ws& ws, const AevConst& ac, int p, int sp, int cr, int ca,
+                                          const uint8_t* pair_su) {
+  const unsigned lane = threadIdx.x & 31;
+  int top = (int)lane < ac.S && cr > 0 ? ac.rcol[lane] >> 6 : 0;
+  for (int q0 = 0; q0 < ac.n_pairs; q0 += 32) {
+    const int q = q0 + (int)lane, su = q < ac.n_pairs ? pair_su[q] : 0;
+    const int cs = __shfl_sync(0xffffffffu, ca, su & 15), cu = __shfl_sync(0xffffffffu, ca, su >> 4);
+    const bool live = (su & 15) == (su >> 4) ? cs >= 2 : (cs > 0 && cu > 0);
+    if (q < ac.n_pairs && live) top = max(top, (ac.acol[q] + 31) >> 6);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (lane == 0)
+    ws.row_key[p] = (uint32_t)top | ((uint32_t)atomicAdd(ws.row_hist + sp * 32 + top, 1) << 5);
+}
+
 // Neighbour lists of centre p by one warp, candidates read from global memory
 // and staged in st_j / st_t (kStageCap each), then species-sorted.  Used for
 // home cells whose 27-cell neighbourhood does not fit the shared-memory stage
 // of k_neighbors.
 __device__ void centre_lists_global(const Ws& ws, const AevConst& ac, int p, int* st_j,
-                                    uint8_t* st_t) {
+                                    uint8_t* st_t, const uint8_t* pair_su) {
   const unsigned lane = threadIdx.x & 31;
   __syncwarp();   // the stage may still be read by the warp's previous centre
   const float4 xi = ws.xyzq[p];
@@ -557,6 +582,7 @@ __device__ void centre_lists_global(const Ws& ws, const AevConst& ac, int p, int
   const int nst = min(cnt, kStageCap);
   // species-sorted radial and angular lists
   int wr_r = 0, wr_a = 0;
+  int my_r = 0, my_a = 0;   // lane s: counts of species s
   uint16_t* hdr = ws.nb_cnt + (size_t)p * 16;
   int* out_r = ws.nb_r + (size_t)p * ws.cap_r;
   int* out_a = ws.nb_a + (size_t)p * ws.cap_a;
@@ -592,9 +618,11 @@ __device__ void centre_lists_global(const Ws& ws, const AevConst& ac, int p, int
       hdr[s] = (uint16_t)keep_r;
       hdr[8 + s] = (uint16_t)keep_a;
     }
+    if ((int)lane == s) { my_r = cr; my_a = ca; }
     wr_r += cr;
     wr_a += ca;
   }
+  if (ws.row_key) group_row(ws, ac, p, __float_as_int(xi.w), my_r, my_a, pair_su);
   if (lane == 0) {
     for (int s = ac.S; s < 8; ++s) { hdr[s] = 0; hdr[8 + s] = 0; }
     if (cnt > ws.cap_r || wr_a > ws.cap_a || cnt > kStageCap) {
@@ -627,7 +655,8 @@ template <bool MI>
 __device__ __forceinline__ void centre_lists_staged(const Ws& ws, const AevConst& ac, int p,
                                                     const float4* cand, int total, const int* r_beg,
                                                     const int* r_off, uint16_t* kept, NbCount& nc,
-                                                    const int* min_img, const SysDev& d) {
+                                                    const int* min_img, const SysDev& d,
+                                                    const uint8_t* pair_su) {
   const unsigned lane = threadIdx.x & 31, lt = lanemask_lt();
   const float4 xi = ws.xyzq[p];
   const float rl = ac.rc_r + ac.skin, al = ac.rc_a + ac.skin;   // list cutoffs
@@ -694,6 +723,7 @@ __device__ __forceinline__ void centre_lists_staged(const Ws& ws, const AevConst
     if ((int)lane >= o) { off_r += u; off_a += v; }
   }
   const int all_a = __shfl_sync(0xffffffffu, off_a, kMaxSpecies - 1);
+  if (ws.row_key) group_row(ws, ac, p, __float_as_int(xi.w), cr, ca, pair_su);
   off_r -= cr;
   off_a -= ca;
   if (lane < kMaxSpecies) {
@@ -754,9 +784,15 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
   __shared__ float r_shift[27][3];
   __shared__ int min_img[3];
   __shared__ int item_sh;
+  __shared__ uint8_t pair_su[kMaxSpecies * (kMaxSpecies + 1) / 2];   // s | u << 4 of species pair q
   const int tid = threadIdx.x, w = tid >> 5;
   const unsigned lane = tid & 31;
   if (!lists_rebuild(ws)) return;
+  if (tid < ac.n_pairs) {   // (read after the first barrier below)
+    int s = 0, rem = tid;
+    while (rem >= ac.S - s) { rem -= ac.S - s; ++s; }
+    pair_su[tid] = (uint8_t)(s | ((s + rem) << 4));
+  }
   const int n_cells = ws.totals[1];
   // work items: (cell, part) with `parts` CTAs per cell where the cells would not
   // fill the grid
@@ -824,7 +860,7 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
         static_assert(sizeof(cand) >= kNbWarps * kStageCap * 5, "staging space of the global search");
         int* stj = reinterpret_cast<int*>(cand) + w * kStageCap;
         uint8_t* stt = reinterpret_cast<uint8_t*>(reinterpret_cast<int*>(cand) + kNbWarps * kStageCap) + w * kStageCap;
-        for (int p = first + w; p < cend; p += kNbWarps * parts) centre_lists_global(ws, ac, p, stj, stt);
+        for (int p = first + w; p < cend; p += kNbWarps * parts) centre_lists_global(ws, ac, p, stj, stt, pair_su);
       } else {
         for (int r = w; r < 27; r += kNbWarps) {
           const int beg = r_beg[r], off = r_off[r], n = r_off[r + 1] - off;
@@ -841,8 +877,8 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
         __syncthreads();
         const bool mi = min_img[0] | min_img[1] | min_img[2];
         for (int p = first + w; p < cend; p += kNbWarps * parts) {
-          if (mi) centre_lists_staged<true>(ws, ac, p, cand, total, r_beg, r_off, kept[w], counts[w], min_img, d);
-          else centre_lists_staged<false>(ws, ac, p, cand, total, r_beg, r_off, kept[w], counts[w], min_img, d);
+          if (mi) centre_lists_staged<true>(ws, ac, p, cand, total, r_beg, r_off, kept[w], counts[w], min_img, d, pair_su);
+          else centre_lists_staged<false>(ws, ac, p, cand, total, r_beg, r_off, kept[w], counts[w], min_img, d, pair_su);
         }
       }
     }

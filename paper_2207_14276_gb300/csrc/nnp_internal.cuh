@@ -181,6 +181,11 @@ struct Ws {
   // over each 128-row tile; null: every row is written in full
   uint32_t* row_mask;   // [row_cap]
   uint32_t* tile_mask;  // [row_cap / 128 + 1]
+  // rows of a species grouped by their highest live slice (null: rows as the binning
+  // assigned them): per packed atom the slice and the atom's number within its
+  // (species, slice) group, and the groups' sizes; written at every list build
+  uint32_t* row_key;    // [n_in] slice | number << 5
+  int* row_hist;        // [kMaxSpecies][32]
   float* dEdG;          // [row_cap][Dp]
   float* atom_e;        // [row_cap] per-row energy (mean over the ensemble, incl. shift)
   float4* f_pos;        // [n_in] forces on packed atoms
