@@ -32,6 +32,7 @@ int mlp_tc_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, i
                    const float* aev, float* dEdG, bool split, void** state);
 void mlp_tc_release(void* state);
 void mlp_tc_use_chain(void* state, bool on);
+int mlp_tc_e_parts(void* state);
 void launch_aev_to_bf16(const Ws& ws, int n_in, const AevConst& ac, void* out, cudaStream_t st);
 void launch_wait_probe(int* status, unsigned limit, cudaStream_t st);
 }  // namespace nnp
@@ -460,7 +461,7 @@ size_t carve(nnp_handle* h, char* base) {
       mb.d3l = c.take<char>(rows * E * m.md.h3 * 2);
     }
   }
-  mb.e_row = c.take<float>((size_t)E * rows);
+  mb.e_row = c.take<float>((tc ? 2 : 1) * (size_t)E * rows);
   mb.aev_h = tc ? c.take<char>(rows * Dp * 2) : nullptr;
   mb.aev_l = split ? c.take<char>(rows * Dp * 2) : nullptr;
   ws.aev_h = static_cast<uint16_t*>(mb.aev_h);
@@ -696,7 +697,8 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool
     if ((rc = launch_check("aev_bwd"))) return rc;
     {
       StageTimer t(h, st, 10);
-      launch_finalize_e(ws, n_in, h->mb.e_row, m.md.E, ws.row_cap, m.ebias, st);
+      launch_finalize_e(ws, n_in, h->mb.e_row, m.md.E, m.net != kNetSimt ? mlp_tc_e_parts(h->tc_state) : 1,
+                        ws.row_cap, m.ebias, st);
       if (ws.e_det) { launch_det_reduce(ws, any_virial ? 1 : 0, st); ++launches; }
     }
     launches += 2;
@@ -1374,7 +1376,7 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
   launch_aev_fwd_vjp(ws, m.ac, h->vb, n_in, st);
   vjp_networks(h, ws, st);
   launch_aev_bwd_dual(ws, m.ac, h->vb, n_in, st);
-  launch_finalize_e(ws, n_in, h->vb.e_row, m.md.E, ws.row_cap, m.ebias, st);
+  launch_finalize_e(ws, n_in, h->vb.e_row, m.md.E, 1, ws.row_cap, m.ebias, st);
   launch_vjp_scatter(ws, h->vb, n_in, st);
   vjp_weight_grads(h, ws, dL_dweights, st);
   h->last_n_in = n_in;
@@ -1789,7 +1791,7 @@ extern "C" int nnp_energy_forces_noalloc(nnp_handle* h, int64_t n_atoms, const f
     if ((rc = stage_ok("mlp"))) return rc;
     launch_aev_bwd(ws, n, m.ac, virial ? 1 : 0, st);
     if ((rc = stage_ok("aev_bwd"))) return rc;
-    launch_finalize_e(ws, n, mb.e_row, m.md.E, ws.row_cap, m.ebias, st);
+    launch_finalize_e(ws, n, mb.e_row, m.md.E, 1, ws.row_cap, m.ebias, st);
   }
   CU_TRY(cudaGetLastError());
   int status[4] = {0, 0, 0, 0};

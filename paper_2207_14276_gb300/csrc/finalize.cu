@@ -7,7 +7,7 @@ namespace nnp {
 
 namespace {
 
-__global__ void k_finalize(Ws ws, const float* e_row, int E, int e_row_net,
+__global__ void k_finalize(Ws ws, const float* e_row, int E, int parts, int e_row_net,
                            const double* ebias) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p == 0 && ws.skin_state) {
@@ -31,7 +31,23 @@ __global__ void k_finalize(Ws ws, const float* e_row, int E, int e_row_net,
     if (!NNP_IN_BOUNDS(ws.status, kSiteFinalize, slot, ws.row_cap)) slot = 0;
     const int s = __float_as_int(ws.xyzq[p].w);
     float acc = 0.f;
-    for (int e = 0; e < E; ++e) acc += e_row[(size_t)e * e_row_net + slot];
+    // a network's energy is the sum of its parts (one plane per part and network);
+    // eight networks' loads in flight at once
+    for (int e0 = 0; e0 < E; e0 += 8) {
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = e0 + i < E ? e_row[(size_t)(e0 + i) * e_row_net + slot] : 0.f;
+      for (int k = 1; k < parts; ++k) {
+        float u[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) u[i] = e0 + i < E ? e_row[(size_t)(k * E + e0 + i) * e_row_net + slot] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] += u[i];
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (e0 + i < E) acc += v[i];
+    }
     Ei = (double)acc / (double)E + ebias[s];
     ws.atom_e[slot] = (float)Ei;
     const SysDev& d = ws.sys[b];
@@ -186,10 +202,10 @@ void launch_det_reduce(const Ws& ws, int want_virial, cudaStream_t st) {
   k_det_reduce<<<(ws.n_sys + 7) / 8, 256, 0, st>>>(ws, want_virial);
 }
 
-void launch_finalize_e(const Ws& ws, int n_in, const float* e_row, int E, int e_row_net,
+void launch_finalize_e(const Ws& ws, int n_in, const float* e_row, int E, int parts, int e_row_net,
                        const double* ebias, cudaStream_t st) {
   if (n_in <= 0) return;
-  k_finalize<<<(n_in + 255) / 256, 256, 0, st>>>(ws, e_row, E, e_row_net, ebias);
+  k_finalize<<<(n_in + 255) / 256, 256, 0, st>>>(ws, e_row, E, parts, e_row_net, ebias);
 }
 
 void launch_gather_rows(const Ws& ws, int n_in, const float* rows, const uint16_t* rows_h,

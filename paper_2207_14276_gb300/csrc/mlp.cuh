@@ -73,7 +73,7 @@ struct MlpBufs {
   void* H2;   // [rows][E*h2]  (reused for delta2)
   void* D2;   // [rows][E*h2]
   void* d3;   // [rows][E*h3]
-  float* e_row;  // [E][rows]
+  float* e_row;  // [parts][E][rows]: 2 parts per row from the layer GEMMs on tensor cores, else 1
   void* aev_h;   // bf16 copy of the AEV (tensor-core path)
   // split path: low bf16 parts of the AEV, H1, H2 and d3 (same layouts as the
   // high parts, which are aev_h, H1, H2 and d3)

@@ -5,13 +5,13 @@
 // output tiles of one layer GEMM
 //   C[m, n] = sum_k A[m, e*K + k] * B_{e,s}[n, k]
 // for the species s of the tile's 128-row segment and the ensemble member e.
-//   warp 8   TMA producer: 64-wide K slices of A and B into a ring of shared
+//   one warp TMA producer: 64-wide K slices of A and B into a ring of shared
 //            memory stages (128-byte swizzle), completion on mbarriers
-//   warp 9   MMA issuer: tcgen05.mma kind::f16 (M = 128, N = n_tile, K = 16)
+//   one warp MMA issuer: tcgen05.mma kind::f16 (M = 128, N = n_tile, K = 16)
 //            into one of two TMEM accumulators; tcgen05.commit frees a stage
 //            and, after the tile's last K slice, hands the accumulator over
-//   warps 0-7 epilogue: warp w reads accumulator rows 32 (w % 4).. and every
-//            other 16-column chunk (w / 4 picks which); bias, CELU, the width-1
+//   the first 8 or 16 warps: epilogue; warp w reads accumulator rows 32 (w % 4)..
+//            and every second (fourth) 16-column chunk; bias, CELU, the width-1
 //            output layer as a dot product, and in the backward the product
 //            with CELU'(z) rebuilt from the stored activation (1 for h > 0,
 //            1 + h/alpha otherwise); each 32-row x 16-column chunk goes through
@@ -47,9 +47,17 @@ using namespace tcu;
 
 constexpr int kBM = 128;
 constexpr int kBK = 64;           // bf16 elements per K slice (one 128-byte swizzle row)
-constexpr int kEpiWarps = 8;
-constexpr int kProdWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
-constexpr int kThreads = (kEpiWarps + 2) * 32;
+// Epilogue warps (multiples of four: warp w reads the accumulator rows 32 (w % 4) ..).
+// Split operands, CELU layers and TMA'd stored activations: 16; an element's bias, CELU,
+// two roundings and staging are a chain of latencies that two epilogue warps per
+// scheduler do not cover (solvated100k with 8: L1 270 us, B2 394; with 16: 233, 363).
+// The others 8: the output-layer and store epilogues gain nothing (L3 193 against 198,
+// B1 205 against 208), the register prefetch of stored activations would spill, and two
+// BF16 CTAs of narrow layers share an SM's registers.
+constexpr int epi_warps(bool split, int epi, bool auxt) {
+  return split && (epi == kEpiCelu || auxt) ? 16 : 8;
+}
+constexpr int tc_threads(bool split, int epi, bool auxt) { return (epi_warps(split, epi, auxt) + 2) * 32; }
 constexpr int kMaxStages = 4;
 // dynamic shared memory limit: the 227 KB per block minus the kernel's static
 // shared memory (barriers) and some headroom
@@ -139,12 +147,19 @@ __device__ __forceinline__ void stage_store(uint8_t* slot, const float (&v)[16],
 // AUXT (kEpiMul on the split path with TcArgs::aux_tma set): the stored
 // activation comes by TMA into shared memory instead of register prefetches
 template <int EPI, bool SPLIT, bool AUXT = false>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(tc_threads(SPLIT, EPI, AUXT), 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
           const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb2,
           const __grid_constant__ CUtensorMap to, const __grid_constant__ CUtensorMap to2,
           const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap tx2,
           TcArgs g) {
+  constexpr int kEpiWarps = epi_warps(SPLIT, EPI, AUXT), kProdWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
+  constexpr int kGroups = kEpiWarps / 4;      // epilogue warps per accumulator row
+  constexpr int kStep = 16 * kGroups;         // columns between two chunks of a warp
+  // biases and output-layer weights: with 8 epilogue warps fetched before the wait for
+  // the accumulator and kept in shared memory; 16 warps cover the latency of loads
+  // beside the accumulator's (and need the space)
+  constexpr bool kEpiSmem = kEpiWarps == 8 && (EPI == kEpiCelu || EPI == kEpiCeluDot);
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
   __shared__ __align__(8) uint64_t tfull_bar[2], tempty_bar[2], done_bar;
@@ -157,13 +172,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
   const int a_bytes = kBM * kBK * 2, b_bytes = g.n_tile * kBK * 2;
   constexpr int kParts = SPLIT ? 2 : 1;
   const int stage_bytes = kParts * (a_bytes + b_bytes);   // multiple of 1024
-  // after the ring: the epilogue warps' staging slots, then (CELU layers) per
-  // epilogue warp the bias and output-layer weights of its columns of a tile
+  // after the ring: the epilogue warps' staging slots, then
   uint8_t* stg = smem + kStages * stage_bytes;
-  float* epi_sh = reinterpret_cast<float*>(stg + kEpiWarps * g.n_slot * kSlotBytes);
+  float* epi_sh = reinterpret_cast<float*>(stg + kEpiWarps * g.n_slot * kSlotBytes);   // (kEpiSmem)
   // (kEpiMul with aux_tma) per epilogue warp: its chunks of the stored activation,
   // 2 KB each (high part at 0, low part at 1 KB, 32 rows x 16 columns)
-  const int aux_chunks = (g.n_tile / 16 + 1) / 2;
+  const int aux_chunks = (g.n_tile / 16 + kGroups - 1) / kGroups;
   uint8_t* aux_sm = stg + kEpiWarps * g.n_slot * kSlotBytes;
   volatile int* abort_flag = &abort_sh;
 
@@ -273,7 +287,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       mbar_drain(&done_bar, 0);
     }
   } else {
-    // ---- epilogue: warp w owns accumulator rows 32 (w % 4).. and every other
+    // ---- epilogue: warp w owns accumulator rows 32 (w % 4).. and every kGroups-th
     // 16-column chunk starting at chunk w / 4
     const int q = warp & 3, half = warp >> 2;
     const float alpha = g.alpha, inv_alpha = 1.f / g.alpha;
@@ -286,7 +300,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
     float* my_epi = epi_sh + warp * 2 * 128;
     int n_st = 0;   // chunks this warp has stored
     int j = 0;
-    constexpr int kMaxChunks = 256 / 32;   // 16-column chunks of one warp per tile
+    constexpr int kMaxChunks = 256 / kStep;   // 16-column chunks of one warp per tile
     for (int t = blockIdx.x; t < T; t += gridDim.x) {
       const Tile tl = tile_of(t, n_tiles_n, row_tiles, g.nets, g.n_tile, g.seg_start, g.S);
       if (!ntile_live(g, tl.m0, tl.n0)) continue;
@@ -308,7 +322,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       constexpr bool aux_tma = SPLIT && kPre && AUXT;
       uint8_t* my_aux = aux_sm + warp * aux_chunks * 2048;
       auto fetch_aux = [&](int ci) {
-        const int c0 = half * 16 + 32 * ci;
+        const int c0 = half * 16 + kStep * ci;
         if (kPre && !aux_tma && row_ok && c0 < g.n_tile && tl.n0 + c0 < g.N) {
           const uint4* src = reinterpret_cast<const uint4*>(arow + c0);
           pre[ci % kPD][0] = src[0];
@@ -331,12 +345,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
         fence_async_smem();
         unsigned bytes = 0;
         for (int ci = 0; ci < aux_chunks; ++ci) {
-          const int c0 = half * 16 + 32 * ci;
+          const int c0 = half * 16 + kStep * ci;
           if (c0 < g.n_tile && tl.n0 + c0 < g.N) bytes += 2048;
         }
         mbar_expect_tx(&aux_bar[warp], bytes);
         for (int ci = 0; ci < aux_chunks; ++ci) {
-          const int c0 = half * 16 + 32 * ci;
+          const int c0 = half * 16 + kStep * ci;
           if (c0 < g.n_tile && tl.n0 + c0 < g.N) {
             const int x = tl.e * g.aux_net + tl.n0 + c0, y = tl.m0 + q * 32;
             tma_load_2d(my_aux + ci * 2048, &tx, &aux_bar[warp], x, y);
@@ -344,13 +358,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
           }
         }
       }
-      // the bias (and output-layer weights) of this warp's columns, also fetched
-      // before the wait: lane l holds entries l + 32 i of the warp's 16-column chunks
+      // lane l holds entries l + 32 i of the warp's 16-column chunks
       float bpre[4] = {0.f, 0.f, 0.f, 0.f}, wpre[4] = {0.f, 0.f, 0.f, 0.f};
-      if (EPI == kEpiCelu || EPI == kEpiCeluDot) {
+      if (kEpiSmem) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int jj = lane + 32 * i, c0 = half * 16 + 32 * (jj >> 4), n = tl.n0 + c0 + (jj & 15);
+          const int jj = lane + 32 * i, c0 = half * 16 + kStep * (jj >> 4), n = tl.n0 + c0 + (jj & 15);
           if (c0 < g.n_tile && n < g.N) {
             bpre[i] = __ldg(g.bias + tl.e * g.bias_e + tl.s * g.bias_s + n);
             if (EPI == kEpiCeluDot) wpre[i] = __ldg(g.w4 + tl.e * g.w4_e + tl.s * g.w4_s + n);
@@ -365,8 +378,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
         mbar_drain(&aux_bar[warp], j & 1);
         break;
       }
-      if (EPI == kEpiCelu || EPI == kEpiCeluDot) {
-        __syncwarp();   // the previous tile's reads of the warp's bias slots are done
+      if (kEpiSmem) {
+        __syncwarp();   // the previous tile's reads of the warp's slots are done
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           my_epi[lane + 32 * i] = bpre[i];
@@ -379,27 +392,30 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       float dot = 0.f;
 #pragma unroll(kPre ? kMaxChunks : 1)
       for (int ci = 0; ci < kMaxChunks; ++ci) {
-        const int c0 = half * 16 + 32 * ci;
+        const int c0 = half * 16 + kStep * ci;
         if (c0 >= g.n_tile) break;
         const int n = tl.n0 + c0;
+        // the chunk's biases (and output-layer weights), the same on every lane
+        float b[16], w4[16];
+        if ((EPI == kEpiCelu || EPI == kEpiCeluDot) && n < g.N) {
+          const float4* bp = reinterpret_cast<const float4*>(
+              kEpiSmem ? my_epi + ci * 16 : g.bias + tl.e * g.bias_e + tl.s * g.bias_s + n);
+          const float4* wp = reinterpret_cast<const float4*>(
+              kEpiSmem ? my_epi + 128 + ci * 16 : g.w4 + tl.e * g.w4_e + tl.s * g.w4_s + n);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 t4 = kEpiSmem ? bp[k] : __ldg(bp + k);
+            b[4 * k] = t4.x; b[4 * k + 1] = t4.y; b[4 * k + 2] = t4.z; b[4 * k + 3] = t4.w;
+            if (EPI == kEpiCeluDot) {
+              const float4 u4 = kEpiSmem ? wp[k] : __ldg(wp + k);
+              w4[4 * k] = u4.x; w4[4 * k + 1] = u4.y; w4[4 * k + 2] = u4.z; w4[4 * k + 3] = u4.w;
+            }
+          }
+        }
         float v[16];
         tmem_ld16(trow + (uint32_t)c0, v);
         if (n >= g.N) continue;
         if (EPI == kEpiCelu || EPI == kEpiCeluDot) {
-          float b[16];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float4 t4 = *reinterpret_cast<const float4*>(&my_epi[ci * 16 + 4 * k]);
-            b[4 * k] = t4.x; b[4 * k + 1] = t4.y; b[4 * k + 2] = t4.z; b[4 * k + 3] = t4.w;
-          }
-          float w4[16];
-          if (EPI == kEpiCeluDot) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float4 t4 = *reinterpret_cast<const float4*>(&my_epi[128 + ci * 16 + 4 * k]);
-              w4[4 * k] = t4.x; w4[4 * k + 1] = t4.y; w4[4 * k + 2] = t4.z; w4[4 * k + 3] = t4.w;
-            }
-          }
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float z = v[i] + b[i];
@@ -472,9 +488,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
         stage_store<kOut>(slot, v, lane, &to, &to2, tl.e * g.out_net + n, tl.m0 + q * 32);
         ++n_st;
       }
-      // the two warps of a row each add their half of the output-layer dot product
-      // (e_row starts at zero; a sum of two terms does not depend on their order)
-      if (EPI == kEpiCeluDot && row_ok) atomicAdd(g.e_row + (size_t)tl.e * g.e_row_net + m, dot);
+      // every warp of a row stores its part of the output-layer dot product (k_finalize
+      // adds the parts in order)
+      if (EPI == kEpiCeluDot && row_ok) g.e_row[(size_t)(half * g.nets + tl.e) * g.e_row_net + m] = dot;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty_bar[ab]);
@@ -690,10 +706,11 @@ int mlp_tc_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, i
     // (the split path holds both parts of A and B per stage; it takes one CTA per
     // SM where two would leave each CTA fewer than two stages)
     const size_t stage_bytes = (size_t)(split ? 2 : 1) * (kBM * kBK * 2 + nt * kBK * 2);
-    // besides the ring: the epilogue warps' staging slots and, for the CELU
-    // layers, their bias and output-layer weight slots
-    const size_t epi_bytes = (l.epi == kEpiCelu || l.epi == kEpiCeluDot) ? kEpiWarps * 2 * 128 * 4
-                             : aux_tma ? (size_t)kEpiWarps * ((nt / 16 + 1) / 2) * 2048 : 0;
+    // besides the ring: the epilogue warps' staging slots and TMA'd activation boxes
+    const int kEpiWarps = epi_warps(split, l.epi, aux_tma), groups = kEpiWarps / 4;
+    const bool epi_smem = kEpiWarps == 8 && (l.epi == kEpiCelu || l.epi == kEpiCeluDot);
+    const size_t epi_bytes = epi_smem ? (size_t)kEpiWarps * 2 * 128 * 4
+                             : aux_tma ? (size_t)kEpiWarps * ((nt / 16 + groups - 1) / groups) * 2048 : 0;
     auto extra = [&](int slots) { return (size_t)kEpiWarps * slots * kSlotBytes + epi_bytes; };
     auto stages_for = [&](int c, int slots) {
       const size_t budget = std::min((size_t)kMaxDynSmem, (size_t)232448 / c - 2048);
@@ -744,6 +761,12 @@ void mlp_tc_use_chain(void* state, bool on) {
   if (state) static_cast<TcState*>(state)->use_chain = on;
 }
 
+// planes of per-row energy parts that the last layer leaves in MlpBufs::e_row
+int mlp_tc_e_parts(void* state) {
+  const TcState* s = static_cast<const TcState*>(state);
+  return s->chain && s->use_chain ? 1 : epi_warps(s->split, kEpiCeluDot, false) / 4;
+}
+
 void launch_wait_probe(int* status, unsigned limit, cudaStream_t st) {
   k_wait_probe<<<1, 32, 0, st>>>(status, limit);
 }
@@ -779,8 +802,6 @@ int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const M
     a.kmask = (i == 0) ? tmask : nullptr;                       // L1: live K slices
     a.nmask = (i == s->plans.size() - 1) ? tmask : nullptr;     // B1: live N tiles
     if (hook) hook->begin(p.stage_id);
-    // the two epilogue warps of a row add their halves of the output dot product
-    if (a.epi == kEpiCeluDot) cudaMemsetAsync(a.e_row, 0, sizeof(float) * (size_t)md.E * a.e_row_net, st);
     // a masked layer skips N tiles by their index within a row tile; with a grid
     // that is a multiple of the N tiles per row tile every CTA would keep one
     // index (and the CTAs of the skipped ones would idle): take a grid coprime
@@ -792,14 +813,14 @@ int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const M
       while (grid.x > 1 && ntn > 1 && gcd((int)grid.x, ntn) != 1) --grid.x;
     }
 #define NNP_TC_LAUNCH(EPI_, SPLIT_) \
-  k_gemm_tc<EPI_, SPLIT_><<<grid, kThreads, p.smem, st>>>(p.ta, p.tb, p.ta2, p.tb2, p.to, p.to2, p.tx, p.tx2, a)
+  k_gemm_tc<EPI_, SPLIT_><<<grid, tc_threads(SPLIT_, EPI_, false), p.smem, st>>>(p.ta, p.tb, p.ta2, p.tb2, p.to, p.to2, p.tx, p.tx2, a)
     if (s->split) {
       switch (a.epi) {
         case kEpiCelu: NNP_TC_LAUNCH(kEpiCelu, true); break;
         case kEpiCeluDot: NNP_TC_LAUNCH(kEpiCeluDot, true); break;
         case kEpiMul:
           if (a.aux_tma)
-            k_gemm_tc<kEpiMul, true, true><<<grid, kThreads, p.smem, st>>>(p.ta, p.tb, p.ta2, p.tb2, p.to,
+            k_gemm_tc<kEpiMul, true, true><<<grid, tc_threads(true, kEpiMul, true), p.smem, st>>>(p.ta, p.tb, p.ta2, p.tb2, p.to,
                                                                             p.to2, p.tx, p.tx2, a);
           else
             NNP_TC_LAUNCH(kEpiMul, true);

@@ -278,7 +278,7 @@ cudaError_t aev_ensure_smem(const Ws& ws);
 size_t aev_fwd_smem(const Ws& ws);
 size_t aev_bwd_smem(const Ws& ws, int n_pairs = kMaxSpecies * (kMaxSpecies + 1) / 2);
 // ---- finalize.cu
-void launch_finalize_e(const Ws& ws, int n_in, const float* e_row, int E, int e_row_net,
+void launch_finalize_e(const Ws& ws, int n_in, const float* e_row, int E, int parts, int e_row_net,
                        const double* ebias, cudaStream_t st);
 void launch_gather_rows(const Ws& ws, int n_in, const float* rows, const uint16_t* rows_h,
                         const uint16_t* rows_l, int ld, int D, const int16_t* col, float* out,
