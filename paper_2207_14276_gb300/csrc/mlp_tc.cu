@@ -101,6 +101,20 @@ __device__ __forceinline__ bool ntile_live(const TcArgs& g, int m0, int n0) {
   return ((m >> a) & span) != 0u;
 }
 
+// The epilogues work on pairs of columns with packed FP32x2 instructions and take the
+// exponential as 2^x with the scale folded in: an element of a split CELU layer costs
+// about 19 instructions (26 with scalar arithmetic and __expf, whose range handling
+// is not needed: results below 2^-126 flush to zero).  solvated100k: L1 234 -> 208 us,
+// L3 198 -> 186, B3 331 -> 313, B2 361 -> 356.
+__device__ __forceinline__ float2 bf2(uint32_t w) {   // two BF16 values as FP32
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+__device__ __forceinline__ float exp2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // One 32-row x 16-column chunk of an epilogue warp's output, through shared
 // memory: every lane writes its row's 16 values into the warp's staging slot,
 // then lane 0 stores the box with TMA (full-line writes, where direct stores of
@@ -121,8 +135,8 @@ __device__ __forceinline__ void stage_store(uint8_t* slot, const float (&v)[16],
       const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
       wh[i] = *reinterpret_cast<const uint32_t*>(&h);
       if (OUT == 1) {
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
+        const float2 r = __ffma2_rn(bf2(wh[i]), make_float2(-1.f, -1.f), make_float2(v[2 * i], v[2 * i + 1]));
+        const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
         wl[i] = *reinterpret_cast<const uint32_t*>(&l);
       }
     }
@@ -291,6 +305,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
     // 16-column chunk starting at chunk w / 4
     const int q = warp & 3, half = warp >> 2;
     const float alpha = g.alpha, inv_alpha = 1.f / g.alpha;
+    const float ez_scale = 1.4426950408889634f / g.alpha;   // exp(z / alpha) = 2^(z ez_scale)
     constexpr int kOut = EPI == kEpiStore ? 2 : SPLIT ? 1 : 0;
     // BF16 forward layers store straight from registers (measured faster there:
     // 32 bytes per row and chunk; the split and backward layers gain from the
@@ -389,7 +404,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       }
       tc_fence_after();
       const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * g.tmem_cols);
-      float dot = 0.f;
+      float2 dot2 = make_float2(0.f, 0.f);   // sums over even and odd columns
 #pragma unroll(kPre ? kMaxChunks : 1)
       for (int ci = 0; ci < kMaxChunks; ++ci) {
         const int c0 = half * 16 + kStep * ci;
@@ -417,55 +432,54 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
         if (n >= g.N) continue;
         if (EPI == kEpiCelu || EPI == kEpiCeluDot) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float z = v[i] + b[i];
-            const float ez = __expf(z * inv_alpha);
-            const float h = z > 0.f ? z : alpha * (ez - 1.f);
+          for (int i = 0; i < 8; ++i) {
+            const float2 z = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]), make_float2(b[2 * i], b[2 * i + 1]));
+            const float2 t = __fmul2_rn(z, make_float2(ez_scale, ez_scale));
+            const float2 ez = make_float2(exp2_ftz(t.x), exp2_ftz(t.y));   // exp(z / alpha)
+            const float2 n2 = __ffma2_rn(ez, make_float2(alpha, alpha), make_float2(-alpha, -alpha));
+            const float2 h = make_float2(z.x > 0.f ? z.x : n2.x, z.y > 0.f ? z.y : n2.y);
             if (EPI == kEpiCeluDot) {
-              dot = fmaf(h, w4[i], dot);
-              v[i] = w4[i] * (z > 0.f ? 1.f : ez);   // delta3 = w4 * CELU'(z)
+              const float2 w2 = make_float2(w4[2 * i], w4[2 * i + 1]);
+              dot2 = __ffma2_rn(h, w2, dot2);
+              // delta3 = w4 * CELU'(z)
+              const float2 d = __fmul2_rn(w2, make_float2(z.x > 0.f ? 1.f : ez.x, z.y > 0.f ? 1.f : ez.y));
+              v[2 * i] = d.x;
+              v[2 * i + 1] = d.y;
             } else {
-              v[i] = h;   // CELU' is rebuilt from h where it is needed
+              v[2 * i] = h.x;   // CELU' is rebuilt from h where it is needed
+              v[2 * i + 1] = h.y;
             }
           }
         } else if (EPI == kEpiMul) {
           // aux holds the layer's stored activation h = CELU(z): CELU'(z) = 1 for h > 0,
           // 1 + h / alpha otherwise (exp(z/alpha) = 1 + h/alpha on that branch)
-          float a[16];
+          uint32_t w[8], wl[8];   // high and low parts, two columns each
           if (aux_tma) {   // the boxes in shared memory: this lane's row, 32 bytes per part
             const uint4* sh = reinterpret_cast<const uint4*>(my_aux + ci * 2048 + lane * 32);
             const uint4* sl = reinterpret_cast<const uint4*>(my_aux + ci * 2048 + 1024 + lane * 32);
-            const uint4 q4[4] = {sh[0], sh[1], sl[0], sl[1]};
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(q4);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-              const float2 fl = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[8 + i]));
-              a[2 * i] = f.x + fl.x;
-              a[2 * i + 1] = f.y + fl.y;
-            }
+            *reinterpret_cast<uint4*>(w) = sh[0];
+            *reinterpret_cast<uint4*>(w + 4) = sh[1];
+            *reinterpret_cast<uint4*>(wl) = sl[0];
+            *reinterpret_cast<uint4*>(wl + 4) = sl[1];
           } else {
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(pre[kPre ? ci % kPD : 0]);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-              a[2 * i] = f.x;
-              a[2 * i + 1] = f.y;
-            }
-          }
-          if (SPLIT && !aux_tma) {
-            // the stored activation h = hi + lo (about 16 significant bits)
-            const uint32_t* wl = reinterpret_cast<const uint32_t*>(prel[kPre && SPLIT ? ci % kPD : 0]);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&wl[i]));
-              a[2 * i] += f.x;
-              a[2 * i + 1] += f.y;
+            *reinterpret_cast<uint4*>(w) = pre[kPre ? ci % kPD : 0][0];
+            *reinterpret_cast<uint4*>(w + 4) = pre[kPre ? ci % kPD : 0][1];
+            if (SPLIT) {
+              *reinterpret_cast<uint4*>(wl) = prel[kPre && SPLIT ? ci % kPD : 0][0];
+              *reinterpret_cast<uint4*>(wl + 4) = prel[kPre && SPLIT ? ci % kPD : 0][1];
             }
           }
           if (ci + kPD < kMaxChunks) fetch_aux(ci + kPD);   // the slot just read is free
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] *= (a[i] > 0.f) ? 1.f : fmaf(a[i], inv_alpha, 1.f);
+          for (int i = 0; i < 8; ++i) {
+            float2 a = bf2(w[i]);
+            if (SPLIT) a = __fadd2_rn(a, bf2(wl[i]));   // h = hi + lo (about 16 significant bits)
+            const float2 d = __ffma2_rn(a, make_float2(inv_alpha, inv_alpha), make_float2(1.f, 1.f));
+            const float2 r = __fmul2_rn(make_float2(v[2 * i], v[2 * i + 1]),
+                                        make_float2(a.x > 0.f ? 1.f : d.x, a.y > 0.f ? 1.f : d.y));
+            v[2 * i] = r.x;
+            v[2 * i + 1] = r.y;
+          }
         }
         if (kDirect && !row_ok) continue;   // bounds-checked build only
         if (!row_ok) {   // bounds-checked build only: a row past the segments stays zero
@@ -490,7 +504,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       }
       // every warp of a row stores its part of the output-layer dot product (k_finalize
       // adds the parts in order)
-      if (EPI == kEpiCeluDot && row_ok) g.e_row[(size_t)(half * g.nets + tl.e) * g.e_row_net + m] = dot;
+      if (EPI == kEpiCeluDot && row_ok) g.e_row[(size_t)(half * g.nets + tl.e) * g.e_row_net + m] = dot2.x + dot2.y;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty_bar[ab]);
