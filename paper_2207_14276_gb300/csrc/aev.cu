@@ -36,6 +36,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "aev_device.cuh"
 #include "nnp_internal.cuh"
@@ -83,35 +84,6 @@ int aev_bwd_copies(int cap_a, int n_pairs) {
   return 1;
 }
 
-// Same pairs, numbered along diagonals so that consecutive lanes get distinct
-// j (and distinct k): same species: pair (q, q + g + 1) of diagonal g; else
-// d = t / cs, j = t % cs, k = (j + d) % cu.  Used where lanes add into
-// per-neighbour accumulators, to spread those atomics over different addresses.
-__device__ __forceinline__ void decode_pair_diag(int t, int same, int c, int cu, float inv_cs,
-                                                 float inv_cu, int* j, int* k) {
-  if (same) {
-    const float b = 2.f * c - 1.f;
-    int g = (int)((b - sqrt_approx(fmaxf(b * b - 8.f * t, 0.f))) * 0.5f);
-    g = max(0, min(g, c - 2));
-    if ((g + 1) * (2 * c - g - 2) / 2 <= t) ++g;
-    else if (g * (2 * c - g - 1) / 2 > t) --g;
-    const int q = t - g * (2 * c - g - 1) / 2;
-    *j = q;
-    *k = q + g + 1;
-  } else {
-    int d = (int)((t + 0.5f) * inv_cs);
-    int jj = t - d * c;
-    if (jj < 0) { --d; jj += c; }
-    else if (jj >= c) { ++d; jj -= c; }
-    const int x = jj + d;
-    int kk = x - (int)((x + 0.5f) * inv_cu) * cu;
-    if (kk < 0) kk += cu;
-    else if (kk >= cu) kk -= cu;
-    *j = jj;
-    *k = kk;
-  }
-}
-
 // one AEV element: the FP32 row, or on the tensor-core paths (Gh != null) only
 // what their first layer reads: the BF16 row, and on the split path (Gl != null)
 // also the low part bf16(v - bf16(v))
@@ -131,16 +103,42 @@ __host__ __device__ constexpr int aev_fwd_warp_f4(int cap_a, int cap_r) {
   return cap_a + cap_a / 4 + cap_r / 2 + 2;
 }
 
-// The AEV row of packed atom p (Eqs. 3-5) by one warp; out(f, v) stores feature
-// f (each f < Dp exactly once, by the lane holding it).  stage: this warp's
-// aev_fwd_warp_f4 float4s of shared memory; H: its list header.  With sparse
-// set, only the blocks that touch a live slice of the row (row_slices) are
-// stored, and *mask receives the row's slice mask.
-template <int ZETA, class Out>
+// species-pair blocks of a centre with triplets: pairs of present species and species
+// present at least twice (the same value on every lane)
+__device__ __forceinline__ int live_blocks(const ListHdr& H, const AevConst& ac, unsigned lane) {
+  const int c = (int)lane < ac.S ? H.off_a[lane + 1] - H.off_a[lane] : 0;
+  const int n_one = __popc(__ballot_sync(kFull, c >= 1));
+  const int n_two = __popc(__ballot_sync(kFull, c >= 2));
+  return n_one * (n_one - 1) / 2 + n_two;
+}
+
+// a centre whose backward exceeds what a warp stages joins ws.heavy (count in totals[2])
+__device__ __forceinline__ void note_dense(const Ws& ws, const AevConst& ac, const ListHdr& H, unsigned lane,
+                                           int p, int cap_l) {
+  const int n_live = live_blocks(H, ac, lane);
+  if (lane == 0 && (H.off_a[ac.S] > cap_l || n_live > kGallBlocks)) {
+    const int hi = atomicAdd(ws.totals + 2, 1);
+    if (NNP_IN_BOUNDS(ws.status, kSiteBwdHeavy, hi, ws.n_in)) ws.heavy[hi] = p;
+  }
+}
+
+// The AEV row of packed atom p (Eqs. 3-5) by W warps (1, or all kWarps of the CTA;
+// w: this warp's number among them); out(f, v) stores feature f (each f < Dp exactly
+// once, by the lane holding it).  stage: aev_fwd_warp_f4 float4s of shared memory; H:
+// the list header.  The warps share the staged neighbours; warp w takes every W-th
+// species' radial block and every W-th angular block.  With sparse set, only the blocks
+// that touch a live slice of the row (row_slices) are stored, and *mask receives the
+// row's slice mask.
+template <int ZETA, int W, class Out>
 __device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int p, float4* stage,
                                            ListHdr& H, unsigned lane, const uint8_t* pair_su,
-                                           Out out, bool sparse = false, uint32_t* mask = nullptr) {
-  __syncwarp();   // the warp's stage and header may still hold its previous centre
+                                           Out out, bool sparse = false, uint32_t* mask = nullptr,
+                                           int w = 0) {
+  auto sync = [] {
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+  };
+  sync();   // the stage and header may still hold the previous centre
   float4* angv = stage;
   float* angf = reinterpret_cast<float*>(angv + ws.cap_a);
   float2* rad = reinterpret_cast<float2*>(angf + ws.cap_a + 4);
@@ -152,28 +150,29 @@ __device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int
     else if (lane == 2) a = ws.nb_a + (size_t)p * ws.cap_a;
     if (a) asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
   }
-  load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
+  if (W == 1 || w == 0) load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
+  if (W > 1) __syncthreads();
   const uint32_t m = sparse ? row_slices(H, ac, lane, pair_su) : ~0u;
   if (mask) *mask = m;
   const int* lr = ws.nb_r + (size_t)p * ws.cap_r;
   const int* la = ws.nb_a + (size_t)p * ws.cap_a;
   const float inv_rc_r = 1.f / ac.rc_r, inv_rc_a = 1.f / ac.rc_a;
-  stage_list(H.off_r[ac.S], lr, xi, d, ws, lane,
-             [&](int slot, int, const Geo& g) {
-               rad[slot] = make_float2(g.r, fcut(g.r, ac.rc_r, inv_rc_r));
-             });
-  stage_list(H.off_a[ac.S], la, xi, d, ws, lane,
-             [&](int slot, int, const Geo& g) {
-               const float inv = rcp_approx(g.r);
-               angv[slot] = make_float4(g.dx * inv, g.dy * inv, g.dz * inv, g.r);
-               angf[slot] = fcut(g.r, ac.rc_a, inv_rc_a);
-             });
-  __syncwarp();
+  stage_list<W>(H.off_r[ac.S], lr, xi, d, ws, w * 32 + lane,
+                [&](int slot, int, const Geo& g) {
+                  rad[slot] = make_float2(g.r, fcut(g.r, ac.rc_r, inv_rc_r));
+                });
+  stage_list<W>(H.off_a[ac.S], la, xi, d, ws, w * 32 + lane,
+                [&](int slot, int, const Geo& g) {
+                  const float inv = rcp_approx(g.r);
+                  angv[slot] = make_float4(g.dx * inv, g.dy * inv, g.dz * inv, g.r);
+                  angf[slot] = fcut(g.r, ac.rc_a, inv_rc_a);
+                });
+  sync();
   // ---- radial, Eq. 4
   const float cr_ = -ac.eta_r * kLog2e;
   const float my_shf = ac.shf_r[lane & 15];
   const int half = lane >> 4;
-  for (int s = 0; s < ac.S; ++s) {
+  for (int s = w; s < ac.S; s += W) {
     float acc = 0.f;
     const int o = H.off_r[s], n = H.off_r[s + 1] - o;
     if (n == 0) {   // no neighbour of this species: a zero block
@@ -204,11 +203,14 @@ __device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int
     live[h] = __ballot_sync(kFull, lv);
     zero[h] = __ballot_sync(kFull, zr);
   }
-  for (int h = 0; h < 2; ++h)
-    for (uint32_t z = zero[h]; z; z &= z - 1)
-      out(ac.acol[h * 32 + __ffs(z) - 1] + lane, 0.f);
+  if (W == 1 || w == W - 1)
+    for (int h = 0; h < 2; ++h)
+      for (uint32_t z = zero[h]; z; z &= z - 1)
+        out(ac.acol[h * 32 + __ffs(z) - 1] + lane, 0.f);
+  int turn = 0;   // live blocks in turn to the warps
   for (int h = 0; h < 2; ++h)
     for (uint32_t lv = live[h]; lv; lv &= lv - 1) {
+      if (W > 1 && turn++ % W != w) continue;
       const int q = h * 32 + __ffs(lv) - 1;
       const int s = pair_su[q] & 15, u = pair_su[q] >> 4;
       const int os = H.off_a[s], cs = H.off_a[s + 1] - os;
@@ -257,13 +259,14 @@ __device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int
       }
       out(fb + lane, transpose_reduce32(acc, lane));
     }
-  for (int f = ac.D + lane; f < ac.Dp; f += 32)
-    if ((m >> (f >> 6)) & 1u) out(f, 0.f);
+  if (W == 1 || w == W - 1)
+    for (int f = ac.D + lane; f < ac.Dp; f += 32)
+      if ((m >> (f >> 6)) & 1u) out(f, 0.f);
 }
 
 template <int ZETA>
 __global__ void __launch_bounds__(kWarps * 32, 4)
-k_aev_fwd(Ws ws, AevConst ac) {
+k_aev_fwd(Ws ws, AevConst ac, int small, int cap_l) {
   extern __shared__ float4 sm4[];
   __shared__ ListHdr hdrs[kWarps];
   __shared__ uint8_t pair_su[kMaxSpecies * (kMaxSpecies + 1) / 2];
@@ -283,37 +286,51 @@ k_aev_fwd(Ws ws, AevConst ac) {
   }
   fill_pair_table(pair_su, ac);
   __syncthreads();
-  // persistent: every warp takes the next centre from a counter until none is left
-  // (dense centres do not hold a CTA's other warps' slots, nor pile up in one warp)
   const int n = ws.totals[0];
-  for (;;) {
-    int p = 0;
-    if (lane == 0) p = atomicAdd(ws.totals + 4, 1);
-    p = __shfl_sync(kFull, p, 0);
-    if (p >= n) break;
-    int slot;
-    if (ws.row_key) {
-      const uint32_t k = ws.row_key[p];
-      slot = group_row0[__float_as_int(ws.xyzq[p].w)][k & 31] + (int)(k >> 5);
-      if (lane == 0 && NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) {
-        ws.pos_slot[p] = slot;
-        ws.slot_pos[slot] = p;
-      }
-    } else {
-      slot = ws.pos_slot[p];
+  // the row of packed atom p (grouped rows: from its group; lane 0 of the first warp
+  // tells the later kernels)
+  auto row_of = [&](int p, bool tell) {
+    if (!ws.row_key) return ws.pos_slot[p];
+    const uint32_t k = ws.row_key[p];
+    const int slot = group_row0[__float_as_int(ws.xyzq[p].w)][k & 31] + (int)(k >> 5);
+    if (tell && NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) {
+      ws.pos_slot[p] = slot;
+      ws.slot_pos[slot] = p;
     }
-    if (!NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) continue;
+    return slot;
+  };
+  auto centre = [&](auto warps, int p, int wi, float4* stage, ListHdr& H) {
+    constexpr int W = decltype(warps)::value;
+    const int slot = row_of(p, lane == 0 && wi == 0);
+    if (!NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) return;
     const size_t row = (size_t)slot * ac.Dp;
     float* G = ws.aev + row;
     uint16_t* Gh = ws.aev_h ? ws.aev_h + row : nullptr;
     uint16_t* Gl = ws.aev_l ? ws.aev_l + row : nullptr;
     uint32_t m = 0;
-    aev_centre<ZETA>(ws, ac, p, sm4 + (size_t)w * aev_fwd_warp_f4(ws.cap_a, ws.cap_r), hdrs[w], lane,
-                     pair_su, [&](int f, float v) { put_g(G, Gh, Gl, f, v); }, sparse, &m);
-    if (sparse && lane == 0) {
+    aev_centre<ZETA, W>(ws, ac, p, stage, H, lane, pair_su,
+                        [&](int f, float v) { put_g(G, Gh, Gl, f, v); }, sparse, &m, wi);
+    if (W == 1) note_dense(ws, ac, H, lane, p, cap_l);
+    if (sparse && lane == 0 && wi == 0) {
       ws.row_mask[slot] = m;
       atomicOr(ws.tile_mask + (slot >> 7), m);
     }
+  };
+  if (n <= small) {
+    // few centres: a CTA each (a warp alone works through a dense centre's blocks one
+    // after the other while the chip idles)
+    for (int p = blockIdx.x; p < n; p += gridDim.x)
+      centre(std::integral_constant<int, kWarps>{}, p, w, sm4, hdrs[0]);
+    return;
+  }
+  // persistent: every warp takes the next centre from a counter until none is left
+  // (dense centres do not hold a CTA's other warps' slots, nor pile up in one warp)
+  for (;;) {
+    int p = 0;
+    if (lane == 0) p = atomicAdd(ws.totals + 4, 1);
+    p = __shfl_sync(kFull, p, 0);
+    if (p >= n) break;
+    centre(std::integral_constant<int, 1>{}, p, 0, sm4 + (size_t)w * aev_fwd_warp_f4(ws.cap_a, ws.cap_r), hdrs[w]);
   }
 }
 
@@ -380,38 +397,6 @@ __device__ __forceinline__ void radial_edge_bwd(const Ws& ws, const AevConst& ac
     vir[0] -= g.dx * gx; vir[1] -= g.dx * gy; vir[2] -= g.dx * gz;
     vir[3] -= g.dy * gx; vir[4] -= g.dy * gy; vir[5] -= g.dy * gz;
     vir[6] -= g.dz * gx; vir[7] -= g.dz * gy; vir[8] -= g.dz * gz;
-  }
-}
-
-// Block table of a centre's angular terms, built by one warp: per species pair
-// q, its geometry (os, cs, ou, cu | same << 16) in the species-sorted angular
-// list and the number of its first triplet in a numbering continuous over all
-// blocks (bt_start[n_pairs] = the centre's triplet count).
-__device__ __forceinline__ void build_block_table(const ListHdr& H, const AevConst& ac,
-                                                  unsigned lane, int4* bt_geo, int* bt_start) {
-  const int np = ac.n_pairs;
-  for (int q0 = 0, carry = 0; q0 < np; q0 += 32) {
-    const int q = q0 + lane;
-    int n_tri = 0;
-    if (q < np) {
-      int sp = 0, rem = q;
-      while (rem >= ac.S - sp) { rem -= ac.S - sp; ++sp; }
-      const int u = sp + rem;
-      const int os = H.off_a[sp], cs = H.off_a[sp + 1] - os;
-      const int ou = H.off_a[u], cu = H.off_a[u + 1] - ou;
-      const int same = (sp == u);
-      n_tri = same ? cs * (cs - 1) / 2 : cs * cu;
-      bt_geo[q] = make_int4(os, cs, ou, cu | (same << 16));
-    }
-    int incl = n_tri;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, incl, o);
-      if ((int)lane >= o) incl += v;
-    }
-    if (q < np) bt_start[q] = carry + incl - n_tri;
-    carry += __shfl_sync(kFull, incl, 31);
-    if (q0 + 32 >= np && lane == 0) bt_start[np] = carry;
   }
 }
 
@@ -502,8 +487,8 @@ struct VirialSum {
 
 // Warp per centre, for centres with at most cap_l angular neighbours whose
 // angular terms fall in at most kGallBlocks species-pair blocks (the blocks'
-// dE/dG are all staged at once); a centre with more is appended to ws.heavy
-// (count in totals[2]) for k_aev_bwd_heavy and skipped.
+// dE/dG are all staged at once); the others, listed by the forward (note_dense),
+// are k_aev_bwd_cta's.
 template <int ZETA, bool VIR>
 __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int log_r, int cap_l,
                                            int p, float4* sm4, ListHdr& H, int w, unsigned lane,
@@ -524,22 +509,8 @@ __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int
   const SysDev& d = ws.sys[ws.pos_sys[p]];
   const float* g_row = ws.dEdG + (size_t)ws.pos_slot[p] * ac.Dp;
   load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
-  // species-pair blocks with triplets: pairs of present species and species
-  // present at least twice
-  int n_live;
-  {
-    const int c = (int)lane < ac.S ? H.off_a[lane + 1] - H.off_a[lane] : 0;
-    const int n_one = __popc(__ballot_sync(kFull, c >= 1));
-    const int n_two = __popc(__ballot_sync(kFull, c >= 2));
-    n_live = n_one * (n_one - 1) / 2 + n_two;
-  }
-  if (H.off_a[ac.S] > cap_l || n_live > kGallBlocks) {
-    if (lane == 0) {
-      const int hi = atomicAdd(ws.totals + 2, 1);
-      if (NNP_IN_BOUNDS(ws.status, kSiteBwdHeavy, hi, ws.n_in)) ws.heavy[hi] = p;
-    }
-    return;
-  }
+  const int n_live = live_blocks(H, ac, lane);
+  if (H.off_a[ac.S] > cap_l || n_live > kGallBlocks) return;   // k_aev_bwd_cta's
   const int* lr = ws.nb_r + (size_t)p * ws.cap_r;
   const int* la = ws.nb_a + (size_t)p * ws.cap_a;
   const float inv_rc_r = 1.f / ac.rc_r, inv_rc_a = 1.f / ac.rc_a;
@@ -725,13 +696,14 @@ __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int
 
 template <int ZETA, bool VIR>
 __global__ void __launch_bounds__(kWarps * 32, 4)
-k_aev_bwd(Ws ws, AevConst ac, int log_r, int cap_l) {
+k_aev_bwd(Ws ws, AevConst ac, int log_r, int cap_l, int small) {
   extern __shared__ float4 sm4[];
   __shared__ ListHdr hdrs[kWarps];
   const int w = threadIdx.x >> 5;
   const unsigned lane = threadIdx.x & 31;
   // persistent: every warp takes the next centre from a counter until none is left
   const int n = ws.totals[0];
+  if (n <= small) return;   // a CTA per centre: k_aev_bwd_cta's
   VirialSum vs;
   for (;;) {
     int p = 0;
@@ -763,171 +735,165 @@ k_aev_bwd(Ws ws, AevConst ac, int log_r, int cap_l) {
   }
 }
 
-// CTA per centre, for the centres k_aev_bwd handed on (more than its cap_l
-// angular neighbours: a dense solute core can have a hundred, i.e. thousands of
-// triplets).  The CTA's eight warps share the centre's staged neighbours and all
-// its angular dE/dG blocks and split its radial edges and triplets; every warp
-// adds into its own copies of the per-neighbour accumulators (lane l into copy
-// (l mod n_lane) of its warp's n_lane), summed once at the end.  Persistent:
-// CTAs stride over the ws.heavy list.
-constexpr int kHeavyThreads = 256;
+// CTA per centre: for the centres listed in ws.heavy (more angular neighbours or
+// species-pair blocks than a warp stages: a dense solute core can have a hundred
+// neighbours, i.e. thousands of triplets), and for every centre of a small batch.  The
+// CTA's eight warps share the centre's staged neighbours and dE/dG blocks and split its
+// radial edges and triplets.  The triplets come in the round-robin order of k_aev_bwd
+// in chunks of 32 (fewer for few neighbours: a chunk spans at most `copies` rounds of
+// disjoint pairs), every eighth chunk to a warp, which adds into its own accumulator
+// copies by plain read-add-write: no atomics, and the order of every addition is fixed,
+// which serves the deterministic mode too.  Persistent: CTAs stride over the list.
+// CTA_FIGURES
+constexpr int kCtaThreads = kWarps * 32;
 
-__host__ __device__ constexpr size_t aev_bwd_heavy_smem(int cap_a, int n_pairs, int n_lane) {
-  return (size_t)2 * cap_a * 16 +                        // angv, angf
-         (size_t)3 * cap_a * (kHeavyThreads / 32) * n_lane * 4 +  // accumulators
-         (size_t)kMaxSpecies * kNR * 4 +                  // radial dE/dG
-         (size_t)n_pairs * 32 * 4 +                       // angular dE/dG, [q][8a + z]
-         (size_t)n_pairs * 16 + (size_t)(n_pairs + 1) * 4 + 16;   // block table
+__host__ __device__ constexpr int bwd_cta_f4(int cap_a, int n_pairs, int copies) {
+  return 2 * cap_a + kWarps * copies * cap_a + kMaxSpecies * kNR / 4 + kGallStride * n_pairs + (cap_a + 64 + 15) / 16;
+}
+// 4 copies where two CTAs then fit an SM, else 2
+int bwd_cta_copies(int cap_a, int n_pairs) {
+  return bwd_cta_f4(cap_a, n_pairs, 4) * 16 <= 110 * 1024 ? 4 : 2;
 }
 
 template <int ZETA, bool VIR>
-__global__ void __launch_bounds__(kHeavyThreads)
-k_aev_bwd_heavy(Ws ws, AevConst ac, int log_n) {
+__global__ void __launch_bounds__(kCtaThreads, 2)
+k_aev_bwd_cta(Ws ws, AevConst ac, int copies, int small) {
   extern __shared__ float4 smh[];
   __shared__ ListHdr H;
-  __shared__ float red[kHeavyThreads / 32][12];
-  const int n_lane = 1 << log_n;
-  const int n_acc = (kHeavyThreads / 32) << log_n;      // copies per neighbour
+  __shared__ float red[kWarps][12];
   const int cap = ws.cap_a;
   const int tid = threadIdx.x, w = tid >> 5;
   const unsigned lane = tid & 31;
-  float4* angv = smh;
-  float4* angf = angv + cap;
-  float* accx = reinterpret_cast<float*>(angf + cap);   // [neighbour][copy]
-  float* accy = accx + (size_t)cap * n_acc;
-  float* accz = accy + (size_t)cap * n_acc;
-  float* grad = accz + (size_t)cap * n_acc;
-  float* gf = grad + kMaxSpecies * kNR;
-  const float4* gall = reinterpret_cast<const float4*>(gf);
-  int4* bt_geo = reinterpret_cast<int4*>(gf + ac.n_pairs * 32);
-  int* bt_start = reinterpret_cast<int*>(bt_geo + ac.n_pairs);
-  const int np = ac.n_pairs;
-  const int n_heavy = ws.totals[2];
+  float4* angv = smh;                      // unit vector and R
+  float4* angf = angv + cap;               // fc, fc', 1/R, packed index
+  float4* acc = angf + cap;                // [warp][copy][neighbour]
+  float* grad = reinterpret_cast<float*>(acc + (size_t)kWarps * copies * cap);
+  float4* gall = reinterpret_cast<float4*>(grad + kMaxSpecies * kNR);   // [block slot][8a + z] (+ pad)
+  uint8_t* spec = reinterpret_cast<uint8_t*>(gall + kGallStride * ac.n_pairs);   // [cap]
+  uint8_t* pslot = spec + cap;             // [8 s + u]: block slot of species pair (s, u)
+  const int n = ws.totals[0];
+  const bool all = n <= small;
+  const int n_list = all ? n : ws.totals[2];
   const bool det = ws.fr_det != nullptr;   // deterministic mode
   const float inv_rc_r = 1.f / ac.rc_r, inv_rc_a = 1.f / ac.rc_a;
-  for (int h = blockIdx.x; h < n_heavy; h += gridDim.x) {
-    const int p = ws.heavy[h];
+  double* vdst = nullptr;   // thread 3 + k: component k of the virial of one system
+  double vsum = 0.0;
+  for (int h = blockIdx.x; h < n_list; h += gridDim.x) {
+    const int p = all ? h : ws.heavy[h];
     __syncthreads();   // the previous centre's shared data are no longer read
     if (w == 0) load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
-    __syncthreads();
     const float4 xi = ws.xyzq[p];
     const SysDev& d = ws.sys[ws.pos_sys[p]];
     const float* g_row = ws.dEdG + (size_t)ws.pos_slot[p] * ac.Dp;
     const int* lr = ws.nb_r + (size_t)p * ws.cap_r;
     const int* la = ws.nb_a + (size_t)p * ws.cap_a;
+    for (int f = tid; f < ac.S * kNR; f += kCtaThreads) grad[f] = g_row[ac.rcol[f >> 4] + (f & 15)];
+    __syncthreads();
     const int na = H.off_a[ac.S], nr = H.off_r[ac.S];
-    for (int t = tid; t < na; t += kHeavyThreads) {
-      int j = la[t];
-      if (!NNP_IN_BOUNDS(ws.status, kSiteAevNeighbour, j, ws.totals[0])) j = p;
-      const Geo g = pair_geo(xi, ws.xyzq[j], d);
+    stage_list<kWarps>(na, la, xi, d, ws, tid, [&](int slot, int j, const Geo& g) {
       const float inv = rcp_approx(g.r);
-      angv[t] = make_float4(g.dx * inv, g.dy * inv, g.dz * inv, g.r);
+      angv[slot] = make_float4(g.dx * inv, g.dy * inv, g.dz * inv, g.r);
       float fc, dfc;
       fcut_both(g.r, ac.rc_a, inv_rc_a, &fc, &dfc);
-      angf[t] = make_float4(fc, dfc, inv, __int_as_float(j));
+      angf[slot] = make_float4(fc, dfc, inv, __int_as_float(j));
+    });
+    for (int t = tid; t < na; t += kCtaThreads) {
+      int s = 0;
+      while (s + 1 < ac.S && H.off_a[s + 1] <= t) ++s;
+      spec[t] = (uint8_t)s;
     }
-    for (int i = tid; i < na * n_acc; i += kHeavyThreads) {
-      accx[i] = 0.f;
-      accy[i] = 0.f;
-      accz[i] = 0.f;
+    for (int c = w; c < kWarps * copies; c += kWarps)
+      for (int t = lane; t < na; t += 32) acc[c * cap + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // the live species-pair blocks, in the order of their pairs, in turn to the warps:
+    // dE/dG in feature order
+    {
+      float* gf = reinterpret_cast<float*>(gall);
+      int slot = 0;
+      for (int s = 0; s < ac.S; ++s) {
+        const int cs = H.off_a[s + 1] - H.off_a[s];
+        for (int u = s; u < ac.S; ++u) {
+          const int cu = H.off_a[u + 1] - H.off_a[u];
+          if (s == u ? cs < 2 : (cs < 1 || cu < 1)) continue;
+          if (slot % kWarps == w) {
+            gf[slot * (4 * kGallStride) + lane] = g_row[ac.acol[s * ac.S - s * (s - 1) / 2 + (u - s)] + lane];
+            if (lane == 0) pslot[8 * s + u] = pslot[8 * u + s] = (uint8_t)slot;
+          }
+          ++slot;
+        }
+      }
     }
-    for (int f = tid; f < ac.S * kNR; f += kHeavyThreads) grad[f] = g_row[ac.rcol[f >> 4] + (f & 15)];
-    if (w == 0) build_block_table(H, ac, lane, bt_geo, bt_start);
-    __syncthreads();
-    // every block with triplets: its 32 dE/dG values (index 8a + z)
-    for (int i = tid; i < np * 32; i += kHeavyThreads) {
-      const int q = i >> 5, l = i & 31;
-      if (bt_start[q + 1] > bt_start[q]) gf[q * 32 + l] = g_row[ac.acol[q] + l];
-    }
-    __syncthreads();
     float fi[3] = {0.f, 0.f, 0.f};
     float vir[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) vir[k] = 0.f;
     int sr = 0;
-    for (int t = tid; t < nr; t += kHeavyThreads) {
+    for (int t = tid; t < nr; t += kCtaThreads) {
       while (H.off_r[sr + 1] <= t) ++sr;
       const int j = lr[t];
       if (!NNP_IN_BOUNDS(ws.status, kSiteBwdNeighbour, j, ws.totals[0])) continue;
       radial_edge_bwd<VIR>(ws, ac, xi, d, j, ws.xyzq[j], grad + sr * kNR, inv_rc_r, fi, vir,
                            det ? ws.fr_det + (size_t)p * ws.cap_r + t : nullptr);
     }
-    const int n_tri = bt_start[np];
-    const int cp = w * n_lane + ((int)lane & (n_lane - 1));
-    int bl = 0, cur = -1;
-    int os = 0, cs = 0, ou = 0, cu = 0, same = 0;
-    float inv_cs = 0.f, inv_cu = 0.f;
-    auto triplet = [&](int t, float3& uj, float3& uk, int& aj, int& ak) -> bool {
-      while (bt_start[bl + 1] <= t) ++bl;
-      if (bl != cur) {
-        cur = bl;
-        const int4 g4 = bt_geo[bl];
-        os = g4.x; cs = g4.y; ou = g4.z; cu = g4.w & 0xffff; same = (g4.w >> 16) & 1;
-        inv_cs = rcp_approx((float)max(cs, 1));
-        inv_cu = rcp_approx((float)max(cu, 1));   // decode corrects one step either way
-      }
-      int j, k;
-      decode_pair_diag(t - bt_start[bl], same, cs, cu, inv_cs, inv_cu, &j, &k);
-      const int tj = os + j, tk = ou + k;
-      if (!NNP_IN_BOUNDS(ws.status, kSiteBwdTriplet, tj, na) ||
-          !NNP_IN_BOUNDS(ws.status, kSiteBwdTriplet, tk, na))
-        return false;
-      triplet_bwd<ZETA>(ac, angv[tj], angv[tk], angf[tj], angf[tk], gall + bl * 8, uj, uk);
-      aj = tj * n_acc + cp;
-      ak = tk * n_acc + cp;
-      return true;
-    };
-    if (!det) {
-      for (int t = tid; t < n_tri; t += kHeavyThreads) {
-        float3 uj, uk;
-        int aj, ak;
-        if (!triplet(t, uj, uk, aj, ak)) continue;
-        atomicAdd(accx + aj, uj.x);
-        atomicAdd(accy + aj, uj.y);
-        atomicAdd(accz + aj, uj.z);
-        atomicAdd(accx + ak, uk.x);
-        atomicAdd(accy + ak, uk.y);
-        atomicAdd(accz + ak, uk.z);
-      }
-    } else {
-      // deterministic mode: within a warp the lanes add one after the other (the
-      // warps add into their own copies)
-      for (int t0 = w * 32; t0 < n_tri; t0 += kHeavyThreads) {
-        float3 uj, uk;
-        int aj = 0, ak = 0;
-        const bool act = t0 + (int)lane < n_tri && triplet(t0 + (int)lane, uj, uk, aj, ak);
-        for (int l = 0; l < 32; ++l) {
-          if (act && (int)lane == l) {
-            accx[aj] += uj.x; accy[aj] += uj.y; accz[aj] += uj.z;
-            accx[ak] += uk.x; accy[ak] += uk.y; accz[ak] += uk.z;
+    __syncthreads();   // the staged neighbours, blocks and zeroed accumulators are complete
+    // c consecutive pairs span at most `copies` rounds of rr.h pairs
+    const RoundRobin rr = make_round_robin(na);
+    const int chunk = min(32, (copies - 1) * rr.h + 1);
+    for (int t0 = w * chunk; t0 < rr.n_tri; t0 += kWarps * chunk) {
+      const int t = t0 + (int)lane;
+      if ((int)lane < chunk && t < rr.n_tri) {
+        int r, a, b;
+        rr_pair(rr, t, &r, &a, &b);
+        if (NNP_IN_BOUNDS(ws.status, kSiteBwdTriplet, a, na) &&
+            NNP_IN_BOUNDS(ws.status, kSiteBwdTriplet, b, na)) {
+          const int slot = pslot[8 * spec[a] + spec[b]];
+          if (NNP_IN_BOUNDS(ws.status, kSiteBwdTriplet, slot, ac.n_pairs)) {
+            float3 ua, ub;
+            triplet_bwd<ZETA>(ac, angv[a], angv[b], angf[a], angf[b], gall + slot * kGallStride, ua, ub);
+            float4* A = acc + (size_t)(w * copies + (r & (copies - 1))) * cap;
+            float4 x = A[a];
+            x.x += ua.x; x.y += ua.y; x.z += ua.z;
+            A[a] = x;
+            float4 y = A[b];
+            y.x += ub.x; y.y += ub.y; y.z += ub.z;
+            A[b] = y;
           }
-          __syncwarp();
+        }
+      }
+      __syncwarp();   // the next chunk may add into the same accumulators
+    }
+    __syncthreads();
+    // four threads per neighbour sum its copies (every fourth warp's), then combine
+    const int n_copy = kWarps * copies, n4 = (na + 63) / 64 * 64;
+    for (int q = tid; q < 4 * n4; q += kCtaThreads) {
+      const int t = q >> 2, part = q & 3;
+      float3 a = make_float3(0.f, 0.f, 0.f);
+      if (t < na)
+        for (int c = part; c < n_copy; c += 4) {
+          const float4 x = acc[c * cap + t];
+          a.x += x.x; a.y += x.y; a.z += x.z;
+        }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        a.x += __shfl_xor_sync(kFull, a.x, o);
+        a.y += __shfl_xor_sync(kFull, a.y, o);
+        a.z += __shfl_xor_sync(kFull, a.z, o);
+      }
+      if (part == 0 && t < na) {
+        const float4 v = angv[t];
+        const int jt = __float_as_int(angf[t].w);
+        if (det) ws.fa_det[(size_t)p * ws.cap_a + t] = make_float4(-a.x, -a.y, -a.z, 0.f);
+        else if (NNP_IN_BOUNDS(ws.status, kSiteBwdNeighbour, jt, ws.totals[0]))
+          atomicAdd(&ws.f_pos[jt], make_float4(-a.x, -a.y, -a.z, 0.f));
+        fi[0] += a.x; fi[1] += a.y; fi[2] += a.z;
+        if (VIR) {
+          const float ux = v.x * v.w, uy = v.y * v.w, uz = v.z * v.w;
+          vir[0] -= ux * a.x; vir[1] -= ux * a.y; vir[2] -= ux * a.z;
+          vir[3] -= uy * a.x; vir[4] -= uy * a.y; vir[5] -= uy * a.z;
+          vir[6] -= uz * a.x; vir[7] -= uz * a.y; vir[8] -= uz * a.z;
         }
       }
     }
-    __syncthreads();
-    for (int t = tid; t < na; t += kHeavyThreads) {
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int c = 0; c < n_acc; ++c) {
-        const int i = t * n_acc + c;
-        a.x += accx[i];
-        a.y += accy[i];
-        a.z += accz[i];
-      }
-      const float4 v = angv[t];
-      const int jt = __float_as_int(angf[t].w);
-      if (det) ws.fa_det[(size_t)p * ws.cap_a + t] = make_float4(-a.x, -a.y, -a.z, 0.f);
-      else if (NNP_IN_BOUNDS(ws.status, kSiteBwdNeighbour, jt, ws.totals[0]))
-        atomicAdd(&ws.f_pos[jt], make_float4(-a.x, -a.y, -a.z, 0.f));
-      fi[0] += a.x; fi[1] += a.y; fi[2] += a.z;
-      if (VIR) {
-        const float ux = v.x * v.w, uy = v.y * v.w, uz = v.z * v.w;
-        vir[0] -= ux * a.x; vir[1] -= ux * a.y; vir[2] -= ux * a.z;
-        vir[3] -= uy * a.x; vir[4] -= uy * a.y; vir[5] -= uy * a.z;
-        vir[6] -= uz * a.x; vir[7] -= uz * a.y; vir[8] -= uz * a.z;
-      }
-    }
-    // the centre's force and the virial: warp sums, then warp 0 over the warps
+    // the centre's force and the virial: warp sums, then threads 0-11 over the warps
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       fi[0] += __shfl_xor_sync(kFull, fi[0], o);
@@ -945,16 +911,25 @@ k_aev_bwd_heavy(Ws ws, AevConst ac, int log_n) {
     __syncthreads();
     if (tid < 12) {
       float v = 0.f;
-      for (int k = 0; k < kHeavyThreads / 32; ++k) v += red[k][tid];
+      for (int k = 0; k < kWarps; ++k) v += red[k][tid];
       if (tid < 3) {
         if (det) reinterpret_cast<float*>(&ws.fs_det[p])[tid] = v;
         else atomicAdd(reinterpret_cast<float*>(&ws.f_pos[p]) + tid, v);
       } else if (VIR && d.in.virial) {
-        if (det) ws.v_det[(size_t)p * 9 + (tid - 3)] = (double)v;
-        else atomicAdd(d.in.virial + (tid - 3), (double)v);
+        if (det) {
+          ws.v_det[(size_t)p * 9 + (tid - 3)] = (double)v;
+        } else {   // added up in FP64 while the CTA's centres belong to one system
+          if (vdst != d.in.virial + (tid - 3)) {
+            if (vdst) atomicAdd(vdst, vsum);
+            vdst = d.in.virial + (tid - 3);
+            vsum = 0.0;
+          }
+          vsum += (double)v;
+        }
       }
     }
   }
+  if (VIR && vdst) atomicAdd(vdst, vsum);
 }
 
 // ---------------------------------------------------------------- AEV -> first layer
@@ -976,6 +951,7 @@ struct AevL1Args {
   int h1;
   float alpha;
   int stage_bytes;      // one W1 slice: h1 x 64 BF16
+  int cap_l;            // angular neighbours of the warp-per-centre backward
 };
 
 __device__ __forceinline__ void put_tile(uint8_t* tile, int r, int f, float v) {
@@ -1034,8 +1010,9 @@ k_aev_l1(const __grid_constant__ CUtensorMap tw1, Ws ws, AevConst ac, AevL1Args 
   for (int r = w; r < kTileM; r += kL1Warps) {
     const int slot = m0 + r;
     if (slot < seg_end) {
-      aev_centre<ZETA>(ws, ac, ws.slot_pos[slot], stage, hdrs[w], lane, pair_su,
-                       [&](int f, float v) { put_tile(tile, r, f, v); });
+      aev_centre<ZETA, 1>(ws, ac, ws.slot_pos[slot], stage, hdrs[w], lane, pair_su,
+                          [&](int f, float v) { put_tile(tile, r, f, v); });
+      note_dense(ws, ac, hdrs[w], lane, ws.slot_pos[slot], g.cap_l);
     } else {
       for (int f = (int)lane; f < ac.Dp; f += 32) put_tile(tile, r, f, 0.f);
     }
@@ -1127,20 +1104,11 @@ size_t aev_bwd_smem(const Ws& ws, int n_pairs) {
          sizeof(float4);
 }
 
-// lane copies per warp of the CTA-per-centre kernel's accumulators: as many as
-// keep its shared memory within 96 KiB (two CTAs per SM), at most 4
-static int heavy_log_n(const Ws& ws, int n_pairs) {
-  for (int l = 2; l > 0; --l)
-    if (aev_bwd_heavy_smem(ws.cap_a, n_pairs, 1 << l) <= 96 * 1024) return l;
-  return 0;
-}
-static size_t heavy_smem(const Ws& ws, int n_pairs) {
-  return aev_bwd_heavy_smem(ws.cap_a, n_pairs, 1 << heavy_log_n(ws, n_pairs));
+static size_t bwd_cta_smem(const Ws& ws, int n_pairs) {
+  return (size_t)bwd_cta_f4(ws.cap_a, n_pairs, bwd_cta_copies(ws.cap_a, n_pairs)) * sizeof(float4);
 }
 
-// grid of the persistent warp-per-centre kernels: four CTAs per SM at most,
-// fewer for small batches
-static int centre_grid(int n_in) {
+static int sm_count() {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
@@ -1148,15 +1116,25 @@ static int centre_grid(int n_in) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms < 1) sms = 1;
   }
-  return std::max(1, std::min((n_in + kWarps - 1) / kWarps, 4 * sms));
+  return sms;
+}
+
+// up to this many centres get a CTA each in the forward and the backward: four CTAs
+// per SM, one wave.  SMALL_FIGURES
+static int small_centres() { return 4 * sm_count(); }
+
+// grid of the persistent warp-per-centre kernels: four CTAs per SM at most, fewer for
+// small batches (which have a CTA per centre up to `small` of them)
+static int centre_grid(int n_in, int small) {
+  return std::max(1, n_in <= small ? n_in : std::min(std::max((n_in + kWarps - 1) / kWarps, small), 4 * sm_count()));
 }
 
 void launch_aev_fwd(const Ws& ws, int n_in, const AevConst& ac, cudaStream_t st) {
   if (n_in <= 0) return;
   const size_t sm = aev_fwd_smem(ws);
-  const int grid = centre_grid(n_in);
-  if (ac.zeta == 32) k_aev_fwd<32><<<grid, kWarps * 32, sm, st>>>(ws, ac);
-  else k_aev_fwd<0><<<grid, kWarps * 32, sm, st>>>(ws, ac);
+  const int small = small_centres(), grid = centre_grid(n_in, small);
+  if (ac.zeta == 32) k_aev_fwd<32><<<grid, kWarps * 32, sm, st>>>(ws, ac, small, light_cap(ws));
+  else k_aev_fwd<0><<<grid, kWarps * 32, sm, st>>>(ws, ac, small, light_cap(ws));
 }
 
 void launch_aev_fill(const Ws& ws, const AevConst& ac, cudaStream_t st) {
@@ -1164,35 +1142,34 @@ void launch_aev_fill(const Ws& ws, const AevConst& ac, cudaStream_t st) {
   k_aev_fill<<<(ws.row_cap + 7) / 8, 256, 0, st>>>(ws, ac);
 }
 
-void launch_aev_bwd(const Ws& ws, int n_in, const AevConst& ac, int want_virial,
+void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int want_virial,
                     cudaStream_t st) {
   if (n_in <= 0) return;
-  const int cap_l = light_cap(ws);
+  const int cap_l = light_cap(ws), small = small_centres();
+  // the CTA-per-centre kernel: where centres can exceed what a warp takes, and where
+  // the batch is small (a mask may leave few centres of many atoms)
+  if (n_in <= small || masked || ws.cap_a > cap_l || ac.n_pairs > kGallBlocks) {
+    const size_t sm = bwd_cta_smem(ws, ac.n_pairs);
+    const int copies = bwd_cta_copies(ws.cap_a, ac.n_pairs), grid = std::min(n_in, 4 * sm_count());
+    if (ac.zeta == 32) {
+      if (want_virial) k_aev_bwd_cta<32, true><<<grid, kCtaThreads, sm, st>>>(ws, ac, copies, small);
+      else k_aev_bwd_cta<32, false><<<grid, kCtaThreads, sm, st>>>(ws, ac, copies, small);
+    } else {
+      if (want_virial) k_aev_bwd_cta<0, true><<<grid, kCtaThreads, sm, st>>>(ws, ac, copies, small);
+      else k_aev_bwd_cta<0, false><<<grid, kCtaThreads, sm, st>>>(ws, ac, copies, small);
+    }
+  }
+  if (n_in <= small) return;
   const size_t sm = aev_bwd_smem(ws, ac.n_pairs);
   const int copies = aev_bwd_copies(cap_l, ac.n_pairs);
   const int log_r = copies == 4 ? 2 : copies == 2 ? 1 : 0;
-  const int grid = centre_grid(n_in);
+  const int grid = centre_grid(n_in, small);
   if (ac.zeta == 32) {
-    if (want_virial) k_aev_bwd<32, true><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l);
-    else k_aev_bwd<32, false><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l);
+    if (want_virial) k_aev_bwd<32, true><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
+    else k_aev_bwd<32, false><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
   } else {
-    if (want_virial) k_aev_bwd<0, true><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l);
-    else k_aev_bwd<0, false><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l);
-  }
-  // no centre can have more neighbours or live species-pair blocks than the warps take
-  if (ws.cap_a <= cap_l && ac.n_pairs <= kGallBlocks) return;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int hgrid = std::max(1, std::min(n_in, 4 * std::max(sms, 1)));
-  const size_t hs = heavy_smem(ws, ac.n_pairs);
-  const int log_n = heavy_log_n(ws, ac.n_pairs);
-  if (ac.zeta == 32) {
-    if (want_virial) k_aev_bwd_heavy<32, true><<<hgrid, kHeavyThreads, hs, st>>>(ws, ac, log_n);
-    else k_aev_bwd_heavy<32, false><<<hgrid, kHeavyThreads, hs, st>>>(ws, ac, log_n);
-  } else {
-    if (want_virial) k_aev_bwd_heavy<0, true><<<hgrid, kHeavyThreads, hs, st>>>(ws, ac, log_n);
-    else k_aev_bwd_heavy<0, false><<<hgrid, kHeavyThreads, hs, st>>>(ws, ac, log_n);
+    if (want_virial) k_aev_bwd<0, true><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
+    else k_aev_bwd<0, false><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
   }
 }
 
@@ -1207,14 +1184,14 @@ cudaError_t aev_ensure_smem(const Ws& ws) {
   const int need_f = (int)aev_fwd_smem(ws);
   int need_h = 0;
   for (int np = 1; np <= kMaxSpecies * (kMaxSpecies + 1) / 2; ++np)
-    need_h = std::max(need_h, (int)heavy_smem(ws, np));
+    need_h = std::max(need_h, (int)bwd_cta_smem(ws, np));
   const void* fwd[2] = {(const void*)k_aev_fwd<32>, (const void*)k_aev_fwd<0>};
   const void* bwd[4] = {(const void*)k_aev_bwd<32, false>, (const void*)k_aev_bwd<32, true>,
                         (const void*)k_aev_bwd<0, false>, (const void*)k_aev_bwd<0, true>};
-  const void* hvy[4] = {(const void*)k_aev_bwd_heavy<32, false>,
-                        (const void*)k_aev_bwd_heavy<32, true>,
-                        (const void*)k_aev_bwd_heavy<0, false>,
-                        (const void*)k_aev_bwd_heavy<0, true>};
+  const void* hvy[4] = {(const void*)k_aev_bwd_cta<32, false>,
+                        (const void*)k_aev_bwd_cta<32, true>,
+                        (const void*)k_aev_bwd_cta<0, false>,
+                        (const void*)k_aev_bwd_cta<0, true>};
   for (int pass = 0; pass < 3; ++pass)
     for (int i = 0; i < (pass == 0 ? 2 : 4); ++i) {
       const void* fn = pass == 0 ? fwd[i] : pass == 1 ? bwd[i] : hvy[i];
@@ -1247,6 +1224,7 @@ void launch_aev_l1(const Ws& ws, const AevConst& ac, const void* w1_bf16, const 
   g.h1 = h1;
   g.alpha = alpha;
   g.stage_bytes = h1 * 64 * 2;
+  g.cap_l = light_cap(ws);
   const size_t sm = aev_l1_smem(ws, ac, h1);
   const int grid = (ws.row_cap + tcu::kTileM - 1) / tcu::kTileM;
   if (ac.zeta == 32) k_aev_l1<32><<<grid, kL1Warps * 32, sm, st>>>(m, ws, ac, g);

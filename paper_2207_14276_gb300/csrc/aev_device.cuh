@@ -74,12 +74,13 @@ __device__ __forceinline__ Geo pair_geo(const float4& xi, const float4& xj, cons
 
 // One lane per entry of a neighbour list: visit(slot, j, geometry) stages entry j.
 // A lane takes two entries per pass and issues both gathers before either is used.
-template <class Visit>
+// W warps share the list (lane: the thread's number among their 32 W).
+template <int W = 1, class Visit>
 __device__ __forceinline__ void stage_list(int n, const int* lst, const float4& xi, const SysDev& d,
                                            const Ws& ws, unsigned lane, Visit visit) {
   const float4* xyzq = ws.xyzq;
-  for (int t0 = 0; t0 < n; t0 += 64) {
-    const int ta = t0 + (int)lane, tb = ta + 32;
+  for (int t0 = 0; t0 < n; t0 += 64 * W) {
+    const int ta = t0 + (int)lane, tb = ta + 32 * W;
     int ja = ta < n ? lst[ta] : -1;
     int jb = tb < n ? lst[tb] : -1;
     if (ja >= 0 && !NNP_IN_BOUNDS(ws.status, kSiteAevNeighbour, ja, ws.totals[0])) ja = -1;

@@ -643,7 +643,7 @@ Ws call_ws(const nnp_handle* h) {
 
 // front_done: the whole front end ran in the first part's one CTA; energy_only: no system asks
 // for forces or a virial
-int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool energy_only,
+int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool masked, bool any_virial, bool energy_only,
                  cudaStream_t st, int* n_launch) {
   const Model& m = *h->model;
   const Ws ws = call_ws(h);
@@ -691,7 +691,7 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool any_virial, bool
     if ((rc = launch_check("mlp"))) return rc;
     if (!energy_only) {
       StageTimer t(h, st, 9);
-      launch_aev_bwd(ws, n_in, ac, any_virial ? 1 : 0, st);
+      launch_aev_bwd(ws, n_in, masked, ac, any_virial ? 1 : 0, st);
       if (ws.fr_det) { launch_det_force_gather(ws, n_in, st); ++launches; }
     }
     if ((rc = launch_check("aev_bwd"))) return rc;
@@ -719,7 +719,7 @@ void drop_graph(nnp_handle* h) {
 
 // a call's graph: its first part as kernel nodes, the rest captured behind them
 int capture_call(nnp_handle* h, const std::vector<FrontLaunch>& front, int n_in, bool front_done,
-                 bool any_virial, bool energy_only) {
+                 bool masked, bool any_virial, bool energy_only) {
   if (!h->cap_stream) CU_TRY(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   drop_graph(h);
   CU_TRY(cudaGraphCreate(&h->graph, 0));
@@ -738,7 +738,7 @@ int capture_call(nnp_handle* h, const std::vector<FrontLaunch>& front, int n_in,
   CU_TRY(cudaStreamBeginCaptureToGraph(h->cap_stream, h->graph, &h->front_nodes.back(), nullptr, 1,
                                        cudaStreamCaptureModeThreadLocal));
   int rest = 0;
-  const int rc = enqueue_rest(h, n_in, front_done, any_virial, energy_only, h->cap_stream, &rest);
+  const int rc = enqueue_rest(h, n_in, front_done, masked, any_virial, energy_only, h->cap_stream, &rest);
   cudaGraph_t same = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(h->cap_stream, &same);
   cudaError_t ei = cudaSuccess;
@@ -840,7 +840,8 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     }
     ++h->skin_calls;
   }
-  bool energy_only = true;
+  bool masked = false, energy_only = true;
+  for (int b = 0; b < n_sys; ++b) masked |= (sy[b].mask != nullptr);
   for (int b = 0; b < n_sys; ++b) energy_only &= (sy[b].forces == nullptr && sy[b].virial == nullptr);
   const bool front_done = one_cta_front(h, chunks.size(), n_in);
   if (n_in > 0) {   // what the diagnostic reads find in the arena, by replay too
@@ -878,13 +879,13 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     put(&ws.row_cap, sizeof(int));
     put(&ws.cell_cap, sizeof(int));
     put(&h->skin, sizeof(h->skin));
-    const bool flags[] = {ws.skin_state != nullptr, front_done,      any_virial,     energy_only,
+    const bool flags[] = {ws.skin_state != nullptr, front_done,      masked,         any_virial, energy_only,
                           h->fused_chain,           h->fused_aev_l1, h->sparse_rows, h->det};
     put(flags, sizeof(flags));
     for (const FrontLaunch& f : front) put(&f.fn, sizeof(f.fn));   // the nodes, whose grids may change
     // captured on the shape's second occurrence in a row, replayed afterwards
     if (!(h->gexec && sig == h->gsig) && sig == h->last_sig) {
-      if ((rc = capture_call(h, front, n_in, front_done, any_virial, energy_only))) return rc;
+      if ((rc = capture_call(h, front, n_in, front_done, masked, any_virial, energy_only))) return rc;
       h->gsig = sig;
     }
     if (h->gexec && sig == h->gsig) {
@@ -903,7 +904,7 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     ++launches;
   }
   if ((rc = launch_check("init/prep"))) return rc;
-  rc = enqueue_rest(h, n_in, front_done, any_virial, energy_only, st, &launches);
+  rc = enqueue_rest(h, n_in, front_done, masked, any_virial, energy_only, st, &launches);
   if (rc) return rc;
   h->last_launches = launches;
   h->last_n_in = n_in;
@@ -1789,7 +1790,7 @@ extern "C" int nnp_energy_forces_noalloc(nnp_handle* h, int64_t n_atoms, const f
     if ((rc = stage_ok("aev_fwd"))) return rc;
     launch_mlp_fp32(ws, m.md, m.mw, mb, m.alpha, st, nullptr, nullptr);
     if ((rc = stage_ok("mlp"))) return rc;
-    launch_aev_bwd(ws, n, m.ac, virial ? 1 : 0, st);
+    launch_aev_bwd(ws, n, mask != nullptr, m.ac, virial ? 1 : 0, st);
     if ((rc = stage_ok("aev_bwd"))) return rc;
     launch_finalize_e(ws, n, mb.e_row, m.md.E, 1, ws.row_cap, m.ebias, st);
   }

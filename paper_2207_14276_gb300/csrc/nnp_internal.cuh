@@ -189,7 +189,7 @@ struct Ws {
   float* dEdG;          // [row_cap][Dp]
   float* atom_e;        // [row_cap] per-row energy (mean over the ensemble, incl. shift)
   float4* f_pos;        // [n_in] forces on packed atoms
-  int* heavy;           // [n_in] packed positions of the centres the warp-per-centre
+  int* heavy;           // [n_in] packed positions of the centres that exceed the warp-per-centre
                         // AEV backward hands on (count in totals[2])
   // deterministic mode (null otherwise): the force kernels write every
   // contribution to its own slot instead of adding it atomically, and fixed-order
@@ -272,7 +272,8 @@ bool aev_l1_supported(const Ws& ws, const AevConst& ac, int E, int h1);
 void launch_aev_l1(const Ws& ws, const AevConst& ac, const void* w1_bf16, const float* b1,
                    void* H1, int h1, float alpha, cudaStream_t st);
 cudaError_t aev_l1_ensure_smem(const Ws& ws, const AevConst& ac, int h1);
-void launch_aev_bwd(const Ws& ws, int n_in, const AevConst& ac, int want_virial,
+// masked: some system has a mask (fewer centres than atoms)
+void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int want_virial,
                     cudaStream_t st);
 cudaError_t aev_ensure_smem(const Ws& ws);
 size_t aev_fwd_smem(const Ws& ws);
