@@ -50,7 +50,7 @@ constexpr int kWarps = 8;
 // dE/dG blocks of a centre held in shared memory by the warp-per-centre backward
 // kernel (the blocks with triplets, in block order; a centre with more goes to
 // the CTA-per-centre kernel)
-constexpr int kGallBlocks = 16;
+constexpr int kGallBlocks = kDenseBlocks;
 
 // float4s of shared memory per warp of the backward kernel: neighbour geometry
 // and cutoffs (2 cap_a), `copies` copies of the float4 accumulators (one per
@@ -103,23 +103,9 @@ __host__ __device__ constexpr int aev_fwd_warp_f4(int cap_a, int cap_r) {
   return cap_a + cap_a / 4 + cap_r / 2 + 2;
 }
 
-// species-pair blocks of a centre with triplets: pairs of present species and species
-// present at least twice (the same value on every lane)
-__device__ __forceinline__ int live_blocks(const ListHdr& H, const AevConst& ac, unsigned lane) {
-  const int c = (int)lane < ac.S ? H.off_a[lane + 1] - H.off_a[lane] : 0;
-  const int n_one = __popc(__ballot_sync(kFull, c >= 1));
-  const int n_two = __popc(__ballot_sync(kFull, c >= 2));
-  return n_one * (n_one - 1) / 2 + n_two;
-}
-
-// a centre whose backward exceeds what a warp stages joins ws.heavy (count in totals[2])
-__device__ __forceinline__ void note_dense(const Ws& ws, const AevConst& ac, const ListHdr& H, unsigned lane,
-                                           int p, int cap_l) {
-  const int n_live = live_blocks(H, ac, lane);
-  if (lane == 0 && (H.off_a[ac.S] > cap_l || n_live > kGallBlocks)) {
-    const int hi = atomicAdd(ws.totals + 2, 1);
-    if (NNP_IN_BOUNDS(ws.status, kSiteBwdHeavy, hi, ws.n_in)) ws.heavy[hi] = p;
-  }
+// whether a centre's list header makes it a dense one (the same value on every lane)
+__device__ __forceinline__ bool hdr_dense(const ListHdr& H, const AevConst& ac, unsigned lane) {
+  return is_dense(ac, H.off_a[ac.S], (int)lane < ac.S ? H.off_a[lane + 1] - H.off_a[lane] : 0);
 }
 
 // The AEV row of packed atom p (Eqs. 3-5) by W warps (1, or all kWarps of the CTA;
@@ -128,12 +114,12 @@ __device__ __forceinline__ void note_dense(const Ws& ws, const AevConst& ac, con
 // the list header.  The warps share the staged neighbours; warp w takes every W-th
 // species' radial block and every W-th angular block.  With sparse set, only the blocks
 // that touch a live slice of the row (row_slices) are stored, and *mask receives the
-// row's slice mask.
+// row's slice mask.  With skip_dense set a dense centre is left out (returns false).
 template <int ZETA, int W, class Out>
-__device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int p, float4* stage,
+__device__ __forceinline__ bool aev_centre(const Ws& ws, const AevConst& ac, int p, float4* stage,
                                            ListHdr& H, unsigned lane, const uint8_t* pair_su,
                                            Out out, bool sparse = false, uint32_t* mask = nullptr,
-                                           int w = 0) {
+                                           int w = 0, bool skip_dense = false) {
   auto sync = [] {
     if (W == 1) __syncwarp();
     else __syncthreads();
@@ -152,6 +138,7 @@ __device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int
   }
   if (W == 1 || w == 0) load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
   if (W > 1) __syncthreads();
+  if (skip_dense && hdr_dense(H, ac, lane)) return false;
   const uint32_t m = sparse ? row_slices(H, ac, lane, pair_su) : ~0u;
   if (mask) *mask = m;
   const int* lr = ws.nb_r + (size_t)p * ws.cap_r;
@@ -262,11 +249,12 @@ __device__ __forceinline__ void aev_centre(const Ws& ws, const AevConst& ac, int
   if (W == 1 || w == W - 1)
     for (int f = ac.D + lane; f < ac.Dp; f += 32)
       if ((m >> (f >> 6)) & 1u) out(f, 0.f);
+  return true;
 }
 
 template <int ZETA>
 __global__ void __launch_bounds__(kWarps * 32, 4)
-k_aev_fwd(Ws ws, AevConst ac, int small, int cap_l) {
+k_aev_fwd(Ws ws, AevConst ac, int small) {
   extern __shared__ float4 sm4[];
   __shared__ ListHdr hdrs[kWarps];
   __shared__ uint8_t pair_su[kMaxSpecies * (kMaxSpecies + 1) / 2];
@@ -301,28 +289,29 @@ k_aev_fwd(Ws ws, AevConst ac, int small, int cap_l) {
   };
   auto centre = [&](auto warps, int p, int wi, float4* stage, ListHdr& H) {
     constexpr int W = decltype(warps)::value;
-    const int slot = row_of(p, lane == 0 && wi == 0);
+    const int slot = row_of(p, lane == 0 && wi == 0);   // (a dense centre's: the same twice)
     if (!NNP_IN_BOUNDS(ws.status, kSiteAevRow, slot, ws.row_cap)) return;
     const size_t row = (size_t)slot * ac.Dp;
     float* G = ws.aev + row;
     uint16_t* Gh = ws.aev_h ? ws.aev_h + row : nullptr;
     uint16_t* Gl = ws.aev_l ? ws.aev_l + row : nullptr;
     uint32_t m = 0;
-    aev_centre<ZETA, W>(ws, ac, p, stage, H, lane, pair_su,
-                        [&](int f, float v) { put_g(G, Gh, Gl, f, v); }, sparse, &m, wi);
-    if (W == 1) note_dense(ws, ac, H, lane, p, cap_l);
-    if (sparse && lane == 0 && wi == 0) {
+    const bool done = aev_centre<ZETA, W>(ws, ac, p, stage, H, lane, pair_su,
+                                          [&](int f, float v) { put_g(G, Gh, Gl, f, v); }, sparse, &m, wi,
+                                          W == 1);
+    if (done && sparse && lane == 0 && wi == 0) {
       ws.row_mask[slot] = m;
       atomicOr(ws.tile_mask + (slot >> 7), m);
     }
   };
-  if (n <= small) {
-    // few centres: a CTA each (a warp alone works through a dense centre's blocks one
-    // after the other while the chip idles)
-    for (int p = blockIdx.x; p < n; p += gridDim.x)
-      centre(std::integral_constant<int, kWarps>{}, p, w, sm4, hdrs[0]);
-    return;
-  }
+  // a CTA each for the centres of a small batch and for the dense ones (a warp alone
+  // works through their blocks one after the other while the chip idles)
+  const bool all = n <= small;
+  const int n_cta = all ? n : ws.totals[2];
+  for (int h = blockIdx.x; h < n_cta; h += gridDim.x)
+    centre(std::integral_constant<int, kWarps>{}, all ? h : ws.heavy[h], w, sm4, hdrs[0]);
+  if (all) return;
+  __syncthreads();   // the stage and header become the warps' own
   // persistent: every warp takes the next centre from a counter until none is left
   // (dense centres do not hold a CTA's other warps' slots, nor pile up in one warp)
   for (;;) {
@@ -485,10 +474,8 @@ struct VirialSum {
   }
 };
 
-// Warp per centre, for centres with at most cap_l angular neighbours whose
-// angular terms fall in at most kGallBlocks species-pair blocks (the blocks'
-// dE/dG are all staged at once); the others, listed by the forward (note_dense),
-// are k_aev_bwd_cta's.
+// Warp per centre, for centres that are not dense (at most cap_l angular neighbours, in
+// at most kGallBlocks species-pair blocks, whose dE/dG are all staged at once).
 template <int ZETA, bool VIR>
 __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int log_r, int cap_l,
                                            int p, float4* sm4, ListHdr& H, int w, unsigned lane,
@@ -509,8 +496,8 @@ __device__ __forceinline__ void bwd_centre(const Ws& ws, const AevConst& ac, int
   const SysDev& d = ws.sys[ws.pos_sys[p]];
   const float* g_row = ws.dEdG + (size_t)ws.pos_slot[p] * ac.Dp;
   load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
-  const int n_live = live_blocks(H, ac, lane);
-  if (H.off_a[ac.S] > cap_l || n_live > kGallBlocks) return;   // k_aev_bwd_cta's
+  if (hdr_dense(H, ac, lane)) return;   // k_aev_bwd_cta's
+  const int n_live = live_blocks((int)lane < ac.S ? H.off_a[lane + 1] - H.off_a[lane] : 0);
   const int* lr = ws.nb_r + (size_t)p * ws.cap_r;
   const int* la = ws.nb_a + (size_t)p * ws.cap_a;
   const float inv_rc_r = 1.f / ac.rc_r, inv_rc_a = 1.f / ac.rc_a;
@@ -735,28 +722,28 @@ k_aev_bwd(Ws ws, AevConst ac, int log_r, int cap_l, int small) {
   }
 }
 
-// CTA per centre: for the centres listed in ws.heavy (more angular neighbours or
-// species-pair blocks than a warp stages: a dense solute core can have a hundred
-// neighbours, i.e. thousands of triplets), and for every centre of a small batch.  The
+// CTA per centre: for the dense centres (ws.heavy; a dense solute core can have a
+// hundred neighbours, i.e. thousands of triplets), and for every centre of a small batch.  The
 // CTA's eight warps share the centre's staged neighbours and dE/dG blocks and split its
 // radial edges and triplets.  The triplets come in the round-robin order of k_aev_bwd
 // in chunks of 32 (fewer for few neighbours: a chunk spans at most `copies` rounds of
 // disjoint pairs), every eighth chunk to a warp, which adds into its own accumulator
 // copies by plain read-add-write: no atomics, and the order of every addition is fixed,
 // which serves the deterministic mode too.  Persistent: CTAs stride over the list.
-// CTA_FIGURES
+// Dense centres of solvated100k: 44 us (65 us with shared-memory float atomics into
+// lane copies and pairs numbered by species block).
 constexpr int kCtaThreads = kWarps * 32;
 
 __host__ __device__ constexpr int bwd_cta_f4(int cap_a, int n_pairs, int copies) {
   return 2 * cap_a + kWarps * copies * cap_a + kMaxSpecies * kNR / 4 + kGallStride * n_pairs + (cap_a + 64 + 15) / 16;
 }
-// 4 copies where two CTAs then fit an SM, else 2
+// 4 copies where three CTAs then fit an SM, else 2
 int bwd_cta_copies(int cap_a, int n_pairs) {
-  return bwd_cta_f4(cap_a, n_pairs, 4) * 16 <= 110 * 1024 ? 4 : 2;
+  return bwd_cta_f4(cap_a, n_pairs, 4) * 16 <= 74 * 1024 ? 4 : 2;
 }
 
 template <int ZETA, bool VIR>
-__global__ void __launch_bounds__(kCtaThreads, 2)
+__global__ void __launch_bounds__(kCtaThreads, 3)
 k_aev_bwd_cta(Ws ws, AevConst ac, int copies, int small) {
   extern __shared__ float4 smh[];
   __shared__ ListHdr H;
@@ -951,7 +938,6 @@ struct AevL1Args {
   int h1;
   float alpha;
   int stage_bytes;      // one W1 slice: h1 x 64 BF16
-  int cap_l;            // angular neighbours of the warp-per-centre backward
 };
 
 __device__ __forceinline__ void put_tile(uint8_t* tile, int r, int f, float v) {
@@ -1012,7 +998,6 @@ k_aev_l1(const __grid_constant__ CUtensorMap tw1, Ws ws, AevConst ac, AevL1Args 
     if (slot < seg_end) {
       aev_centre<ZETA, 1>(ws, ac, ws.slot_pos[slot], stage, hdrs[w], lane, pair_su,
                           [&](int f, float v) { put_tile(tile, r, f, v); });
-      note_dense(ws, ac, hdrs[w], lane, ws.slot_pos[slot], g.cap_l);
     } else {
       for (int f = (int)lane; f < ac.Dp; f += 32) put_tile(tile, r, f, 0.f);
     }
@@ -1093,10 +1078,8 @@ size_t aev_l1_smem(const Ws& ws, const AevConst& ac, int h1) {
 size_t aev_fwd_smem(const Ws& ws) {
   return (size_t)kWarps * aev_fwd_warp_f4(ws.cap_a, ws.cap_r) * sizeof(float4);
 }
-// angular neighbours the warp-per-centre backward handles; centres with more go
-// to the CTA-per-centre kernel
-constexpr int kLightCapA = 48;
-static int light_cap(const Ws& ws) { return std::min(ws.cap_a, kLightCapA); }
+// angular neighbours a warp of the warp-per-centre backward stages
+static int light_cap(const Ws& ws) { return std::min(ws.cap_a, kDenseNeighbours); }
 
 size_t aev_bwd_smem(const Ws& ws, int n_pairs) {
   const int cap_l = light_cap(ws);
@@ -1120,21 +1103,23 @@ static int sm_count() {
 }
 
 // up to this many centres get a CTA each in the forward and the backward: four CTAs
-// per SM, one wave.  SMALL_FIGURES
+// per SM, one wave.  A 50-atom region: forward 34 -> 12 us, backward 28 -> 10 us; a
+// 24-atom molecule 9.1 -> 7.4 and 7.5 -> 6.0 us.
 static int small_centres() { return 4 * sm_count(); }
 
 // grid of the persistent warp-per-centre kernels: four CTAs per SM at most, fewer for
-// small batches (which have a CTA per centre up to `small` of them)
-static int centre_grid(int n_in, int small) {
-  return std::max(1, n_in <= small ? n_in : std::min(std::max((n_in + kWarps - 1) / kWarps, small), 4 * sm_count()));
+// small batches (up to `small` centres have a CTA each, and a mask may leave so few)
+static int centre_grid(int n_in, int small, bool masked) {
+  const int want = n_in <= small ? n_in : std::max((n_in + kWarps - 1) / kWarps, masked ? small : 1);
+  return std::max(1, std::min(want, 4 * sm_count()));
 }
 
-void launch_aev_fwd(const Ws& ws, int n_in, const AevConst& ac, cudaStream_t st) {
+void launch_aev_fwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, cudaStream_t st) {
   if (n_in <= 0) return;
   const size_t sm = aev_fwd_smem(ws);
-  const int small = small_centres(), grid = centre_grid(n_in, small);
-  if (ac.zeta == 32) k_aev_fwd<32><<<grid, kWarps * 32, sm, st>>>(ws, ac, small, light_cap(ws));
-  else k_aev_fwd<0><<<grid, kWarps * 32, sm, st>>>(ws, ac, small, light_cap(ws));
+  const int small = small_centres(), grid = centre_grid(n_in, small, masked);
+  if (ac.zeta == 32) k_aev_fwd<32><<<grid, kWarps * 32, sm, st>>>(ws, ac, small);
+  else k_aev_fwd<0><<<grid, kWarps * 32, sm, st>>>(ws, ac, small);
 }
 
 void launch_aev_fill(const Ws& ws, const AevConst& ac, cudaStream_t st) {
@@ -1143,9 +1128,19 @@ void launch_aev_fill(const Ws& ws, const AevConst& ac, cudaStream_t st) {
 }
 
 void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int want_virial,
-                    cudaStream_t st) {
+                    cudaStream_t st, const SideStream* side) {
   if (n_in <= 0) return;
   const int cap_l = light_cap(ws), small = small_centres();
+  // The two kernels add to different accumulators or atomically, so with a side stream
+  // they run together: the CTA-per-centre kernel first (higher priority), the other
+  // beside it as room allows (6k solvated atoms: 43 us one after the other, 34 together).
+  if (n_in <= small) side = nullptr;
+  const cudaStream_t main_st = st;
+  if (side) {
+    cudaEventRecord(side->fork, st);
+    cudaStreamWaitEvent(side->st, side->fork, 0);
+    st = side->st;
+  }
   // the CTA-per-centre kernel: where centres can exceed what a warp takes, and where
   // the batch is small (a mask may leave few centres of many atoms)
   if (n_in <= small || masked || ws.cap_a > cap_l || ac.n_pairs > kGallBlocks) {
@@ -1160,10 +1155,12 @@ void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int
     }
   }
   if (n_in <= small) return;
+  if (side) cudaEventRecord(side->join, st);
+  st = main_st;
   const size_t sm = aev_bwd_smem(ws, ac.n_pairs);
   const int copies = aev_bwd_copies(cap_l, ac.n_pairs);
   const int log_r = copies == 4 ? 2 : copies == 2 ? 1 : 0;
-  const int grid = centre_grid(n_in, small);
+  const int grid = centre_grid(n_in, small, masked);
   if (ac.zeta == 32) {
     if (want_virial) k_aev_bwd<32, true><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
     else k_aev_bwd<32, false><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
@@ -1171,6 +1168,7 @@ void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int
     if (want_virial) k_aev_bwd<0, true><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
     else k_aev_bwd<0, false><<<grid, kWarps * 32, sm, st>>>(ws, ac, log_r, cap_l, small);
   }
+  if (side) cudaStreamWaitEvent(st, side->join, 0);
 }
 
 // raise (never lower) the dynamic shared-memory limit of the AEV kernels to what
@@ -1224,7 +1222,6 @@ void launch_aev_l1(const Ws& ws, const AevConst& ac, const void* w1_bf16, const 
   g.h1 = h1;
   g.alpha = alpha;
   g.stage_bytes = h1 * 64 * 2;
-  g.cap_l = light_cap(ws);
   const size_t sm = aev_l1_smem(ws, ac, h1);
   const int grid = (ws.row_cap + tcu::kTileM - 1) / tcu::kTileM;
   if (ac.zeta == 32) k_aev_l1<32><<<grid, kL1Warps * 32, sm, st>>>(m, ws, ac, g);

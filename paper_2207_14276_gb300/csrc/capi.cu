@@ -118,6 +118,7 @@ struct nnp_handle {
   VjpBufs vb{};
   // the calls of one shape as a CUDA graph
   cudaStream_t cap_stream = nullptr;
+  nnp::SideStream side{nullptr, nullptr, nullptr};   // a branch of the graph
   cudaGraph_t graph = nullptr;      // kept: the nodes below belong to it
   cudaGraphExec_t gexec = nullptr;
   std::vector<cudaGraphNode_t> front_nodes;   // the kernels that take the descriptors
@@ -675,7 +676,7 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool masked, bool any
       launch_aev_l1(ws, ac, m.mw.W1cat_h, m.mw.b1cat, h->mb.H1, m.md.h1, m.alpha, st);
     } else {
       StageTimer t(h, st, 2);
-      launch_aev_fwd(wa, n_in, ac, st);
+      launch_aev_fwd(wa, n_in, masked, ac, st);
       if (wa.row_mask) { launch_aev_fill(wa, ac, st); ++launches; }
     }
     if ((rc = launch_check("aev_fwd"))) return rc;
@@ -691,7 +692,7 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool masked, bool any
     if ((rc = launch_check("mlp"))) return rc;
     if (!energy_only) {
       StageTimer t(h, st, 9);
-      launch_aev_bwd(ws, n_in, masked, ac, any_virial ? 1 : 0, st);
+      launch_aev_bwd(ws, n_in, masked, ac, any_virial ? 1 : 0, st, h->cap_stream && st == h->cap_stream ? &h->side : nullptr);
       if (ws.fr_det) { launch_det_force_gather(ws, n_in, st); ++launches; }
     }
     if ((rc = launch_check("aev_bwd"))) return rc;
@@ -720,7 +721,14 @@ void drop_graph(nnp_handle* h) {
 // a call's graph: its first part as kernel nodes, the rest captured behind them
 int capture_call(nnp_handle* h, const std::vector<FrontLaunch>& front, int n_in, bool front_done,
                  bool masked, bool any_virial, bool energy_only) {
-  if (!h->cap_stream) CU_TRY(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+  if (!h->cap_stream) {
+    int lo = 0, hi = 0;
+    CU_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    CU_TRY(cudaStreamCreateWithPriority(&h->side.st, cudaStreamNonBlocking, hi));
+    CU_TRY(cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming));
+    CU_TRY(cudaEventCreateWithFlags(&h->side.join, cudaEventDisableTiming));
+    CU_TRY(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+  }
   drop_graph(h);
   CU_TRY(cudaGraphCreate(&h->graph, 0));
   for (const FrontLaunch& f : front) {
@@ -992,6 +1000,9 @@ void nnp_destroy(nnp_handle* h) {
   if (h->tc_state) mlp_tc_release(h->tc_state);
   drop_graph(h);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+  if (h->side.st) cudaStreamDestroy(h->side.st);
+  if (h->side.fork) cudaEventDestroy(h->side.fork);
+  if (h->side.join) cudaEventDestroy(h->side.join);
   if (h->arena) cudaFree(h->arena);
   if (h->stage) cudaFree(h->stage);
   if (h->vjp_arena) cudaFree(h->vjp_arena);
@@ -1786,7 +1797,7 @@ extern "C" int nnp_energy_forces_noalloc(nnp_handle* h, int64_t n_atoms, const f
     if ((rc = stage_ok("cells"))) return rc;
     launch_neighbors(ws, n, m.ac, st);
     if ((rc = stage_ok("neighbors"))) return rc;
-    launch_aev_fwd(ws, n, m.ac, st);
+    launch_aev_fwd(ws, n, mask != nullptr, m.ac, st);
     if ((rc = stage_ok("aev_fwd"))) return rc;
     launch_mlp_fp32(ws, m.md, m.mw, mb, m.alpha, st, nullptr, nullptr);
     if ((rc = stage_ok("mlp"))) return rc;

@@ -623,6 +623,7 @@ __device__ void centre_lists_global(const Ws& ws, const AevConst& ac, int p, int
     wr_a += ca;
   }
   if (ws.row_key) group_row(ws, ac, p, __float_as_int(xi.w), my_r, my_a, pair_su);
+  if (ac.skin <= 0.f) note_dense(ws, ac, p, min(wr_a, ws.cap_a), my_a);   // (else the refresh does)
   if (lane == 0) {
     for (int s = ac.S; s < 8; ++s) { hdr[s] = 0; hdr[8 + s] = 0; }
     if (cnt > ws.cap_r || wr_a > ws.cap_a || cnt > kStageCap) {
@@ -724,6 +725,7 @@ __device__ __forceinline__ void centre_lists_staged(const Ws& ws, const AevConst
   }
   const int all_a = __shfl_sync(0xffffffffu, off_a, kMaxSpecies - 1);
   if (ws.row_key) group_row(ws, ac, p, __float_as_int(xi.w), cr, ca, pair_su);
+  if (ac.skin <= 0.f) note_dense(ws, ac, p, min(all_a, ws.cap_a), ca);   // (else the refresh does)
   off_r -= cr;
   off_a -= ca;
   if (lane < kMaxSpecies) {
@@ -796,7 +798,7 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
   const int n_cells = ws.totals[1];
   // work items: (cell, part) with `parts` CTAs per cell where the cells would not
   // fill the grid
-  const int parts = n_cells > 0 ? max(1, min((int)gridDim.x / n_cells, 8)) : 1;
+  const int parts = n_cells > 0 ? min(((int)gridDim.x + n_cells - 1) / n_cells, 8) : 1;
   const int n_items = n_cells * parts;
   int item = blockIdx.x;
   while (item < n_items) {
@@ -906,6 +908,7 @@ __global__ void __launch_bounds__(256) k_list_refresh(Ws ws, AevConst ac) {
   int* out_r = ws.nb_r + (size_t)p * ws.cap_r;
   int* out_a = ws.nb_a + (size_t)p * ws.cap_a;
   int off = 0, wr_r = 0, wr_a = 0;
+  int my_a = 0;   // lane s: angular neighbours of species s
   for (int s = 0; s < ac.S; ++s) {
     const int end = off + hm[s];
     int cr = 0, ca = 0;
@@ -944,10 +947,12 @@ __global__ void __launch_bounds__(256) k_list_refresh(Ws ws, AevConst ac) {
       hdr[s] = (uint16_t)max(0, min(cr, ws.cap_r - wr_r));
       hdr[8 + s] = (uint16_t)max(0, min(ca, ws.cap_a - wr_a));
     }
+    if ((int)lane == s) my_a = max(0, min(ca, ws.cap_a - wr_a));
     wr_r += cr;
     wr_a += ca;
     off = end;
   }
+  note_dense(ws, ac, p, min(wr_a, ws.cap_a), my_a);
   if (lane == 0) {
     for (int s = ac.S; s < 8; ++s) { hdr[s] = 0; hdr[8 + s] = 0; }
     if (wr_r > ws.cap_r || wr_a > ws.cap_a) {   // the call reports it; the retry grows the lists

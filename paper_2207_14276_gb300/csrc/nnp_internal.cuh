@@ -16,6 +16,13 @@ constexpr int kNZ = 8;             // angular sections (Eq. 5)
 constexpr int kRowTile = 128;      // species segments of AEV rows are padded to this
 constexpr int kMaxBatchParam = 64; // systems per kernel-parameter chunk
 constexpr int kStageCap = 512;     // staged radial neighbours per centre (hard cap)
+// A centre with more angular neighbours, or with more species pairs that have triplets,
+// than this is dense: the neighbour search (or, with persistent lists, the refresh)
+// lists it in Ws::heavy, and the AEV kernels give it a CTA instead of a warp.
+// (A warp alone on a solute's core set the duration of the forward: 6k solvated atoms
+// 42 us, 33 with the dense centres on CTAs.  Liquid water has 17 angular neighbours.)
+constexpr int kDenseNeighbours = 32;
+constexpr int kDenseBlocks = 16;
 
 // status word bits (device)
 enum : int {
@@ -189,8 +196,7 @@ struct Ws {
   float* dEdG;          // [row_cap][Dp]
   float* atom_e;        // [row_cap] per-row energy (mean over the ensemble, incl. shift)
   float4* f_pos;        // [n_in] forces on packed atoms
-  int* heavy;           // [n_in] packed positions of the centres that exceed the warp-per-centre
-                        // AEV backward hands on (count in totals[2])
+  int* heavy;           // [n_in] packed positions of the dense centres (is_dense below)
   // deterministic mode (null otherwise): the force kernels write every
   // contribution to its own slot instead of adding it atomically, and fixed-order
   // gathers and reductions sum them (results bitwise repeatable)
@@ -209,6 +215,25 @@ struct Ws {
   int* nbs_r;           // [n_in][cap_r]
   int* nbs_a;           // [n_in][cap_a]
 };
+
+// species pairs with triplets (one warp; c: lane s's angular neighbours of species s, 0
+// on the other lanes): pairs of present species and species present at least twice
+__device__ __forceinline__ int live_blocks(int c) {
+  const int n_one = __popc(__ballot_sync(0xffffffffu, c >= 1));
+  const int n_two = __popc(__ballot_sync(0xffffffffu, c >= 2));
+  return n_one * (n_one - 1) / 2 + n_two;
+}
+__device__ __forceinline__ bool is_dense(const AevConst& ac, int n_angular, int c) {
+  return n_angular > kDenseNeighbours || (ac.n_pairs > kDenseBlocks && live_blocks(c) > kDenseBlocks);
+}
+// packed atom p joins the list of dense centres (count in totals[2]) if it is one
+__device__ __forceinline__ void note_dense(const Ws& ws, const AevConst& ac, int p, int n_angular, int c) {
+  const bool dense = is_dense(ac, n_angular, c);
+  if (dense && (threadIdx.x & 31) == 0) {
+    const int hi = atomicAdd(ws.totals + 2, 1);
+    if (NNP_IN_BOUNDS(ws.status, kSiteBwdHeavy, hi, ws.n_in)) ws.heavy[hi] = p;
+  }
+}
 
 // whether this call rebuilds the cell lists and neighbour lists
 __device__ __forceinline__ bool lists_rebuild(const Ws& ws) {
@@ -261,7 +286,14 @@ void launch_det_force_gather(const Ws& ws, int n_in, cudaStream_t st);
 // positions in order
 void launch_det_reduce(const Ws& ws, int want_virial, cudaStream_t st);
 // ---- aev.cu
-void launch_aev_fwd(const Ws& ws, int n_in, const AevConst& ac, cudaStream_t st);
+// A second stream for work beside the call's: side work starts after fork (recorded on
+// the call's stream) and the call's stream goes on after join
+struct SideStream {
+  cudaStream_t st;
+  cudaEvent_t fork, join;
+};
+// masked: some system has a mask (fewer centres than atoms)
+void launch_aev_fwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, cudaStream_t st);
 // sparse rows (ws.row_mask set): zero the slices of each row that its tile reads
 // (tile mask) but the row itself left unwritten
 void launch_aev_fill(const Ws& ws, const AevConst& ac, cudaStream_t st);
@@ -272,9 +304,8 @@ bool aev_l1_supported(const Ws& ws, const AevConst& ac, int E, int h1);
 void launch_aev_l1(const Ws& ws, const AevConst& ac, const void* w1_bf16, const float* b1,
                    void* H1, int h1, float alpha, cudaStream_t st);
 cudaError_t aev_l1_ensure_smem(const Ws& ws, const AevConst& ac, int h1);
-// masked: some system has a mask (fewer centres than atoms)
 void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int want_virial,
-                    cudaStream_t st);
+                    cudaStream_t st, const SideStream* side = nullptr);
 cudaError_t aev_ensure_smem(const Ws& ws);
 size_t aev_fwd_smem(const Ws& ws);
 size_t aev_bwd_smem(const Ws& ws, int n_pairs = kMaxSpecies * (kMaxSpecies + 1) / 2);
