@@ -120,7 +120,8 @@ def fp32_alu_peak_tflops(sm_mhz):
 STAGE_SOURCE = {"mlp": "mlp_fused.cu", "aev_bwd": "aev.cu", "aev_fwd": "aev.cu",
                 "neighbors": "nl.cu", "mlp_l1": "mlp_tc.cu", "mlp_l2": "mlp_tc.cu",
                 "mlp_l3": "mlp_tc.cu", "mlp_b3": "mlp_tc.cu", "mlp_b2": "mlp_tc.cu",
-                "mlp_b1": "mlp_tc.cu", "mlp_chain": "mlp_chain.cu", "aev_l1": "aev.cu"}
+                "mlp_b1": "mlp_tc.cu", "mlp_chain": "mlp_chain.cu", "mlp_head": "mlp_head.cu",
+                "aev_l1": "aev.cu"}
 
 
 def recorded_traffic(stage, workload):
@@ -200,6 +201,9 @@ def stage_work(stage, spec, counts, n_atoms, path, sparse=(1.0, 1.0)):
     if stage == "mlp_chain":   # L2, L3, B3, B2 of every member, one fused kernel
         bound = {"bf16": "tensor", "fp32_split": "tensor_split"}.get(path, "alu")
         return 2.0 * n_atoms * E * (2 * h1 * h2 + 2 * h2 * h3), "FLOP", bound
+    if stage == "mlp_head":   # L3 and B3 of every member, one fused kernel
+        bound = {"bf16": "tensor", "fp32_split": "tensor_split"}.get(path, "alu")
+        return 2.0 * n_atoms * E * 2 * h2 * h3, "FLOP", bound
     gemm = {"mlp_l1": (D, E * h1), "mlp_l2": (h1, h2 * E), "mlp_l3": (h2, h3 * E),
             "mlp_b3": (h3, h2 * E), "mlp_b2": (h2, h1 * E), "mlp_b1": (E * h1, D)}
     if stage in gemm:
@@ -231,6 +235,7 @@ def gemm_bytes(stage, spec, n_atoms, path, sparse=(1.0, 1.0)):
                "mlp_l2": E * h1 * v + E * h2 * v,
                "mlp_l3": E * h2 * v + E * h3 * v + E * 4,
                "mlp_b3": E * h3 * v + 2 * E * h2 * v,
+               "mlp_head": 2 * E * h2 * v + E * 4,
                "mlp_b2": E * h2 * v + 2 * E * h1 * v,
                "mlp_b1": E * h1 * v + D * sparse[1] * 4}
     return n * per_row[stage] if stage in per_row else None

@@ -32,7 +32,7 @@ int mlp_tc_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, i
                    const float* aev, float* dEdG, bool split, void** state);
 void mlp_tc_release(void* state);
 void mlp_tc_use_chain(void* state, bool on);
-int mlp_tc_e_parts(void* state);
+int mlp_tc_e_parts(void* state, bool energy_only);
 void launch_aev_to_bf16(const Ws& ws, int n_in, const AevConst& ac, void* out, cudaStream_t st);
 void launch_wait_probe(int* status, unsigned limit, cudaStream_t st);
 }  // namespace nnp
@@ -358,6 +358,26 @@ int build_model(Model* m, const nnp_species_t* sp, const nnp_aev_params_t* a,
     if ((rc = upb(W3T, &mw.W3T_h, sp ? &mw.W3T_l : nullptr))) return rc;
     if ((rc = upb(W2T, &mw.W2T_h, sp ? &mw.W2T_l : nullptr))) return rc;
     if ((rc = upb(W1Tcat, &mw.W1Tcat_h, sp ? &mw.W1Tcat_l : nullptr))) return rc;
+    // images [c][K / 32][part][N] of the 64-byte rows that a 32-wide K slice of a [c][N][K]
+    // operand has in shared memory under the 64-byte swizzle (16-byte piece j of row r at
+    // j ^ (r / 2 % 4)); zeros past K
+    auto pack = [&](const std::vector<float>& v, size_t c_n, int N, int K, void** dst) {
+      const int n_sl = (K + 31) / 32, parts = sp ? 2 : 1;
+      std::vector<uint16_t> img(c_n * n_sl * parts * N * 32, 0);
+      for (size_t c = 0; c < c_n; ++c)
+        for (int r = 0; r < N; ++r)
+          for (int k = 0; k < K; ++k) {
+            const float x = v[(c * N + r) * K + k];
+            const uint16_t hb = bf16_bits(x);
+            const size_t piece = (size_t)(((k % 32) / 8) ^ ((r / 2) % 4));
+            const size_t at = (((c * n_sl + k / 32) * parts) * N + r) * 32 + piece * 8 + k % 8;
+            img[at] = hb;
+            if (sp) img[at + (size_t)N * 32] = bf16_bits(x - bf16_value(hb));
+          }
+      return upload(img.data(), img.size() * sizeof(uint16_t), dst);
+    };
+    if ((rc = pack(W3, (size_t)E * S, h3, h2, &mw.W3_img))) return rc;
+    if ((rc = pack(W3T, (size_t)E * S, h2, h3, &mw.W3T_img))) return rc;
   }
   return NNP_OK;
 }
@@ -462,7 +482,7 @@ size_t carve(nnp_handle* h, char* base) {
       mb.d3l = c.take<char>(rows * E * m.md.h3 * 2);
     }
   }
-  mb.e_row = c.take<float>((tc ? 2 : 1) * (size_t)E * rows);
+  mb.e_row = c.take<float>((tc ? kHeadParts : 1) * (size_t)E * rows);
   mb.aev_h = tc ? c.take<char>(rows * Dp * 2) : nullptr;
   mb.aev_l = split ? c.take<char>(rows * Dp * 2) : nullptr;
   ws.aev_h = static_cast<uint16_t*>(mb.aev_h);
@@ -528,8 +548,8 @@ int ensure_arena(nnp_handle* h, int n_in, int n_sys) {
 // stage names (index = stage id) reported by nnp_profile_read
 const char* kStageNames[] = {"prep", "neighbors", "aev_fwd", "mlp_l1", "mlp_l2", "mlp_l3",
                              "mlp_b3", "mlp_b2", "mlp_b1", "aev_bwd", "finalize", "mlp_cvt",
-                             "mlp", "mlp_chain", "aev_l1"};
-constexpr int kNumStages = 15;
+                             "mlp", "mlp_chain", "aev_l1", "mlp_head"};
+constexpr int kNumStages = 16;
 
 cudaEvent_t prof_event(nnp_handle* h) {
   if (!h->prof_pool.empty()) {
@@ -698,7 +718,7 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool masked, bool any
     if ((rc = launch_check("aev_bwd"))) return rc;
     {
       StageTimer t(h, st, 10);
-      launch_finalize_e(ws, n_in, h->mb.e_row, m.md.E, m.net != kNetSimt ? mlp_tc_e_parts(h->tc_state) : 1,
+      launch_finalize_e(ws, n_in, h->mb.e_row, m.md.E, m.net != kNetSimt ? mlp_tc_e_parts(h->tc_state, energy_only) : 1,
                         ws.row_cap, m.ebias, st);
       if (ws.e_det) { launch_det_reduce(ws, any_virial ? 1 : 0, st); ++launches; }
     }

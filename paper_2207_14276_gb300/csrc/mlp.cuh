@@ -64,7 +64,12 @@ struct MlpWeights {
   void* W1cat_h; void* W2_h; void* W3_h; void* W3T_h; void* W2T_h; void* W1Tcat_h;
   // split path: the low parts w - bf16(w), rounded to bf16 (same layouts)
   void* W1cat_l; void* W2_l; void* W3_l; void* W3T_l; void* W2T_l; void* W1Tcat_l;
+  // W3 and W3T as the fused L3 -> B3 kernel copies them (all parts): [E S][K / 32][part][N][32], swizzled
+  void* W3_img; void* W3T_img;
 };
+
+// planes of per-row energies of the fused L3 -> B3 kernel (its column groups of epilogue warps)
+constexpr int kHeadParts = 4;
 
 // activation buffers
 struct MlpBufs {
@@ -73,7 +78,7 @@ struct MlpBufs {
   void* H2;   // [rows][E*h2]  (reused for delta2)
   void* D2;   // [rows][E*h2]
   void* d3;   // [rows][E*h3]
-  float* e_row;  // [parts][E][rows]: 2 parts per row from the layer GEMMs on tensor cores, else 1
+  float* e_row;  // [parts][E][rows]: parts per row by the kernel of the last layer (mlp_tc_e_parts; 1 on FP32)
   void* aev_h;   // bf16 copy of the AEV (tensor-core path)
   // split path: low bf16 parts of the AEV, H1, H2 and d3 (same layouts as the
   // high parts, which are aev_h, H1, H2 and d3)

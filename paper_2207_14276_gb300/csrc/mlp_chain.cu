@@ -65,17 +65,6 @@ struct ChainArgs {
   int energy_only;
 };
 
-// shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row atoms 512 B apart
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;               // leading byte offset (unused with this swizzle)
-  d |= (uint64_t)(512 >> 4) << 32;      // stride byte offset
-  d |= (uint64_t)1 << 46;               // descriptor version
-  d |= (uint64_t)4 << 61;               // 64-byte swizzle
-  return d;
-}
-
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

@@ -40,6 +40,10 @@ namespace nnp {
 void* chain_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, int row_cap, bool split);
 void chain_release(void* plan);
 void launch_chain(void* plan, const Ws& ws, float alpha, bool energy_only, cudaStream_t st);
+// L3, the output and B3 in one kernel (mlp_head.cu)
+void* head_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, int row_cap, bool split);
+void head_release(void* plan);
+void launch_head(void* plan, const Ws& ws, float alpha, cudaStream_t st);
 
 namespace {
 
@@ -106,15 +110,6 @@ __device__ __forceinline__ bool ntile_live(const TcArgs& g, int m0, int n0) {
 // about 19 instructions (26 with scalar arithmetic and __expf, whose range handling
 // is not needed: results below 2^-126 flush to zero).  solvated100k: L1 234 -> 208 us,
 // L3 198 -> 186, B3 331 -> 313, B2 361 -> 356.
-__device__ __forceinline__ float2 bf2(uint32_t w) {   // two BF16 values as FP32
-  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-__device__ __forceinline__ float exp2_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // One 32-row x 16-column chunk of an epilogue warp's output, through shared
 // memory: every lane writes its row's 16 values into the warp's staging slot,
 // then lane 0 stores the box with TMA (full-line writes, where direct stores of
@@ -556,8 +551,10 @@ struct TcState {
   bool split = false;
   void* chain = nullptr;     // fused L2 -> L3 -> B3 -> B2 (null: the four layer GEMMs)
   bool use_chain = true;
+  void* head = nullptr;      // fused L3 -> B3 (null: two layer GEMMs)
   ~TcState() {
     if (chain) chain_release(chain);
+    if (head) head_release(head);
   }
 };
 
@@ -764,6 +761,7 @@ int mlp_tc_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, i
       return NNP_ERR_CUDA;
     }
   st->chain = chain_prepare(md, mw, mb, row_cap, split);
+  st->head = head_prepare(md, mw, mb, row_cap, split);
   *state_out = st;
   return NNP_OK;
 }
@@ -776,8 +774,9 @@ void mlp_tc_use_chain(void* state, bool on) {
 }
 
 // planes of per-row energy parts that the last layer leaves in MlpBufs::e_row
-int mlp_tc_e_parts(void* state) {
+int mlp_tc_e_parts(void* state, bool energy_only) {
   const TcState* s = static_cast<const TcState*>(state);
+  if (!(s->chain && s->use_chain) && s->head && !energy_only) return kHeadParts;
   return s->chain && s->use_chain ? 1 : epi_warps(s->split, kEpiCeluDot, false) / 4;
 }
 
@@ -792,8 +791,10 @@ int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const M
   TcState* s = static_cast<TcState*>(state);
   if (!s) return NNP_ERR_ARG;
   // plans 0-2 are the forward layers, 3-5 the backward to the input; with the
-  // fused chain: plan 0 (L1), the chain (L2, L3, B3, B2), plan 5 (B1)
+  // fused chain: plan 0 (L1), the chain (L2, L3, B3, B2), plan 5 (B1); without it a
+  // call for forces has L3 and B3 in one kernel (plans 2 and 3)
   const bool chain = s->chain && s->use_chain;
+  const bool head = !chain && s->head && !energy_only;
   const size_t n_plans = energy_only ? 3 : s->plans.size();
   // sparse AEV rows of this call (the AEV kernel wrote the tile masks)
   const uint32_t* tmask = (ws.row_mask && !skip_l1) ? ws.tile_mask : nullptr;
@@ -803,6 +804,14 @@ int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const M
       if (i == 1) {
         if (hook) hook->begin(13);
         launch_chain(s->chain, ws, alpha, energy_only, st);
+        if (hook) hook->end();
+      }
+      continue;
+    }
+    if (head && (i == 2 || i == 3)) {
+      if (i == 2) {
+        if (hook) hook->begin(15);
+        launch_head(s->head, ws, alpha, st);
         if (hook) hook->end();
       }
       continue;
@@ -852,7 +861,7 @@ int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const M
 #undef NNP_TC_LAUNCH
     if (hook) hook->end();
   }
-  if (n_launch) *n_launch += (chain ? (energy_only ? 2 : 3) : (int)n_plans) - (skip_l1 ? 1 : 0);
+  if (n_launch) *n_launch += (chain ? (energy_only ? 2 : 3) : (int)n_plans - (head ? 1 : 0)) - (skip_l1 ? 1 : 0);
   return NNP_OK;
 }
 

@@ -13,6 +13,18 @@
 namespace nnp {
 namespace tcu {
 
+// a walk around a ring of n slots: the slot, and the parity of its barrier's phase.  (A
+// division and a remainder per slot are a chain of a few hundred cycles for the one
+// thread that issues.)
+struct Ring {
+  int n, i = 0;
+  unsigned phase = 0;
+  __device__ explicit Ring(int n_) : n(n_) {}
+  __device__ void next() {
+    if (++i == n) { i = 0; phase ^= 1u; }
+  }
+};
+
 // polls of a bounded mbarrier wait before it gives up
 constexpr unsigned kWaitLimit = 1u << 24;
 // rows of an MMA tile (M) and of a species segment's row tiles
@@ -56,6 +68,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, volati
   return false;
 }
 
+// the same by a whole warp, the same answer on every lane
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, unsigned parity, volatile int* abort_flag) {
+  for (unsigned it = 0; it < kWaitLimit; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+
 // bounded wait that ignores the abort flag (used to drain in-flight work)
 __device__ __forceinline__ void mbar_drain(uint64_t* bar, unsigned parity) {
   for (unsigned it = 0; it < kWaitLimit; ++it)
@@ -68,6 +90,15 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+
+// contiguous bytes (a multiple of 16, both addresses 16-byte aligned)
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -109,6 +140,17 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   d |= (uint64_t)(1024 >> 4) << 32;     // stride byte offset
   d |= (uint64_t)1 << 46;               // descriptor version
   d |= (uint64_t)2 << 61;               // 128-byte swizzle
+  return d;
+}
+
+// shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row atoms 512 B apart
+__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)1 << 16;               // leading byte offset (unused with this swizzle)
+  d |= (uint64_t)(512 >> 4) << 32;      // stride byte offset
+  d |= (uint64_t)1 << 46;               // descriptor version
+  d |= (uint64_t)4 << 61;               // 64-byte swizzle
   return d;
 }
 
@@ -170,6 +212,15 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t taddr0, uint32_t taddr1, fl
     v0[i] = __uint_as_float(r[i]);
     v1[i] = __uint_as_float(r[16 + i]);
   }
+}
+
+__device__ __forceinline__ float2 bf2(uint32_t w) {   // two BF16 values as FP32
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+__device__ __forceinline__ float exp2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 __device__ __forceinline__ void store_bf16x16(__nv_bfloat16* dst, const float (&v)[16]) {
