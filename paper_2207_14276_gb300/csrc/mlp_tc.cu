@@ -175,7 +175,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
   __shared__ __align__(8) uint64_t aux_bar[kEpiWarps];   // per epilogue warp: its TMA'd aux boxes
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int kStages = g.stages;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int a_bytes = kBM * kBK * 2, b_bytes = g.n_tile * kBK * 2;
@@ -224,7 +224,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
   if (warp == kProdWarp) {
     if (lane == 0) {
       // ---- TMA producer
-      int it = 0;
+      int it = 0;   // copies issued so far
+      Ring rg(kStages);
       bool ok = true;
       for (int t = blockIdx.x; t < T && ok; t += gridDim.x) {
         const Tile tl = tile_of(t, n_tiles_n, row_tiles, g.nets, g.n_tile, g.seg_start, g.S);
@@ -233,9 +234,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
         const int a_c1 = tl.e * g.a_c1_per_e, b_c2 = tl.e * g.b_c2_per_e + tl.s;
         for (int kb = 0; kb < g.n_k; ++kb) {
           if (!((km >> kb) & 1u)) continue;   // an all-zero K slice of the tile
-          const int st = it % kStages;
-          const unsigned round = it / kStages;
-          if (it >= kStages && !mbar_wait(&empty_bar[st], (round - 1) & 1, abort_flag)) { ok = false; break; }
+          const int st = rg.i;
+          if (it >= kStages && !mbar_wait(&empty_bar[st], rg.phase ^ 1u, abort_flag)) { ok = false; break; }
           uint8_t* sa = smem + st * stage_bytes;
           uint8_t* sb = sa + kParts * a_bytes;
           mbar_expect_tx(&full_bar[st], (unsigned)stage_bytes);
@@ -245,7 +245,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
             tma_load_3d(sa + a_bytes, &ta2, &full_bar[st], kb * kBK, a_c1, tl.m0);
             tma_load_3d(sb + b_bytes, &tb2, &full_bar[st], kb * kBK, tl.n0, b_c2);
           }
-          ++it;   // copies issued so far
+          ++it;
+          rg.next();
         }
       }
       // every issued copy has landed before the CTA may exit
@@ -254,45 +255,47 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
           mbar_drain(&full_bar[k % kStages], (k / kStages) & 1);
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      // ---- MMA issuer
-      int it = 0, j = 0;
+    {
+      // ---- MMA issuer (the whole warp walks; lane 0 issues)
+      const uint32_t leader = lane == 0;
+      Ring rg(kStages);
+      int j = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < T && ok; t += gridDim.x) {
         const Tile tl = tile_of(t, n_tiles_n, row_tiles, g.nets, g.n_tile, g.seg_start, g.S);
         if (!ntile_live(g, tl.m0, tl.n0)) continue;
         const uint32_t km = g.kmask ? g.kmask[tl.m0 >> 7] : ~0u;
         const int ab = j & 1;
-        if (j >= 2 && !mbar_wait(&tempty_bar[ab], ((j >> 1) - 1) & 1, abort_flag)) break;
+        if (j >= 2 && !mbar_wait_warp(&tempty_bar[ab], ((j >> 1) - 1) & 1, abort_flag)) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(ab * g.tmem_cols);
         bool first_k = true;
         for (int kb = 0; kb < g.n_k; ++kb) {
           if (!((km >> kb) & 1u)) continue;
-          const int st = it % kStages;
-          if (!mbar_wait(&full_bar[st], (it / kStages) & 1, abort_flag)) { ok = false; break; }
-          ++it;
+          const int st = rg.i;
+          if (!mbar_wait_warp(&full_bar[st], rg.phase, abort_flag)) { ok = false; break; }
+          rg.next();
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + st * stage_bytes);
           const uint32_t sb = sa + kParts * a_bytes;
           const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sb);
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk) {
-            umma_bf16(d, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), g.idesc,
-                      (!first_k || kk > 0) ? 1u : 0u);
+            umma_bf16_w(d, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), g.idesc,
+                      (!first_k || kk > 0) ? 1u : 0u, leader);
             if (SPLIT) {
               const uint64_t adl = sw128_desc(sa + a_bytes), bdl = sw128_desc(sb + b_bytes);
-              umma_bf16(d, adl + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), g.idesc, 1u);
-              umma_bf16(d, ad + (uint64_t)(kk * 2), bdl + (uint64_t)(kk * 2), g.idesc, 1u);
+              umma_bf16_w(d, adl + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), g.idesc, 1u, leader);
+              umma_bf16_w(d, ad + (uint64_t)(kk * 2), bdl + (uint64_t)(kk * 2), g.idesc, 1u, leader);
             }
           }
-          umma_commit(&empty_bar[st]);
+          umma_commit_w(&empty_bar[st], leader);
           first_k = false;
         }
-        if (ok) umma_commit(&tfull_bar[ab]);
+        if (ok) umma_commit_w(&tfull_bar[ab], leader);
         ++j;
       }
-      umma_commit(&done_bar);   // arrives when every MMA issued above has completed
+      umma_commit_w(&done_bar, leader);   // arrives when every MMA issued above has completed
       mbar_drain(&done_bar, 0);
     }
   } else {
