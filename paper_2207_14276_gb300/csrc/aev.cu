@@ -103,6 +103,20 @@ __host__ __device__ constexpr int aev_fwd_warp_f4(int cap_a, int cap_r) {
   return cap_a + cap_a / 4 + cap_r / 2 + 2;
 }
 
+// (j, k) of triplet t of a species pair's block, cu the second species' neighbours: j = t /
+// cu, k = t % cu, and for one species the pairs around a circle, (t % cu, t % cu + t / cu
+// + 1).  The estimate is exact: t / cu < 512, its error below 2e-4, and (t + 0.5) / cu at
+// least 0.5 / 512 from a whole number.  (With the row-major triangle, whose row takes a
+// square root and two corrections, the forward of 100k solvated atoms took 299 us, 281 so;
+// 313 before the radial shells and the angular Gaussians went in packed pairs, too.)
+__device__ __forceinline__ void fwd_pair(int t, int same, int cu, float inv_cu, int* j, int* k) {
+  const int a = (int)((t + 0.5f) * inv_cu), b = t - a * cu;
+  int c = b + a + 1;
+  if (c >= cu) c -= cu;
+  *j = same ? b : a;
+  *k = same ? c : b;
+}
+
 // whether a centre's list header makes it a dense one (the same value on every lane)
 __device__ __forceinline__ bool hdr_dense(const ListHdr& H, const AevConst& ac, unsigned lane) {
   return is_dense(ac, H.off_a[ac.S], (int)lane < ac.S ? H.off_a[lane + 1] - H.off_a[lane] : 0);
@@ -155,24 +169,26 @@ __device__ __forceinline__ bool aev_centre(const Ws& ws, const AevConst& ac, int
                   angf[slot] = fcut(g.r, ac.rc_a, inv_rc_a);
                 });
   sync();
-  // ---- radial, Eq. 4
+  // ---- radial, Eq. 4: eight lanes per neighbour, two shells per lane (packed FP32x2),
+  // four neighbours at a time
   const float cr_ = -ac.eta_r * kLog2e;
-  const float my_shf = ac.shf_r[lane & 15];
-  const int half = lane >> 4;
+  const float2 my_shf = make_float2(ac.shf_r[2 * (lane & 7)], ac.shf_r[2 * (lane & 7) + 1]);
   for (int s = w; s < ac.S; s += W) {
-    float acc = 0.f;
     const int o = H.off_r[s], n = H.off_r[s + 1] - o;
-    if (n == 0) {   // no neighbour of this species: a zero block
-      if (lane < 16 && block_in(m, ac.rcol[s], kNR)) out(ac.rcol[s] + lane, 0.f);
-      continue;
-    }
-    for (int t = half; t < n; t += 2) {
+    if (!block_in(m, ac.rcol[s], kNR)) continue;
+    float2 acc = make_float2(0.f, 0.f);
+    for (int t = (int)lane >> 3; t < n; t += 4) {
       const float2 q = rad[o + t];
-      const float x = q.x - my_shf;
-      acc = fmaf(fast_exp2(cr_ * x * x), q.y, acc);
+      const float2 x = __fadd2_rn(make_float2(q.x, q.x), make_float2(-my_shf.x, -my_shf.y));
+      const float2 e = __fmul2_rn(__fmul2_rn(x, x), make_float2(cr_, cr_));
+      acc = __ffma2_rn(make_float2(fast_exp2(e.x), fast_exp2(e.y)), make_float2(q.y, q.y), acc);
     }
-    acc += __shfl_xor_sync(kFull, acc, 16);
-    if (lane < 16 && block_in(m, ac.rcol[s], kNR)) out(ac.rcol[s] + lane, acc);
+    // sums over the four neighbour lanes; lanes 0-15 hold the shells in turn
+    float v = (lane & 8) ? acc.y : acc.x;
+    const float u = (lane & 8) ? acc.x : acc.y;
+    v += __shfl_xor_sync(kFull, u, 8);
+    v += __shfl_xor_sync(kFull, v, 16);
+    if (lane < 16) out(ac.rcol[s] + 2 * (lane & 7) + (lane >> 3), v);
   }
   // ---- angular, Eq. 5: the blocks of species pairs with a pair j < k, and the
   // zero blocks of the other pairs where the row is written
@@ -205,7 +221,7 @@ __device__ __forceinline__ bool aev_centre(const Ws& ws, const AevConst& ac, int
       const int same = (s == u);
       const int n_tri = same ? cs * (cs - 1) / 2 : cs * cu;
       const int fb = ac.acol[q];
-      const float inv_cu = rcp_approx((float)max(cu, 1));   // decode corrects one step either way
+      const float inv_cu = rcp_approx((float)cu);
       // acc2[4a + m] holds features 8a + 2m and 8a + 2m + 1 (packed FP32x2 FMAs)
       float2 acc2[16];
 #pragma unroll
@@ -214,7 +230,7 @@ __device__ __forceinline__ bool aev_centre(const Ws& ws, const AevConst& ac, int
         const int t = t0 + lane;
         if (t < n_tri) {
           int j, k;
-          decode_pair(t, same, cs, cu, inv_cu, &j, &k);
+          fwd_pair(t, same, cu, inv_cu, &j, &k);
           const float4 vj = angv[os + j];
           const float4 vk = angv[ou + k];
           const float fjk = ac.ang_pre * angf[os + j] * angf[ou + k];
@@ -224,10 +240,12 @@ __device__ __forceinline__ bool aev_centre(const Ws& ws, const AevConst& ac, int
           const float rb = 0.5f * (vj.w + vk.w);
           float2 A[kNA];
 #pragma unroll
-          for (int a = 0; a < kNA; ++a) {
-            const float x = rb - ac.shf_a[a];
-            const float v = fast_exp2(ca_ * x * x) * fjk;
-            A[a] = make_float2(v, v);
+          for (int a = 0; a < kNA; a += 2) {
+            const float2 x = __fadd2_rn(make_float2(rb, rb), make_float2(-ac.shf_a[a], -ac.shf_a[a + 1]));
+            const float2 e = __fmul2_rn(__fmul2_rn(make_float2(ca_, ca_), x), x);
+            const float v0 = fast_exp2(e.x) * fjk, v1 = fast_exp2(e.y) * fjk;
+            A[a] = make_float2(v0, v0);
+            A[a + 1] = make_float2(v1, v1);
           }
           const float2 c2 = make_float2(c, c), s2 = make_float2(sn, sn);
 #pragma unroll

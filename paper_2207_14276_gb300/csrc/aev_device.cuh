@@ -169,14 +169,13 @@ __device__ __forceinline__ RoundRobin make_round_robin(int n) {
   rr.h = max(odd ? (n - 1) / 2 : n / 2, 1);
   rr.off = odd ? 1 : 0;
   rr.n_tri = n * (n - 1) / 2;
-  rr.inv_h = rcp_approx((float)rr.h);   // rr_round corrects the estimate by one step
+  rr.inv_h = rcp_approx((float)rr.h);
   return rr;
 }
-// round of pair t (exact: the float estimate is corrected by one step)
+// round of pair t.  Exact: t / h is below 512 (kStageCap neighbours), so the estimate is
+// within 2e-4 of (t + 0.5) / h, which is at least 0.5 / 256 from a whole number.
 __device__ __forceinline__ int rr_round(const RoundRobin& rr, int t) {
   int r = (int)((t + 0.5f) * rr.inv_h);
-  if (r * rr.h > t) --r;
-  else if ((r + 1) * rr.h <= t) ++r;
   return r;
 }
 __device__ __forceinline__ void rr_pair(const RoundRobin& rr, int t, int* round, int* a, int* b) {
