@@ -27,7 +27,7 @@ using namespace nnp;
 namespace nnp {
 int launch_mlp_tc(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb,
                   float alpha, cudaStream_t st, int* n_launch, StageHook* hook, void* state,
-                  bool energy_only, bool skip_l1);
+                  bool energy_only, bool skip_l1, bool masked);
 int mlp_tc_prepare(const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb, int row_cap,
                    const float* aev, float* dEdG, bool split, void** state);
 void mlp_tc_release(void* state);
@@ -704,7 +704,7 @@ int enqueue_rest(nnp_handle* h, int n_in, bool front_done, bool masked, bool any
     StageHook hook{h, st};
     if (m.net != kNetSimt) {
       rc = launch_mlp_tc(wa, m.md, m.mw, h->mb, m.alpha, st, &launches, &hook, h->tc_state, energy_only,
-                         fuse_l1);
+                         fuse_l1, masked);
       if (rc) return rc;
     } else {
       launch_mlp_fp32(wa, m.md, m.mw, h->mb, m.alpha, st, &launches, &hook, energy_only);
