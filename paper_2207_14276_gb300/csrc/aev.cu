@@ -5,11 +5,11 @@
 // radial list, (unit vector, R) and (f_c, f_c') for the angular sub-list.
 //
 // Forward
-//   radial  (Eq. 4): two half-warps take alternate neighbours of one species, a
-//           lane owns one Gaussian shell r; an xor-16 shuffle adds the halves
-//           and lanes 0..15 write the block's 16 features.
+//   radial  (Eq. 4): eight lanes per neighbour of one species, four neighbours at a
+//           time, a lane owns two Gaussian shells (packed FP32x2); two shuffles add
+//           the four and lanes 0..15 write the block's 16 features.
 //   angular (Eq. 5): lane-per-triplet.  The (j, k) pairs of one unordered
-//           species pair are numbered and decoded in closed form; every lane
+//           species pair are numbered by a quotient and a remainder; every lane
 //           forms the 4 Gaussians of the averaged distance and the 8 angular
 //           factors of its pair (two sections per packed FP32x2 instruction)
 //           and accumulates all 32 products in registers.
