@@ -892,8 +892,11 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
 }
 
 // Lists at the cutoffs from the persistent lists at the cutoffs + skin, one warp
-// per centre: the entries of each species block of the longer radial list whose
-// current distance is within rc_r (radial) or rc_a (angular), in their order.
+// per centre: the entries of the longer radial list whose current distance is within
+// rc_r (radial) or rc_a (angular), in their order.  Bound by the chain of loads of a
+// centre, so its entries are taken 32 at a time whatever their species, and lane s counts
+// those of species s (one species block after the other: seven such chains, 6.5 us for
+// a 50-atom region, 3.5 so).
 __global__ void __launch_bounds__(256) k_list_refresh(Ws ws, AevConst ac) {
   const int p = blockIdx.x * 8 + (threadIdx.x >> 5);
   const unsigned lane = threadIdx.x & 31;
@@ -902,64 +905,68 @@ __global__ void __launch_bounds__(256) k_list_refresh(Ws ws, AevConst ac) {
   const SysDev& d = ws.sys[ws.pos_sys[p]];
   const int per = d.in.periodic;
   const float rr2 = ac.rc_r * ac.rc_r, ra2 = ac.rc_a * ac.rc_a;
-  const uint16_t* hm = ws.nbs_cnt + (size_t)p * 16;
   const int* lm = ws.nbs_r + (size_t)p * ws.cap_r;
   uint16_t* hdr = ws.nb_cnt + (size_t)p * 16;
   int* out_r = ws.nb_r + (size_t)p * ws.cap_r;
   int* out_a = ws.nb_a + (size_t)p * ws.cap_a;
-  int off = 0, wr_r = 0, wr_a = 0;
-  int my_a = 0;   // lane s: angular neighbours of species s
-  for (int s = 0; s < ac.S; ++s) {
-    const int end = off + hm[s];
-    int cr = 0, ca = 0;
-    for (int t0 = off; t0 < end; t0 += 32) {
-      const int t = t0 + (int)lane;
-      bool keep = false, ang = false;
-      int j = 0;
-      if (t < end) {
-        j = lm[t];
-        const float4 xj = ws.xyzq[j];
-        float dv[3] = {xj.x - xi.x, xj.y - xi.y, xj.z - xi.z};
-        if (per)
-          for (int c = 0; c < 3; ++c) {
-            const float n = rintf(dv[c] / d.in.box_hi[c]);
-            dv[c] = fmaf(-n, d.in.box_lo[c], fmaf(-n, d.in.box_hi[c], dv[c]));
-          }
-        const float r2 = dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2];
-        keep = r2 <= rr2 && r2 > 1e-12f;
-        ang = keep && r2 <= ra2;
-      }
-      const unsigned br = __ballot_sync(0xffffffffu, keep);
-      const unsigned ba = __ballot_sync(0xffffffffu, ang);
-      if (keep) {
-        const int at = wr_r + cr + __popc(br & lanemask_lt());
-        if (at < ws.cap_r && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j, ws.totals[0])) out_r[at] = j;
-      }
-      if (ang) {
-        const int at = wr_a + ca + __popc(ba & lanemask_lt());
-        if (at < ws.cap_a && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j, ws.totals[0])) out_a[at] = j;
-      }
-      cr += __popc(br);
-      ca += __popc(ba);
+  // lane s: species s's entries [off, end) of the longer list, and how many are kept
+  const int cnt = (int)lane < ac.S ? ws.nbs_cnt[(size_t)p * 16 + lane] : 0;
+  auto before = [&](int c) {   // exclusive sum over the lanes
+    int incl = c;
+    for (int o = 1; o < 8; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((int)lane >= o) incl += u;
     }
-    // counts clamped so that the lists stay inside their capacity
-    if (lane == 0) {
-      hdr[s] = (uint16_t)max(0, min(cr, ws.cap_r - wr_r));
-      hdr[8 + s] = (uint16_t)max(0, min(ca, ws.cap_a - wr_a));
+    return incl - c;
+  };
+  const int off = before(cnt), end = off + cnt;
+  const int total = __shfl_sync(0xffffffffu, end, 7);
+  auto below = [](int n) { return n >= 32 ? 0xffffffffu : n <= 0 ? 0u : (1u << n) - 1u; };
+  int cr = 0, ca = 0, wr_r = 0, wr_a = 0;
+  for (int t0 = 0; t0 < total; t0 += 32) {
+    const int t = t0 + (int)lane;
+    bool keep = false, ang = false;
+    int j = 0;
+    if (t < total) {
+      j = lm[t];
+      const float4 xj = ws.xyzq[j];
+      float dv[3] = {xj.x - xi.x, xj.y - xi.y, xj.z - xi.z};
+      if (per)
+        for (int c = 0; c < 3; ++c) {
+          const float n = rintf(dv[c] / d.in.box_hi[c]);
+          dv[c] = fmaf(-n, d.in.box_lo[c], fmaf(-n, d.in.box_hi[c], dv[c]));
+        }
+      const float r2 = dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2];
+      keep = r2 <= rr2 && r2 > 1e-12f;
+      ang = keep && r2 <= ra2;
     }
-    if ((int)lane == s) my_a = max(0, min(ca, ws.cap_a - wr_a));
-    wr_r += cr;
-    wr_a += ca;
-    off = end;
+    const unsigned br = __ballot_sync(0xffffffffu, keep);
+    const unsigned ba = __ballot_sync(0xffffffffu, ang);
+    if (keep) {
+      const int at = wr_r + __popc(br & lanemask_lt());
+      if (at < ws.cap_r && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j, ws.totals[0])) out_r[at] = j;
+    }
+    if (ang) {
+      const int at = wr_a + __popc(ba & lanemask_lt());
+      if (at < ws.cap_a && NNP_IN_BOUNDS(ws.status, kSiteNbCandidate, j, ws.totals[0])) out_a[at] = j;
+    }
+    const unsigned mine = below(end - t0) & ~below(off - t0);
+    cr += __popc(br & mine);
+    ca += __popc(ba & mine);
+    wr_r += __popc(br);
+    wr_a += __popc(ba);
   }
-  note_dense(ws, ac, p, min(wr_a, ws.cap_a), my_a);
-  if (lane == 0) {
-    for (int s = ac.S; s < 8; ++s) { hdr[s] = 0; hdr[8 + s] = 0; }
-    if (wr_r > ws.cap_r || wr_a > ws.cap_a) {   // the call reports it; the retry grows the lists
-      atomicOr(ws.status, kStCapacity);
-      atomicMax(ws.status + 1, wr_r);
-      atomicMax(ws.status + 2, wr_a);
-    }
+  // counts clamped so that the lists stay inside their capacity
+  const int fit_a = max(0, min(ca, ws.cap_a - before(ca))), fit_r = max(0, min(cr, ws.cap_r - before(cr)));
+  if (lane < 8) {
+    hdr[lane] = (uint16_t)fit_r;
+    hdr[8 + lane] = (uint16_t)fit_a;
+  }
+  note_dense(ws, ac, p, min(wr_a, ws.cap_a), fit_a);
+  if (lane == 0 && (wr_r > ws.cap_r || wr_a > ws.cap_a)) {   // the call reports it; the retry grows the lists
+    atomicOr(ws.status, kStCapacity);
+    atomicMax(ws.status + 1, wr_r);
+    atomicMax(ws.status + 2, wr_a);
   }
 }
 
