@@ -350,10 +350,8 @@ k_head_tc(const __grid_constant__ CUtensorMap mH, const __grid_constant__ CUtens
             const float2 w2 = u ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
             const float2 z = __fadd2_rn(make_float2(v[2 * p], v[2 * p + 1]),
                                         u ? make_float2(b4.z, b4.w) : make_float2(b4.x, b4.y));
-            const float2 t = __fmul2_rn(z, make_float2(ez_scale, ez_scale));
-            const float2 ez = make_float2(exp2_ftz(t.x), exp2_ftz(t.y));
-            const float2 n2 = __ffma2_rn(ez, make_float2(alpha, alpha), make_float2(-alpha, -alpha));
-            dot2 = __ffma2_rn(make_float2(z.x > 0.f ? z.x : n2.x, z.y > 0.f ? z.y : n2.y), w2, dot2);
+            float2 ez;
+            dot2 = __ffma2_rn(celu2<SPLIT>(z, alpha, inv_alpha, ez_scale, ez), w2, dot2);
             float2 d3 = __fmul2_rn(w2, make_float2(z.x > 0.f ? 1.f : ez.x, z.y > 0.f ? 1.f : ez.y));
             if (!row_ok) d3 = make_float2(0.f, 0.f);   // bounds-checked build only
             hi[ci][p] = split_pair<SPLIT>(d3, &lo[SPLIT ? ci : 0][p]);

@@ -105,8 +105,8 @@ __device__ __forceinline__ bool ntile_live(const TcArgs& g, int n_tile, int m0, 
   return ((m >> a) & span) != 0u;
 }
 
-// The epilogues work on pairs of columns with packed FP32x2 instructions and take the
-// exponential as 2^x with the scale folded in: an element of a split CELU layer costs
+// The epilogues work on pairs of columns with packed FP32x2 instructions and, on split
+// operands, take the exponential as 2^x with the scale folded in (celu2): an element of a split CELU layer costs
 // about 19 instructions (26 with scalar arithmetic and __expf, whose range handling
 // is not needed: results below 2^-126 flush to zero).  solvated100k: L1 234 -> 208 us,
 // L3 198 -> 186, B3 331 -> 313, B2 361 -> 356.
@@ -441,10 +441,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float2 z = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]), make_float2(b[2 * i], b[2 * i + 1]));
-            const float2 t = __fmul2_rn(z, make_float2(ez_scale, ez_scale));
-            const float2 ez = make_float2(exp2_ftz(t.x), exp2_ftz(t.y));   // exp(z / alpha)
-            const float2 n2 = __ffma2_rn(ez, make_float2(alpha, alpha), make_float2(-alpha, -alpha));
-            const float2 h = make_float2(z.x > 0.f ? z.x : n2.x, z.y > 0.f ? z.y : n2.y);
+            float2 ez;   // exp(z / alpha)
+            const float2 h = celu2<SPLIT>(z, alpha, inv_alpha, ez_scale, ez);
             if (EPI == kEpiCeluDot) {
               const float2 w2 = make_float2(w4[2 * i], w4[2 * i + 1]);
               dot2 = __ffma2_rn(h, w2, dot2);

@@ -241,6 +241,24 @@ __device__ __forceinline__ float exp2_ftz(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// CELU of a pair of z, and exp(z / alpha) in ez (CELU' where z <= 0).  On split operands
+// as 2^x with the scale folded in and the packed multiply-add.  On BF16 operands both
+// results are rounded to 16 bits next, where another last bit of FP32 moves a value by
+// 2^-9: there the exponential of z / alpha, rounded step by step as the FP32 networks'
+// formula has it (2^x instead moved the forces by 1.7e-4 of their norm).
+template <bool SPLIT>
+__device__ __forceinline__ float2 celu2(float2 z, float alpha, float inv_alpha, float ez_scale, float2& ez) {
+  float2 n;
+  if (SPLIT) {
+    const float2 t = __fmul2_rn(z, make_float2(ez_scale, ez_scale));
+    ez = make_float2(exp2_ftz(t.x), exp2_ftz(t.y));
+    n = __ffma2_rn(ez, make_float2(alpha, alpha), make_float2(-alpha, -alpha));
+  } else {
+    ez = make_float2(__expf(z.x * inv_alpha), __expf(z.y * inv_alpha));
+    n = make_float2(alpha * (ez.x - 1.f), alpha * (ez.y - 1.f));
+  }
+  return make_float2(z.x > 0.f ? z.x : n.x, z.y > 0.f ? z.y : n.y);
+}
 
 __device__ __forceinline__ void store_bf16x16(__nv_bfloat16* dst, const float (&v)[16]) {
   uint32_t w[8];
