@@ -10,6 +10,8 @@ library holds its own device copy; the tensor carries the gradient).
 """
 from __future__ import annotations
 
+import operator
+
 import torch
 
 
@@ -41,6 +43,11 @@ class NNPBatchFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, coords, weights, potential, species, sizes, boxes=None):
         x, sp = coords.detach().contiguous(), species.contiguous()
+        if isinstance(sizes, int):   # systems of one size, as torch.split takes it
+            sizes = [len(t) for t in torch.split(sp, sizes)]
+        if not isinstance(sizes, (list, tuple)):
+            raise TypeError(f"sizes: an int or a list of ints, not {type(sizes).__name__}")
+        sizes = [operator.index(n) for n in sizes]
         E, F = potential.energy_forces_flat(x, sp, sizes, boxes)
         ctx.set_materialize_grads(False)   # an unused output's gradient stays None
         ctx.potential, ctx.x, ctx.sp, ctx.sizes, ctx.boxes = potential, x, sp, sizes, boxes

@@ -228,6 +228,26 @@ def test_one_graph_for_new_buffers_streams_and_capture(torch_cuda, n_mol):
     check(pot, orc, [boxes[3]], "fp32")
 
 
+@gpu
+def test_batch_sizes_as_torch_split_takes_them(torch_cuda):
+    torch = torch_cuda
+    from paper_2207_14276_gb300 import Potential
+    from paper_2207_14276_gb300.autograd import NNPBatchFunction
+    spec, w = model("ani4")
+    pot = Potential(spec, w)
+    s = to_cuda(synth.workload("gas24")[0][0])
+    x, wt = s["coords"].repeat(3, 1)[:60].contiguous(), torch.from_numpy(w).cuda()
+    sp = s["species"].repeat(3)[:60].contiguous()
+    out = [NNPBatchFunction.apply(x, wt, pot, sp, sizes) for sizes in (24, [24, 24, 12], (24, 24, 12))]
+    for E, F in out[1:]:
+        torch.testing.assert_close(E, out[0][0], rtol=1e-6, atol=1e-6)
+        torch.testing.assert_close(F, out[0][1], rtol=1e-5, atol=1e-5)
+    with pytest.raises(TypeError):
+        NNPBatchFunction.apply(x, wt, pot, sp, [24.0, 24.0, 12.0])
+    with pytest.raises(RuntimeError):
+        NNPBatchFunction.apply(x, wt, pot, sp, [24, 24])
+
+
 def test_pair_numbers_of_the_angular_blocks():
     """The (quotient, remainder) of the forward's triplet numbers from a float
     reciprocal off by up to two units in its last place, for every block of up to 512
