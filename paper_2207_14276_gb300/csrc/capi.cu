@@ -137,6 +137,7 @@ struct nnp_handle {
   // tensor-core paths: AEV rows written only in their live 64-column slices, the
   // first and last layer GEMMs restricted to them (exact: the rest is zero)
   bool sparse_rows = true;
+  bool whole_rows = false;       // FMA paths: the budget has no room for the rows' masks and groups
   bool last_sparse = false;      // the last call ran with sparse rows
   bool last_vjp = false;         // the last call was a force VJP
   // deterministic mode: atoms and AEV rows in sorted order, force and energy
@@ -482,17 +483,24 @@ size_t carve(nnp_handle* h, char* base) {
       mb.d3l = c.take<char>(rows * E * m.md.h3 * 2);
     }
   }
-  mb.e_row = c.take<float>((tc ? kHeadParts : 1) * (size_t)E * rows);
   mb.aev_h = tc ? c.take<char>(rows * Dp * 2) : nullptr;
   mb.aev_l = split ? c.take<char>(rows * Dp * 2) : nullptr;
   ws.aev_h = static_cast<uint16_t*>(mb.aev_h);
   ws.aev_l = static_cast<uint16_t*>(mb.aev_l);
   // rows written only in their live slices (the first layer reads a tile's live
   // slices, the last backward layer computes only those)
-  ws.row_mask = c.take<uint32_t>(rows);
-  ws.tile_mask = c.take<uint32_t>(rows / kRowTile + 1);
-  ws.row_key = c.take<uint32_t>(n);
-  ws.row_hist = c.take<int>(kMaxSpecies * 32);
+  ws.row_mask = h->whole_rows ? nullptr : c.take<uint32_t>(rows);
+  ws.tile_mask = h->whole_rows ? nullptr : c.take<uint32_t>(rows / kRowTile + 1);
+  // The output layer's parts and the row groups.  On the tensor-core paths they lie in
+  // the FP32 rows, which only the force VJP writes there (it reads neither, and the next
+  // energy call rebuilds its lists): an arena at its budget has no room to spare.
+  const size_t e_parts = (tc ? kHeadParts : 1) * (size_t)E * rows;
+  const bool inside = tc && align_up(e_parts * 4, 256) + align_up(n * 4, 256) + kMaxSpecies * 32 * 4 <= rows * Dp * 4;
+  Carve in_rows{reinterpret_cast<char*>(ws.aev)};
+  Carve& x = inside ? in_rows : c;
+  mb.e_row = x.take<float>(e_parts);
+  ws.row_key = h->whole_rows ? nullptr : x.take<uint32_t>(n);
+  ws.row_hist = h->whole_rows ? nullptr : x.take<int>(kMaxSpecies * 32);
   return align_up(c.off, 256);
 }
 
@@ -504,10 +512,17 @@ int ensure_arena(nnp_handle* h, int n_in, int n_sys) {
   const int old_in = h->cap_in, old_sys = h->cap_sys;
   h->cap_in = want_in;
   h->cap_sys = want_sys;
-  const size_t bytes = carve(h, nullptr);
+  const bool old_whole = h->whole_rows;
+  h->whole_rows = false;
+  size_t bytes = carve(h, nullptr);
+  if (h->budget && bytes > h->budget && h->model->net == kNetSimt) {
+    h->whole_rows = true;   // the FMA paths run without the masks as well
+    bytes = carve(h, nullptr);
+  }
   if (h->budget && bytes > h->budget) {
     h->cap_in = old_in;
     h->cap_sys = old_sys;
+    h->whole_rows = old_whole;
     carve(h, static_cast<char*>(h->arena));
     return fail(NNP_ERR_OOM, "work arena of " + std::to_string(bytes) + " bytes exceeds the HBM budget");
   }
@@ -648,7 +663,7 @@ bool fuses_aev_l1(const nnp_handle* h) {
 // (the fused FP32 kernel reads whole rows)
 bool sparse_call(const nnp_handle* h) {
   const Model& m = *h->model;
-  return h->sparse_rows && !fuses_aev_l1(h) && !(m.net == kNetSimt && mlp_fused_supported(m.md));
+  return h->sparse_rows && h->ws.row_mask && !fuses_aev_l1(h) && !(m.net == kNetSimt && mlp_fused_supported(m.md));
 }
 
 // the work space as this call's kernels see it: rows are grouped by their live slices
@@ -1362,7 +1377,7 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
   ws.e_det = ws.v_det = nullptr;
   h->last_aev_fp32 = true;
   h->last_aev_stored = true;
-  h->last_sparse = h->sparse_rows;
+  h->last_sparse = ws.row_mask != nullptr;
   h->last_vjp = true;
   // the force VJP builds its own lists at the cutoffs in the shared buffers:
   // persistent lists of energy calls are rebuilt on the next such call

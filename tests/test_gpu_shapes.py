@@ -248,6 +248,28 @@ def test_batch_sizes_as_torch_split_takes_them(torch_cuda):
         NNPBatchFunction.apply(x, wt, pot, sp, [24, 24])
 
 
+# a budget of what lists, rows and activations alone take has room for the call: the row
+# groups and output parts lie in the FP32 rows, or the FMA paths run without masks
+@gpu
+@pytest.mark.parametrize("kind,precision,ensemble", [
+    ("ani7", "fp32", 1), ("ani7x8", "bf16", 8), ("ani7x8", "fp32_simt", 8), ("ani7", "fp32_simt", 1)])
+def test_a_budget_of_the_arena_without_extras(torch_cuda, kind, precision, ensemble):
+    from paper_2207_14276_gb300 import Potential
+    from paper_2207_14276_gb300._lib import NNPError
+    spec, w = model(kind)
+    systems = [synth.solvated_solute(400, 60, 24.0, seed=6)]
+    room = (systems[0].n_atoms, 1, 288, 96)
+    with pytest.raises(NNPError) as e:
+        Potential(spec, w, precision=precision, hbm_budget=1).reserve(*room)
+    need = int(str(e.value).split("work arena of ")[1].split()[0])
+    pot, orc = Potential(spec, w, precision=precision, hbm_budget=need), oracle.Model(spec, w)
+    pot.reserve(*room)
+    for _ in range(3):
+        check(pot, orc, systems, precision)
+    with pytest.raises(NNPError):
+        Potential(spec, w, precision=precision, hbm_budget=need - 1).reserve(*room)
+
+
 def test_pair_numbers_of_the_angular_blocks():
     """The (quotient, remainder) of the forward's triplet numbers from a float
     reciprocal off by up to two units in its last place, for every block of up to 512
