@@ -89,7 +89,8 @@ struct TcArgs {
   int* status;
   // sparse AEV rows (null: dense): the live 64-column slices of each 128-row
   // tile; the first layer reads only those K slices, the last backward layer
-  // skips the N tiles with none of them
+  // skips the N tiles with none of them.  (An AEV row has 20 slices at most; the K of
+  // the last backward layer, all members' h1, has no mask and no such limit.)
   const uint32_t* kmask;
   const uint32_t* nmask;
   int n_slot;            // output staging slots per epilogue warp (1 or 2)
@@ -237,10 +238,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       for (int t = blockIdx.x; t < T && ok; t += gridDim.x) {
         const Tile tl = tile_of(t, n_tiles_n, row_tiles, g.nets, n_tile, g.seg_start, g.S);
         if (!ntile_live(g, n_tile, tl.m0, tl.n0)) continue;
-        const uint32_t km = g.kmask ? g.kmask[tl.m0 >> 7] : ~0u;
+        const uint32_t km = g.kmask ? g.kmask[tl.m0 >> 7] : 0u;
         const int a_c1 = tl.e * g.a_c1_per_e, b_c2 = tl.e * g.b_c2_per_e + tl.s;
         for (int kb = 0; kb < g.n_k; ++kb) {
-          if (!((km >> kb) & 1u)) continue;   // an all-zero K slice of the tile
+          if (g.kmask && !((km >> kb) & 1u)) continue;   // an all-zero K slice of the tile
           const int st = rg.i;
           if (it >= kStages && !mbar_wait(&empty_bar[st], rg.phase ^ 1u, abort_flag)) { ok = false; break; }
           uint8_t* sa = smem + st * stage_bytes;
@@ -273,14 +274,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       for (int t = blockIdx.x; t < T && ok; t += gridDim.x) {
         const Tile tl = tile_of(t, n_tiles_n, row_tiles, g.nets, n_tile, g.seg_start, g.S);
         if (!ntile_live(g, n_tile, tl.m0, tl.n0)) continue;
-        const uint32_t km = g.kmask ? g.kmask[tl.m0 >> 7] : ~0u;
+        const uint32_t km = g.kmask ? g.kmask[tl.m0 >> 7] : 0u;
         const int ab = j & 1;
         if (j >= 2 && !mbar_wait_warp(&tempty_bar[ab], ((j >> 1) - 1) & 1, abort_flag)) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(ab * g.tmem_cols);
         bool first_k = true;
         for (int kb = 0; kb < g.n_k; ++kb) {
-          if (!((km >> kb) & 1u)) continue;
+          if (g.kmask && !((km >> kb) & 1u)) continue;
           const int st = rg.i;
           if (!mbar_wait_warp(&full_bar[st], rg.phase, abort_flag)) { ok = false; break; }
           rg.next();
