@@ -147,6 +147,7 @@ struct nnp_handle {
   float skin = 0.f;
   bool lists_valid = false;   // the lists in the arena belong to list_sig's batch layout
   std::string list_sig;
+  int list_owner = 0;         // its number (a new one whenever lists_valid was lost)
   long long skin_calls = 0;
   // optional per-stage CUDA-event timing
   bool profile = false;
@@ -447,7 +448,7 @@ size_t carve(nnp_handle* h, char* base) {
     ws.e_det = ws.v_det = nullptr;
   }
   if (h->skin > 0.f) {
-    ws.skin_state = c.take<int>(4);
+    ws.skin_state = c.take<int>(5);
     ws.ref = c.take<float4>(n);
     ws.in_pos = c.take<int>(n);
     ws.nbs_cnt = c.take<uint16_t>(n * 16);
@@ -893,7 +894,9 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     h->last_vjp = false;
   }
   const bool forced = ws.skin_state && !h->lists_valid;
-  const std::vector<FrontLaunch> front = front_launches(call_ws(h), chunks, call_const(h), n_in, front_done, forced);
+  if (forced) h->list_owner = h->list_owner % 0x3fffffff + 1;
+  const std::vector<FrontLaunch> front =
+      front_launches(call_ws(h), chunks, call_const(h), n_in, front_done, forced ? -h->list_owner : h->list_owner);
   h->pub_valid = ws.status_pub != nullptr && n_in > 0;
   h->pub_stream = st;
   // systems without atoms: the outputs are the empty sums
@@ -1379,8 +1382,10 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
   h->last_aev_stored = true;
   h->last_sparse = ws.row_mask != nullptr;
   h->last_vjp = true;
-  // the force VJP builds its own lists at the cutoffs in the shared buffers:
-  // persistent lists of energy calls are rebuilt on the next such call
+  // the force VJP builds its own lists at the cutoffs in the shared buffers (and writes
+  // the FP32 AEV rows, where a tensor-core handle's row groups lie): persistent lists of
+  // energy calls are rebuilt on the next such call, on the device too, where a call that
+  // the caller captured finds them
   struct SkinOff {
     Ws& w;
     int* saved;
@@ -1388,6 +1393,8 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
     ~SkinOff() { w.skin_state = saved; }
   } skin_off(ws);
   h->lists_valid = false;
+  if (h->ws.skin_state)
+    CU_TRY(cudaMemsetAsync(h->ws.skin_state + 3, 0, sizeof(int), static_cast<cudaStream_t>(stream)));
   int in_base = 0;
   std::vector<BatchParams> chunks;
   for (int b0 = 0; b0 < n_sys; b0 += kMaxBatchParam) {
@@ -1411,7 +1418,7 @@ extern "C" int nnp_force_vjp_batch(nnp_handle* h, int n_sys, const nnp_vjp_syste
   const bool front_done = chunks.size() == 1 && n_in <= kFrontMaxAtoms;
   h->pub_valid = ws.status_pub != nullptr;
   h->pub_stream = st;
-  for (const FrontLaunch& f : front_launches(ws, chunks, m.ac, n_in, front_done, false)) f.launch(st);
+  for (const FrontLaunch& f : front_launches(ws, chunks, m.ac, n_in, front_done, 0)) f.launch(st);
   if (!front_done) {
     launch_setup(ws, m.ac, st);
     launch_bin(ws, n_in, st);
@@ -1823,7 +1830,7 @@ extern "C" int nnp_energy_forces_noalloc(nnp_handle* h, int64_t n_atoms, const f
       return NNP_OK;
     };
     const std::vector<BatchParams> chunks(1, bp);
-    for (const FrontLaunch& f : front_launches(ws, chunks, m.ac, n, false, false)) f.launch(st);
+    for (const FrontLaunch& f : front_launches(ws, chunks, m.ac, n, false, 0)) f.launch(st);
     if ((rc = stage_ok("init/prep"))) return rc;
     launch_setup(ws, m.ac, st);
     launch_bin(ws, n, st);

@@ -14,7 +14,7 @@ __global__ void k_finalize(Ws ws, const float* e_row, int E, int parts, int e_ro
     if (lists_rebuild(ws)) {
       // the lists built in this call serve later calls unless they overflowed
       ws.skin_state[2] += 1;
-      ws.skin_state[3] = (ws.status[0] & (kStCapacity | kStCells)) ? 0 : 1;
+      ws.skin_state[3] = (ws.status[0] & (kStCapacity | kStCells)) ? 0 : ws.skin_state[4];
     }
     ws.skin_state[0] = ws.skin_state[1] = 0;   // the next call's check starts from here
   }

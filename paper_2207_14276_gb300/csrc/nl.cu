@@ -430,13 +430,17 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(Ws ws, BatchParamsT<N> 
 
 // Largest displacement of an atom of the last build's lists since that build
 // (minimum image in periodic directions), as float bits into skin_state[0]
-// (positive floats order like their bit patterns).
+// (positive floats order like their bit patterns).  owner: number of the batch layout
+// whose lists this call uses, negative where the host knows that they are to be built.
+// The device compares it with the layout of the last build: a call that the caller
+// captured carries the number of its own layout, whatever ran between its replays.
 template <int N>
-__global__ void k_skin_check(Ws ws, BatchParamsT<N> bp, int n_chunk, int forced) {
-  if (forced) {   // the batch's layout changed: nothing to compare with
-    if (blockIdx.x == 0 && threadIdx.x == 0) ws.skin_state[1] = 1;
-    return;
+__global__ void k_skin_check(Ws ws, BatchParamsT<N> bp, int n_chunk, int owner) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ws.skin_state[4] = abs(owner);   // k_finalize notes it as the owner of the lists built
+    if (owner < 0 || ws.skin_state[3] != owner) ws.skin_state[1] = 1;
   }
+  if (owner < 0) return;   // nothing to compare with
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   float d2 = 0.f;
   if (t < n_chunk) {
@@ -973,7 +977,7 @@ __global__ void __launch_bounds__(256) k_list_refresh(Ws ws, AevConst ac) {
 }  // namespace
 
 std::vector<FrontLaunch> front_launches(const Ws& ws, const std::vector<BatchParams>& chunks,
-                                        const AevConst& ac, int n_in, bool one_cta, bool forced) {
+                                        const AevConst& ac, int n_in, bool one_cta, int owner) {
   std::vector<FrontLaunch> out;
   const bool few = chunks.size() == 1 && chunks[0].n_sys <= kFewSystems;
 #define NNP_FEW(kernel) (few ? (const void*)kernel<kFewSystems> : (const void*)kernel<kMaxBatchParam>)
@@ -993,7 +997,7 @@ std::vector<FrontLaunch> front_launches(const Ws& ws, const std::vector<BatchPar
   };
   if (ws.skin_state)
     for (const BatchParams& bp : chunks)
-      if (atoms(bp) > 0) add(NNP_FEW(k_skin_check), forced ? 1 : atoms(bp), all, bp, atoms(bp), forced);
+      if (atoms(bp) > 0) add(NNP_FEW(k_skin_check), owner < 0 ? 1 : atoms(bp), all, bp, atoms(bp), owner);
   // the first chunk's init also zeroes the shared counters
   const int cells = std::min(ws.cell_cap, 2 * ws.n_in + 27 * ws.n_sys);
   for (const BatchParams& bp : chunks) {

@@ -206,8 +206,9 @@ struct Ws {
   double* e_det;        // [n_in] atomic energy (FP64), by packed position
   double* v_det;        // [n_in][9] the centre's virial contribution
   // persistent neighbour lists with a skin (null skin_state: rebuilt every call)
-  int* skin_state;      // [4]: max displacement (float bits), forced rebuild (both zeroed by the
-                        // call's last kernel for the next call), builds, lists valid
+  int* skin_state;      // [5]: max displacement (float bits), forced rebuild (both zeroed by the
+                        // call's last kernel for the next call), builds, the batch layout that
+                        // the lists belong to (0: none), the layout of this call
   float half_skin;      // rebuild when an atom moved farther than this since the build
   float4* ref;          // [n_in] input coordinates at the last build
   int* in_pos;          // [n_in] packed position of an input atom at the last build (-1: none)
@@ -267,9 +268,10 @@ struct FrontLaunch {
   }
 };
 // the launches of a batch in order; one_cta: the whole front end of a one-chunk batch
-// in one CTA; forced: persistent lists are rebuilt whatever the displacements
+// in one CTA; owner: number of the batch layout that persistent lists are kept for,
+// negative: they are built whatever the displacements (0 without persistent lists)
 std::vector<FrontLaunch> front_launches(const Ws& ws, const std::vector<BatchParams>& chunks,
-                                        const AevConst& ac, int n_in, bool one_cta, bool forced);
+                                        const AevConst& ac, int n_in, bool one_cta, int owner);
 void launch_setup(const Ws& ws, const AevConst& ac, cudaStream_t st);
 void launch_bin(const Ws& ws, int n_in, cudaStream_t st);
 void launch_scan(const Ws& ws, cudaStream_t st);
