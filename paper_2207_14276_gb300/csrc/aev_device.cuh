@@ -130,13 +130,12 @@ __device__ __forceinline__ float2 section_pair(const AevConst& ac, int m, float2
   const float2 sz = reinterpret_cast<const float2*>(ac.sin_z)[m];
   const float2 base = __ffma2_rn(s2, sz, __ffma2_rn(c2, cz, make_float2(1.f, 1.f)));
   if constexpr (ZETA == 32) {
-    float2 p = __fmul2_rn(base, base);   // ^2
-    p = __fmul2_rn(p, p);                // ^4
-    p = __fmul2_rn(p, p);                // ^8
-    p = __fmul2_rn(p, p);                // ^16
+    const float2 p2 = __fmul2_rn(base, base), p4 = __fmul2_rn(p2, p2), p8 = __fmul2_rn(p4, p4);
+    const float2 p = __fmul2_rn(p8, p8);   // ^16
     const float2 B = __fmul2_rn(p, p);
-    // base >= 1 + cos(15 pi / 16) > 0: base^31 = base^32 / base
-    if (B1) *B1 = __fmul2_rn(B, make_float2(rcp_approx(base.x), rcp_approx(base.y)));
+    // base^31 by products: base is 0 where a section lies opposite to a collinear pair
+    // (and base^32 / base then 0 times infinity)
+    if (B1) *B1 = __fmul2_rn(__fmul2_rn(p, p8), __fmul2_rn(__fmul2_rn(p4, p2), base));
     return B;
   } else {
     const float2 b1 = make_float2(ipow<0>(base.x, ac.zeta - 1), ipow<0>(base.y, ac.zeta - 1));

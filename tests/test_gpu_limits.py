@@ -2,13 +2,15 @@
 
 Bounds, those of the parity tests: FP32 forces within 1e-4 of their RMS, energies within
 1e-3 kcal/mol and within 1e-4 of sum_i |E_i|; BF16 forces within 2e-2 of their RMS (2^-9
-relative per operand).
+relative per operand); gradients of the loss within 1e-3 of their norm and largest element.
 """
+import numpy as np
 import pytest
 
 import oracle
 import synth
-from tests.test_gpu_shapes import check, model
+from tests._common import to_cuda
+from tests.test_gpu_shapes import check, close, model
 
 gpu = pytest.mark.gpu
 
@@ -34,3 +36,47 @@ def test_first_layers_of_all_members_past_2048_columns(torch_cuda, precision, en
     for sparse in (False, True):
         pot.set_sparse_rows(sparse)
         check(pot, orc, systems, precision)
+
+
+# Sections of 0 .. 0.7 rad and two neighbours on opposite sides of a centre: 1 + cos(theta -
+# theta_z) is exactly 0 in the first section (the distance 2 and its reciprocal are exact) and
+# below 0.24 in the others, whose 32nd powers vanish.  (The two are farther apart than the
+# angular cutoff: seen from one of them the others would lie on one side, where the energy has
+# a cusp.)  The oracle, which divides by sin(theta), has the pair 1e-7 A off the line.
+def collinear():
+    spec, w = model("ani4", shf_z=tuple(0.1 * z for z in range(8)))
+    x = np.array([[0, 0, 0], [0, 0, 2], [0, 0, -2], [1.25, 0.5, 0.25], [-1.5, 0.75, 0.5]], np.float32)
+    s = synth.systems.System("collinear", x, np.array([1, 3, 3, 0, 0], np.uint8))
+    off = x.astype(np.float64)
+    off[1, 0] += 1e-7
+    return spec, w, s, off
+
+
+@gpu
+@pytest.mark.parametrize("precision", ["fp32", "fp32_simt", "bf16"])
+def test_a_section_opposite_to_a_collinear_pair(torch_cuda, precision):
+    from paper_2207_14276_gb300 import Potential
+    spec, w, s, off = collinear()
+    ref = oracle.Model(spec, w).energy_forces(off, s.species)
+    assert np.isfinite(ref["forces"]).all()
+    pot = Potential(spec, w, precision=precision)
+    far = synth.water_box(300, 20.5, 7, seed=41)   # beside it, centres have a warp each
+    for systems in ([s], [s, far]):
+        o = pot.energy_forces_batch([to_cuda(q) for q in systems])[0]
+        close(o, ref, precision)
+
+
+@gpu
+def test_gradients_with_a_section_opposite_to_a_collinear_pair(torch_cuda):
+    torch = torch_cuda
+    from paper_2207_14276_gb300 import Potential
+    spec, w, s, off = collinear()
+    pot, orc = Potential(spec, w), oracle.Model(spec, w)
+    v = np.random.Generator(np.random.PCG64(12)).normal(size=(s.n_atoms, 3))
+    _, _, gx, gw = pot.force_vjp_batch([to_cuda(s)], [0.0], [torch.from_numpy(v).float().cuda()])
+    _, _, gx_ref, gw_ref = orc.force_matching(off, s.species, v.astype(np.float32))
+    for got, ref in ((gx[0], gx_ref), (gw, gw_ref)):
+        assert np.isfinite(ref).all()
+        d = got.cpu().numpy().astype(np.float64) - ref
+        assert np.linalg.norm(d) <= 1e-3 * np.linalg.norm(ref)
+        assert np.abs(d).max() <= 1e-3 * np.abs(ref).max()
