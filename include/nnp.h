@@ -477,7 +477,9 @@ int nnp_noalloc_max_atoms(const nnp_handle* h, int64_t* max_atoms);
  * the handle's arena must not have been reused by a later call.
  *
  * nnp_debug_rows: which = 0 -> atomic environment vectors G_i (Eqs. 4-5),
- *   which = 1 -> dE/dG_i (the network gradient fed to the force kernel).
+ *   which = 1 -> dE/dG_i (the network gradient fed to the force kernel).  An
+ *   energy-only call forms none: on the FP32 FMA chain of ensembles the read
+ *   forms it then, elsewhere the rows are what the last call for forces left.
  *   out: device float32 [n_in_total, aev_dim], row i = input atom i of the
  *   batch (systems concatenated in call order); rows of atoms outside the
  *   mask are left untouched.

@@ -140,6 +140,7 @@ struct nnp_handle {
   bool whole_rows = false;       // FMA paths: the budget has no room for the rows' masks and groups
   bool last_sparse = false;      // the last call ran with sparse rows
   bool last_vjp = false;         // the last call was a force VJP
+  bool last_bwd = false;         // ... or ran its networks' backward
   // deterministic mode: atoms and AEV rows in sorted order, force and energy
   // contributions in their own slots summed in a fixed order (bitwise repeatable)
   bool det = false;
@@ -892,6 +893,7 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
     h->last_aev_stored = !fuses_aev_l1(h);
     h->last_sparse = sparse_call(h);
     h->last_vjp = false;
+    h->last_bwd = !energy_only;
   }
   const bool forced = ws.skin_state && !h->lists_valid;
   if (forced) h->list_owner = h->list_owner % 0x3fffffff + 1;
@@ -1622,21 +1624,26 @@ int nnp_debug_rows(nnp_handle* h, int which, float* out, void* stream) {
   const uint16_t* src_l = planes ? h->ws.aev_l : nullptr;
   Ws gw = h->ws;
   if (!h->last_sparse) gw.row_mask = nullptr;   // the last call wrote whole rows
-  if (which == 1 && h->last_sparse && (h->last_vjp || h->model->net == kNetSimt)) {
+  const Model& m = *h->model;
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (which == 1 && !h->last_vjp && !h->last_bwd && m.net == kNetSimt && !mlp_fused_supported(m.md)) {
+    // after an energy-only call H1 holds activations, not deltas: the backward runs now
+    launch_mlp_fp32_bwd(h->ws, m.md, m.mw, h->mb, m.alpha, st, nullptr, true);
+    h->last_bwd = true;
+    gw.row_mask = nullptr;
+  } else if (which == 1 && h->last_sparse && (h->last_vjp || m.net == kNetSimt)) {
     // the FP32 chains' dE/dG is read back whole: the columns that the call left out
     // (the forces do not read them) are computed now from its deltas
-    const Model& m = *h->model;
     const int kd = m.md.E * m.md.h1;
     GemmArgs g = gemm_base(h->ws, m);
     g.A = h->last_vjp ? h->vb.dl1 : h->mb.H1; g.lda = kd;
     g.B = m.mw.W1Tcat; g.b_s = (long long)m.ac.Dp * kd; g.ldb = kd;
     g.N = m.ac.Dp; g.K = kd; g.epi = kEpiStore;
     g.out = h->ws.dEdG; g.ldo = m.ac.Dp;
-    launch_gemm_fp32(g, h->ws.row_cap, static_cast<cudaStream_t>(stream), 1);
+    launch_gemm_fp32(g, h->ws.row_cap, st, 1);
     gw.row_mask = nullptr;
   }
-  launch_gather_rows(gw, h->last_n_in, src, src_h, src_l, h->model->ac.Dp, h->model->ac.D,
-                     h->model->col_of_feat_dev, out, which == 1, static_cast<cudaStream_t>(stream));
+  launch_gather_rows(gw, h->last_n_in, src, src_h, src_l, m.ac.Dp, m.ac.D, m.col_of_feat_dev, out, which == 1, st);
   CU_TRY(cudaGetLastError());
   return NNP_OK;
 }

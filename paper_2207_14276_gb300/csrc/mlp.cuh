@@ -106,5 +106,7 @@ void launch_mlp_fused(const Ws& ws, const MlpDims& md, const MlpWeights& mw, con
 void launch_mlp_fp32(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb,
                      float alpha, cudaStream_t st, int* n_launch, StageHook* hook,
                      bool energy_only = false);
+void launch_mlp_fp32_bwd(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb,
+                         float alpha, cudaStream_t st, StageHook* hook, bool whole);
 
 }  // namespace nnp

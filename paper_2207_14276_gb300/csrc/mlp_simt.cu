@@ -325,6 +325,49 @@ void launch_gemm_dual(const GemmArgs& g, int row_cap, cudaStream_t st, int n_net
   launch_any(g, row_cap, st, n_nets, true);
 }
 
+// The backward to the input after launch_mlp_fp32's forward (whole: every column of
+// dE/dG, not only the live slices of sparse rows).  delta2 and delta1 go over H2 and H1.
+void launch_mlp_fp32_bwd(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb,
+                         float alpha, cudaStream_t st, StageHook* hook, bool whole) {
+  const int E = md.E, S = md.S, Dp = md.Dp, h1 = md.h1, h2 = md.h2, h3 = md.h3;
+  const int R = ws.row_cap;
+  GemmArgs g{};
+  g.alpha = alpha;
+  g.seg_start = ws.seg_start;
+  g.counts = ws.species_count;
+  g.S = S;
+  // B3: delta2 = (delta3 W3) * D2   (written over H2)
+  g.A = mb.d3; g.lda = E * h3; g.a_net = h3;
+  g.B = mw.W3T; g.b_s = (long long)h2 * h3; g.b_e = (long long)S * h2 * h3; g.ldb = h3;
+  g.N = h2; g.K = h3;
+  g.aux = mb.D2; g.ld_aux = E * h2; g.aux_net = h2;
+  g.out = mb.H2; g.ldo = E * h2; g.out_net = h2;
+  g.epi = kEpiMul;
+  if (hook) hook->begin(6);
+  launch_gemm_fp32(g, R, st, E);
+  if (hook) hook->end();
+  // B2: delta1 = (delta2 W2) * D1   (written over H1)
+  g.A = mb.H2; g.lda = E * h2; g.a_net = h2;
+  g.B = mw.W2T; g.b_s = (long long)h1 * h2; g.b_e = (long long)S * h1 * h2; g.ldb = h2;
+  g.N = h1; g.K = h2;
+  g.aux = mb.D1; g.ld_aux = E * h1; g.aux_net = h1;
+  g.out = mb.H1; g.ldo = E * h1; g.out_net = h1;
+  g.epi = kEpiMul;
+  if (hook) hook->begin(7);
+  launch_gemm_fp32(g, R, st, E);
+  if (hook) hook->end();
+  // B1: dE/dG = [delta1_e]_e [W1_e / E]_e   (K = E*h1)
+  g.A = mb.H1; g.lda = E * h1; g.a_net = 0;
+  g.B = mw.W1Tcat; g.b_s = (long long)Dp * E * h1; g.b_e = 0; g.ldb = E * h1;
+  g.N = Dp; g.K = E * h1;
+  g.out = ws.dEdG; g.ldo = Dp; g.out_net = 0;
+  g.epi = kEpiStore;
+  g.nmask = !whole && ws.row_mask ? ws.tile_mask : nullptr;
+  if (hook) hook->begin(8);
+  launch_gemm_fp32(g, R, st, 1);
+  if (hook) hook->end();
+}
+
 // the six GEMMs of one forward + backward-to-input pass over every species
 // (one fused kernel where the network shape has a compiled variant)
 void launch_mlp_fp32(const Ws& ws, const MlpDims& md, const MlpWeights& mw, const MlpBufs& mb,
@@ -384,36 +427,7 @@ void launch_mlp_fp32(const Ws& ws, const MlpDims& md, const MlpWeights& mw, cons
     if (n_launch) *n_launch += 4;
     return;
   }
-  // B3: delta2 = (delta3 W3) * D2   (written over H2)
-  g.A = mb.d3; g.lda = E * h3; g.a_net = h3;
-  g.B = mw.W3T; g.b_s = (long long)h2 * h3; g.b_e = (long long)S * h2 * h3; g.ldb = h3;
-  g.N = h2; g.K = h3;
-  g.aux = mb.D2; g.ld_aux = E * h2; g.aux_net = h2;
-  g.out = mb.H2; g.ldo = E * h2; g.out_net = h2;
-  g.epi = kEpiMul;
-  if (hook) hook->begin(6);
-  launch_gemm_fp32(g, R, st, E);
-  if (hook) hook->end();
-  // B2: delta1 = (delta2 W2) * D1   (written over H1)
-  g.A = mb.H2; g.lda = E * h2; g.a_net = h2;
-  g.B = mw.W2T; g.b_s = (long long)h1 * h2; g.b_e = (long long)S * h1 * h2; g.ldb = h2;
-  g.N = h1; g.K = h2;
-  g.aux = mb.D1; g.ld_aux = E * h1; g.aux_net = h1;
-  g.out = mb.H1; g.ldo = E * h1; g.out_net = h1;
-  g.epi = kEpiMul;
-  if (hook) hook->begin(7);
-  launch_gemm_fp32(g, R, st, E);
-  if (hook) hook->end();
-  // B1: dE/dG = [delta1_e]_e [W1_e / E]_e   (K = E*h1)
-  g.A = mb.H1; g.lda = E * h1; g.a_net = 0;
-  g.B = mw.W1Tcat; g.b_s = (long long)Dp * E * h1; g.b_e = 0; g.ldb = E * h1;
-  g.N = Dp; g.K = E * h1;
-  g.out = ws.dEdG; g.ldo = Dp; g.out_net = 0;
-  g.epi = kEpiStore;
-  g.nmask = ws.row_mask ? ws.tile_mask : nullptr;
-  if (hook) hook->begin(8);
-  launch_gemm_fp32(g, R, st, 1);
-  if (hook) hook->end();
+  launch_mlp_fp32_bwd(ws, md, mw, mb, alpha, st, hook, false);
   if (n_launch) *n_launch += 7;
 }
 

@@ -80,3 +80,33 @@ def test_gradients_with_a_section_opposite_to_a_collinear_pair(torch_cuda):
         d = got.cpu().numpy().astype(np.float64) - ref
         assert np.linalg.norm(d) <= 1e-3 * np.linalg.norm(ref)
         assert np.abs(d).max() <= 1e-3 * np.abs(ref).max()
+
+
+# the network gradient read back after a call for energies alone, which forms none: the read
+# runs the ensemble's backward (1e-4 of the norm: the parity test's bound of an element)
+@gpu
+@pytest.mark.parametrize("sparse", [True, False])
+def test_gradient_rows_after_an_energy_only_call(torch_cuda, sparse):
+    from paper_2207_14276_gb300 import Potential
+    spec, w = model("ani4", ensemble=3)
+    pot, orc = Potential(spec, w, precision="fp32_simt"), oracle.Model(spec, w)
+    pot.set_sparse_rows(sparse)
+    s = synth.water_box(60, 12.2, 4, seed=61)
+    ref = orc.energy_forces(s.coords, s.species, s.box, want_dEdG=True)["dEdG"]
+    other = to_cuda(synth.water_box(60, 12.2, 4, seed=62))
+    d = to_cuda(s)
+
+    def read():
+        g = pot.debug_rows(1, s.n_atoms).cpu().numpy()
+        assert np.linalg.norm(g - ref) <= 1e-4 * np.linalg.norm(ref)
+
+    for _ in range(3):   # eager, captured, replayed
+        pot.energy_forces_batch([d], forces=False)
+        read()
+        read()
+    pot.energy_forces_batch([other])
+    pot.energy_forces_batch([d])
+    read()
+    pot.energy_forces_batch([other])
+    pot.energy_forces_batch([d], forces=False)
+    read()
