@@ -371,6 +371,9 @@ int nnp_network_path(const nnp_handle* h);
 
 /* Number of kernels the last compute call enqueued (for launch accounting). */
 int nnp_last_launch_count(const nnp_handle* h);
+/* CUDA graphs that the handle's calls have been captured into so far (a shape of
+ * call is captured when it comes repeatedly); -1 for a null handle. */
+int64_t nnp_debug_graph_captures(const nnp_handle* h);
 
 /* Persistent neighbour lists with a Verlet skin (paper Sec. "Neighbour lists":
  * the lists are rebuilt only when atoms have moved far enough, as in the MD

@@ -54,6 +54,7 @@ EXPORTS = (
     "nnp_integrate", "nnp_noalloc_max_atoms", "nnp_debug_cell_grid", "nnp_network_path",
     "nnp_set_fused_chain", "nnp_set_fused_aev_l1", "nnp_set_sparse_rows",
     "nnp_debug_tile_masks", "nnp_build_flags", "nnp_debug_check_index", "nnp_set_deterministic",
+    "nnp_debug_graph_captures",
 )
 
 
@@ -138,6 +139,8 @@ def lib():
     L.nnp_set_deterministic.argtypes = [P, i]
     L.nnp_debug_tile_masks.argtypes = [P, P, P, i, ctypes.POINTER(i)]
     L.nnp_last_launch_count.argtypes = [P]
+    L.nnp_debug_graph_captures.argtypes = [P]
+    L.nnp_debug_graph_captures.restype = i64
     L.nnp_last_error.restype = ctypes.c_char_p
     L.nnp_last_error.argtypes = []
     L.nnp_debug_rows.argtypes = [P, i, P, P]

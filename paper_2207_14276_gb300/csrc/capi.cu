@@ -124,7 +124,11 @@ struct nnp_handle {
   std::vector<cudaGraphNode_t> front_nodes;   // the kernels that take the descriptors
   std::vector<FrontSent> front_sent;          // what those nodes hold now
   std::string gsig;       // shape signature of the captured call
-  std::string last_sig;   // shape signature of the previous eager call
+  std::string last_sig;   // shape signature of the previous call
+  int repeats = 0;        // calls of that shape in a row
+  int capture_after = 2;  // repeats before a capture
+  int graph_calls = 0;    // calls that the present graph served
+  long long captures = 0;
   int last_launches_graph = 0;
   // tensor-core paths: the layers after the first as one fused kernel (off by
   // default: on the 100k-atom ensemble it ties with the four layer GEMMs on the
@@ -826,6 +830,9 @@ int update_front(nnp_handle* h, const std::vector<FrontLaunch>& front) {
   return NNP_OK;
 }
 
+// calls that pay for a graph's capture, and the most repeats that a capture waits for
+constexpr int kPaidCalls = 8, kMaxRepeats = 64;
+
 // enqueue the whole chain for a batch whose descriptors are already validated
 int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st) {
   const Model& m = *h->model;
@@ -931,12 +938,23 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
                           h->fused_chain,           h->fused_aev_l1, h->sparse_rows, h->det};
     put(flags, sizeof(flags));
     for (const FrontLaunch& f : front) put(&f.fn, sizeof(f.fn));   // the nodes, whose grids may change
-    // captured on the shape's second occurrence in a row, replayed afterwards
-    if (!(h->gexec && sig == h->gsig) && sig == h->last_sig) {
+    // Captured on the shape's second occurrence in a row, replayed afterwards.  A capture costs
+    // about 60 us more than the launches it holds and a replay saves 20-40 us, so shapes
+    // that take turns must not throw out each other's graph: one that served few calls
+    // doubles the occurrences that the next capture waits for, one that served many puts
+    // them back to two.  (1,500 water atoms and a molecule in turn, each twice in a row:
+    // 704 us a turn with a capture every second call, 508 so; three molecules, 905 and 673.)
+    h->repeats = sig == h->last_sig ? std::min(h->repeats + 1, kMaxRepeats) : 1;
+    h->last_sig = sig;
+    if (!(h->gexec && sig == h->gsig) && h->repeats >= h->capture_after) {
+      if (h->gexec) h->capture_after = h->graph_calls < kPaidCalls ? std::min(2 * h->capture_after, kMaxRepeats) : 2;
       if ((rc = capture_call(h, front, n_in, front_done, masked, any_virial, energy_only))) return rc;
       h->gsig = sig;
+      h->graph_calls = 0;
+      ++h->captures;
     }
     if (h->gexec && sig == h->gsig) {
+      h->graph_calls = std::min(h->graph_calls + 1, kPaidCalls);
       if ((rc = update_front(h, front))) return rc;
       CU_TRY(cudaGraphLaunch(h->gexec, st));
       h->last_launches = launches + h->last_launches_graph;
@@ -944,7 +962,6 @@ int run_batch(nnp_handle* h, int n_sys, const nnp_system_t* sy, cudaStream_t st)
       h->lists_valid = true;
       return NNP_OK;
     }
-    h->last_sig = sig;
   }
   for (const FrontLaunch& f : front) {
     StageTimer t(h, st, 0);
@@ -1537,6 +1554,7 @@ int nnp_network_path(const nnp_handle* h) {
   return net == kNetBf16 ? NNP_BF16_MLP : net == kNetSplit ? NNP_FP32_SPLIT : NNP_FP32_SIMT;
 }
 int nnp_last_launch_count(const nnp_handle* h) { return h ? h->last_launches : -1; }
+int64_t nnp_debug_graph_captures(const nnp_handle* h) { return h ? h->captures : -1; }
 
 int nnp_set_skin(nnp_handle* h, float skin) {
   g_err.clear();

@@ -110,3 +110,40 @@ def test_gradient_rows_after_an_energy_only_call(torch_cuda, sparse):
     pot.energy_forces_batch([other])
     pot.energy_forces_batch([d], forces=False)
     read()
+
+
+# shapes that take turns on a handle: a graph that another shape's replaces after a call or two
+# costs more than it saves.  Captures end after a few turns, and a shape that stays gets its graph
+@gpu
+@pytest.mark.parametrize("turn", ["AB", "AAB", "AABB", "AAABBB", "AABBCC"])
+def test_shapes_that_take_turns_are_not_captured_each_turn(torch_cuda, turn):
+    from paper_2207_14276_gb300 import Potential, _lib
+    spec, w = model("ani4")
+    pot, orc = Potential(spec, w), oracle.Model(spec, w)
+    systems = dict(zip("ABC", synth.workload("molecules64")[0][:3]))
+    dev = {k: to_cuda(s) for k, s in systems.items()}
+    refs = {k: orc.energy_forces(s.coords, s.species) for k, s in systems.items()}
+
+    def captures():
+        return _lib.lib().nnp_debug_graph_captures(pot._h)
+
+    def call(k):
+        E, F = pot.energy_forces(dev[k]["coords"], dev[k]["species"])
+        return {"energy": E, "forces": F}
+
+    for _ in range(12):
+        for k in turn:
+            call(k)
+    settled = captures()
+    assert settled <= 6   # the wait doubles from 2 to 64
+    for _ in range(12):
+        for k in turn:
+            close(call(k), refs[k], "fp32")
+    assert captures() == settled
+    for k in "CBA":
+        for _ in range(70):
+            call(k)
+        n = captures()
+        close(call(k), refs[k], "fp32")
+        assert captures() == n and n >= settled
+    assert captures() > settled
