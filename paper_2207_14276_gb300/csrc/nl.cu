@@ -780,8 +780,8 @@ __device__ __forceinline__ void centre_lists_staged(const Ws& ws, const AevConst
 // before the scan and listing them per octant of the home cell (what this replaced)
 // shortened the scan but cost 1,450 instructions and four more barriers per cell:
 // solvated100k 219 -> 164 us, 20k atoms 52 -> 34, 72k atoms of water 116 -> 94, 6k
-// solvated atoms 36 -> 17, a 24-atom molecule 9.1 -> 4.8; a 9,000-atom water box, whose
-// 512 cells do not fill the grid, 20 -> 24 us.
+// solvated atoms 36 -> 17, a 24-atom molecule 9.1 -> 4.8; 3,000 and 1,500 atoms of
+// water 20 -> 15 and 14, a 9,000-atom box, whose 512 cells take one and a bit waves, 24 -> 27 us.
 __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac) {
   __shared__ float4 cand[kCandCap];
   __shared__ uint16_t kept[kNbWarps][kStageCap];
@@ -801,7 +801,10 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
   }
   const int n_cells = ws.totals[1];
   // work items: (cell, part) with `parts` CTAs per cell where the cells would not
-  // fill the grid
+  // fill the grid, all cells' first parts before the second ones: a cell's last parts
+  // have no centres, and with its parts side by side the items with centres fell to a
+  // few SMs (3,000 water atoms, 125 cells in 8 parts: 3 SMs of 8 had work; the call
+  // 111.8 us, 104.4 so; 9,000 atoms 155.7 and 153.1)
   const int parts = n_cells > 0 ? min(((int)gridDim.x + n_cells - 1) / n_cells, 8) : 1;
   const int n_items = n_cells * parts;
   int item = blockIdx.x;
@@ -809,7 +812,7 @@ __global__ void __launch_bounds__(kNbThreads, 6) k_neighbors(Ws ws, AevConst ac)
     // the next item is fetched while this one is worked on
     int next = 0;
     if (tid == 0) next = (int)gridDim.x + atomicAdd(ws.totals + 3, 1);
-    const int gc = item / parts, part = item % parts;
+    const int gc = item % n_cells, part = item / n_cells;
     const int cbeg = ws.cell_start[gc], cend = ws.cell_start[gc + 1];
     const int first = cbeg + part * kNbWarps;   // this CTA's first centre
     if (first < cend) {   // uniform across the CTA
