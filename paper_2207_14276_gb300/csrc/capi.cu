@@ -96,7 +96,7 @@ struct nnp_handle {
   // arena
   void* arena = nullptr;
   size_t arena_bytes = 0;
-  int cap_in = 0, cap_sys = 0, cap_r = 128, cap_a = 48;
+  int cap_in = 0, cap_sys = 0, cap_r = nnp::kFirstCapR, cap_a = nnp::kFirstCapA;
   bool dirty = true;  // capacities changed: re-carve before the next call
   Ws ws{};
   MlpBufs mb{};

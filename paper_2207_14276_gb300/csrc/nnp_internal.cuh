@@ -16,6 +16,8 @@ constexpr int kNZ = 8;             // angular sections (Eq. 5)
 constexpr int kRowTile = 128;      // species segments of AEV rows are padded to this
 constexpr int kMaxBatchParam = 64; // systems per kernel-parameter chunk
 constexpr int kStageCap = 512;     // staged radial neighbours per centre (hard cap)
+// Capacities of a handle's neighbour lists (radial, angular) until a call needs longer ones
+constexpr int kFirstCapR = 128, kFirstCapA = 48;
 // A centre with more angular neighbours, or with more species pairs that have triplets,
 // than this is dense: the neighbour search (or, with persistent lists, the refresh)
 // lists it in Ws::heavy, and the AEV kernels give it a CTA instead of a warp.
