@@ -672,11 +672,22 @@ bool sparse_call(const nnp_handle* h) {
   return h->sparse_rows && h->ws.row_mask && !fuses_aev_l1(h) && !(m.net == kNetSimt && mlp_fused_supported(m.md));
 }
 
-// the work space as this call's kernels see it: rows are grouped by their live slices
-// where they are sparse (not in the deterministic mode, whose rows are in packed order)
+// Whether a call's rows are grouped by their live slices.  The counters cost a call of
+// thousands of atoms 2 to 4 us and what they save grows with the slices, networks and rows:
+// one network on 4 species (6 slices), grouped and not, 9,000 water atoms 154.0 and 151.5 us,
+// 20k solvated ones 254.2 and 251.7, 100k 952.8 and 958.6; two networks, 100k, 1,067 and
+// 1,079; 7 species (16 slices), 4.7k solvated atoms 160.5 and 164.2.  Not in the deterministic
+// mode, whose rows are in packed order.
+constexpr int kGroupSlices = 8, kGroupAtoms = 32768;
+bool groups_rows(const nnp_handle* h) {
+  const Model& m = *h->model;
+  return sparse_call(h) && !h->det && (m.md.E * (m.ac.Dp / 64) > kGroupSlices || h->ws.n_in > kGroupAtoms);
+}
+
+// the work space as this call's kernels see it
 Ws call_ws(const nnp_handle* h) {
   Ws ws = h->ws;
-  if (!sparse_call(h) || h->det) {
+  if (!groups_rows(h)) {
     ws.row_key = nullptr;
     ws.row_hist = nullptr;
   }

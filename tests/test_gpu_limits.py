@@ -147,3 +147,28 @@ def test_shapes_that_take_turns_are_not_captured_each_turn(torch_cuda, turn):
         close(call(k), refs[k], "fp32")
         assert captures() == n and n >= settled
     assert captures() > settled
+
+
+# rows are grouped by their live slices past 32,768 atoms, or where slices times networks exceed
+# 8: the same results as whole rows to the last bits of sums of products (1e-5 of the norm), with
+# lists kept between calls too
+@gpu
+@pytest.mark.parametrize("kind,ensemble,n_mol", [("ani4", 1, 10922), ("ani4", 1, 10923), ("ani4", 2, 500)])
+def test_rows_grouped_or_not(torch_cuda, kind, ensemble, n_mol):
+    torch = torch_cuda
+    from paper_2207_14276_gb300 import Potential
+    spec, w = model(kind, ensemble=ensemble)
+    pot = Potential(spec, w)
+    edge = 44.77 * (n_mol / 3000) ** (1 / 3)
+    s = synth.water_box(n_mol, edge, int(np.ceil(n_mol ** (1 / 3))), seed=71)
+    d = to_cuda(s)
+    pot.set_sparse_rows(False)
+    E0, F0 = pot.energy_forces(d["coords"], d["species"], d["box"])
+    pot.set_sparse_rows(True)
+    for skin in (0.0, 0.5):
+        pot.set_skin(skin)
+        for _ in range(3):
+            E, F = pot.energy_forces(d["coords"], d["species"], d["box"])
+            assert float((F - F0).norm()) <= 1e-5 * float(F0.norm())
+            assert abs(float(E[0] - E0[0])) <= 1e-6 * abs(float(E0[0])) + 1e-6 * s.n_atoms ** 0.5
+    pot.set_skin(0.0)
