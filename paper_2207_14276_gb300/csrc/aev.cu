@@ -1152,12 +1152,7 @@ void launch_aev_bwd(const Ws& ws, int n_in, bool masked, const AevConst& ac, int
   // The two kernels add to different accumulators or atomically, so with a side stream
   // they run together: the CTA-per-centre kernel first (higher priority), the other
   // beside it as room allows (6k solvated atoms: 43 us one after the other, 34 together).
-  // A graph with a branch starts later, by 4-6 us where nothing runs ahead of it, so calls
-  // that will hardly have dense centres do without: few species pairs, and lists that never
-  // grew past 48 angular neighbours (1,500, 3,000 and 9,000 water atoms with a cold L2 cache
-  // 112, 118 and 165 us with the branch, 106, 114 and 163 without; 1,200 at three times
-  // the density, all dense, 187 with and 200 without).
-  if (n_in <= small || (ac.n_pairs <= kGallBlocks && ws.cap_a <= kFirstCapA)) side = nullptr;
+  if (n_in <= small) side = nullptr;
   const cudaStream_t main_st = st;
   if (side) {
     cudaEventRecord(side->fork, st);

@@ -19,7 +19,7 @@ __global__ void k_finalize(Ws ws, const float* e_row, int E, int parts, int e_ro
     ws.skin_state[0] = ws.skin_state[1] = 0;   // the next call's check starts from here
   }
   if (p == 0 && ws.status_pub)   // no later kernel of the call sets a flag
-    for (int i = 0; i < 4; ++i) ws.status_pub[i] = ws.status[i];
+    for (int i = 0; i < 4; ++i) ws.status_pub[i] = i < 3 ? ws.status[i] : ws.totals[2];
   const unsigned lane = threadIdx.x & 31;
   const int total = ws.totals[0];
   const bool live = p < total;

@@ -16,8 +16,6 @@ constexpr int kNZ = 8;             // angular sections (Eq. 5)
 constexpr int kRowTile = 128;      // species segments of AEV rows are padded to this
 constexpr int kMaxBatchParam = 64; // systems per kernel-parameter chunk
 constexpr int kStageCap = 512;     // staged radial neighbours per centre (hard cap)
-// Capacities of a handle's neighbour lists (radial, angular) until a call needs longer ones
-constexpr int kFirstCapR = 128, kFirstCapA = 48;
 // A centre with more angular neighbours, or with more species pairs that have triplets,
 // than this is dense: the neighbour search (or, with persistent lists, the refresh)
 // lists it in Ws::heavy, and the AEV kernels give it a CTA instead of a warp.
@@ -148,7 +146,8 @@ using BatchParams = BatchParamsT<kMaxBatchParam>;
 // device work arena (all pointers device)
 struct Ws {
   int* status;       // [4]: flags, max radial count, max angular count, spare
-  int* status_pub;   // host memory: the last kernel of a call copies status here (or null)
+  int* status_pub;   // host memory: the last kernel of a call copies status here (or null), with
+                     // the call's dense centres as the fourth word
   SysDev* sys;       // [max_sys]
   int n_sys;
   int n_in;          // batch input atoms (sum of n_in)
