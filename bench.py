@@ -70,7 +70,7 @@ def parse():
                     choices=["fp32", "fp32_split", "fp32_simt", "bf16"])
     ap.add_argument("--fused-chain", action="store_true",
                     help="tensor-core paths: run L2, L3, B3, B2 as the fused per-network "
-                         "kernel instead of four layer GEMMs")
+                         "kernel instead of layer GEMMs")
     ap.add_argument("--fused-aev-l1", action="store_true",
                     help="BF16 one-network models: AEV computed on chip and fed to the first "
                          "layer in one kernel")

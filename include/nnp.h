@@ -304,8 +304,8 @@ int nnp_aev_dim(const nnp_handle* h);
  * species by packed position (both otherwise follow atomic counters); every
  * force term is written to its own slot (per centre and neighbour-list entry)
  * and a gather sums them in list order, energies and virials are summed over
- * each system's atoms in a fixed order, and the lanes of a warp add into the
- * shared-memory accumulators one after the other.  For catching races: a
+ * each system's atoms in a fixed order (additions into shared-memory accumulators
+ * have a fixed order in either mode).  For catching races: a
  * result that changes between repeated calls in this mode is a bug.  Costs
  * extra memory ((cap_r + cap_a + 1) float4 and 10 doubles per atom) and time.
  * Not covered: the force VJP, and on the FP32 FMA path the ensembles' six-GEMM
@@ -335,10 +335,11 @@ int nnp_debug_check_index(int site, int64_t i, int64_t n, int* status);
  * after the first -- L2, L3 with the output layer, and their backward B3, B2 --
  * as one fused kernel per 128-row tile with the activations in shared memory
  * (widths multiples of 16, at most 256); 0 runs them as four layer GEMMs
- * through HBM.  Both give the same result to rounding order.  Default: off (on
- * the 100k-atom 8-network workload the fused kernel ties with the four GEMMs on
- * the split path and is slower on BF16).  Clones inherit the setting.  No
- * effect on NNP_FP32_SIMT handles. */
+ * through HBM, or L3 and B3 in a kernel of their own where their widths fit it.
+ * All give the same result to rounding order.  Default: off (100k atoms, 8
+ * networks: these layers 1.63 ms against 0.99 without the fused kernel on the split
+ * path, 0.92 against 0.56 on BF16).  Clones inherit the setting.  No effect on
+ * NNP_FP32_SIMT handles. */
 int nnp_set_fused_chain(nnp_handle* h, int enable);
 /* enable != 0 (the default) writes each AEV row only in the
  * 64-column slices that hold a species or species-pair block with any term

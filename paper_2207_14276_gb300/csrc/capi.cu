@@ -131,8 +131,8 @@ struct nnp_handle {
   long long captures = 0;
   int last_launches_graph = 0;
   // tensor-core paths: the layers after the first as one fused kernel (off by
-  // default: on the 100k-atom ensemble it ties with the four layer GEMMs on the
-  // split path and is slower on BF16)
+  // default: on the 100k-atom ensemble 1.63 ms against 0.99 for the kernels it replaces
+  // on the split path, 0.92 against 0.56 on BF16)
   bool fused_chain = false;
   // BF16 one-network models: the AEV computed into shared memory and fed to the
   // first layer in one kernel (off by default)

@@ -27,7 +27,7 @@
 // fewer (split operands at 192 and 160 columns: five slots of 32 KB and five stages of
 // 12 KB) it goes behind, beside B3's epilogue.
 // L3 and B3, two layer GEMMs -> this kernel: 100k solvated atoms, 8 networks, 41 tiles per
-// SM 499 -> 357 us (0.96 GB at least: 140 us); 20k atoms BF16 87 -> 44 us; one tile (24
+// SM 499 -> 357 us (h2 in two parts read and replaced, 1.23 GB: 181 us at least); 20k atoms BF16 87 -> 44 us; one tile (24
 // atoms) 13 -> 10.7 us.  Bound by the chain of a tile: B3 4.3 k cycles, the last block's
 // store, load and share of L3 7.1 k (beside B3's epilogue, 4.8 k), L3's epilogue 3.1 k.
 // Every wait is bounded; a CTA that gives up records a timeout in the status word,

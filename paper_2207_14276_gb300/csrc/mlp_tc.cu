@@ -562,7 +562,7 @@ struct TcState {
   float* e_row = nullptr;
   int row_cap = 0, Dp = 0, E = 1;
   bool split = false;
-  void* chain = nullptr;     // fused L2 -> L3 -> B3 -> B2 (null: the four layer GEMMs)
+  void* chain = nullptr;     // fused L2 -> L3 -> B3 -> B2 (null: the layer GEMMs)
   bool use_chain = true;
   void* head = nullptr;      // fused L3 -> B3 (null: two layer GEMMs)
   ~TcState() {

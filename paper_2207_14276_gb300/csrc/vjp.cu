@@ -87,8 +87,12 @@ __global__ void __launch_bounds__(kWarps * 32) k_aev_fwd_vjp(Ws ws, AevConst ac,
   float* U = vb.U + (size_t)slot * ac.Dp;
   load_hdr(ws.nb_cnt + (size_t)p * 16, ac.S, lane, &H);
   const uint32_t msk = ws.row_mask ? row_slices(H, ac, lane, pair_su) : ~0u;
-  // (the values are formed exactly as in k_aev_fwd: CELU'' jumps at z = 0, so a
-  // gradient depends on the last bits of G where a pre-activation is next to zero)
+  // (G to rounding, not bit by bit the rows of k_aev_fwd, which takes pairs and radial terms
+  // in another order.  CELU'' jumps at z = 0, so where a pre-activation is next to zero a
+  // gradient depends on the last bits of G, in any order: 40 boxes of 1,500 water atoms,
+  // dL/dcoords from 64 bits 1.8e-6 of its norm in the median and 1.0e-4 on average, both with
+  // this order and with the forward's own rows, and two runs, whose cells list their atoms
+  // in different orders, up to 1.8e-4 from each other)
   const float inv_rc_r = 1.f / ac.rc_r, inv_rc_a = 1.f / ac.rc_a;
   stage_list(H.off_r[ac.S], ws.nb_r + (size_t)p * ws.cap_r, xi, d, ws, lane,
              [&](int t, int j, const Geo& g) {

@@ -136,8 +136,8 @@ class Potential:
         return lib().nnp_sync_status(self._h, _stream_ptr(stream))
 
     def set_fused_chain(self, enable):
-        """Tensor-core paths: run L2, L3, B3 and B2 as one fused kernel (default)
-        or as four layer GEMMs."""
+        """Tensor-core paths: run L2, L3, B3 and B2 as one fused kernel, or (default) as
+        layer GEMMs with L3 and B3 in one kernel."""
         check(lib().nnp_set_fused_chain(self._h, 1 if enable else 0))
 
     def set_deterministic(self, enable):
@@ -146,8 +146,8 @@ class Potential:
         check(lib().nnp_set_deterministic(self._h, 1 if enable else 0))
 
     def set_sparse_rows(self, enable):
-        """Tensor-core paths: write and multiply only the live 64-column slices of
-        the AEV rows (default on; the result is the same)."""
+        """Write and multiply only the live 64-column slices of the AEV rows (default on;
+        the result is the same; no effect on the fused kernel of one FP32 FMA network)."""
         check(lib().nnp_set_sparse_rows(self._h, 1 if enable else 0))
 
     def tile_masks(self, max_tiles=1 << 20, stream=None):
